@@ -146,10 +146,10 @@ def _profile_traffic(name, files, function=None):
     return float(fields["traffic_bytes_per_launch"])
 
 
-# the plane pass: its own function text in hpsi_ct.cuh plus the staged-transform core
-PLANE_SOURCES = ["paper_1406_7803_gb300/csrc/fftct.cuh", "paper_1406_7803_gb300/csrc/fft.cuh",
+# the plane pass: its own function text and steps in hpsi2.cuh plus the two-step transform core
+PLANE_SOURCES = ["paper_1406_7803_gb300/csrc/fft2.cuh", "paper_1406_7803_gb300/csrc/fft.cuh",
                  "paper_1406_7803_gb300/csrc/common.cuh"]
-PLANE_FUNCTION = ("paper_1406_7803_gb300/csrc/hpsi_ct.cuh", "k_plane_ct")
+PLANE_FUNCTION = ("paper_1406_7803_gb300/csrc/hpsi2.cuh", "k_plane_pass")
 
 
 def max_over_ranks(x, ws, device):

@@ -18,8 +18,10 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libfde.so")
 BUILD = os.path.join(HERE, "_build")
-SOURCES = ["hpsi.cu", "hpsi_ct32.cu", "hpsi_ct64.cu", "grid.cu", "linalg.cu", "small.cu", "fde_host.cu",
-           "hpsi_static.cu", "precond.cu", "heev.cu", "dense.cu", "gemm_tc.cu", "hostmath.cu", "fft_dd.cu"]
+SOURCES = ["hpsi.cu", "hpsi2.cu", "hpsi2_p32.cu", "hpsi2_p64.cu", "hpsi2_z32.cu", "hpsi2_z64.cu", "fft3_32.cu",
+           "fft3_64.cu", "grid.cu", "linalg.cu", "small.cu", "fde_host.cu",
+           "hpsi_static.cu", "precond.cu", "heev.cu", "dense.cu", "gemm_tc.cu", "hostmath.cu", "fft_dd.cu", "fft_dd_0.cu",
+           "fft_dd_1.cu", "fft_dd_2.cu", "fft_dd_3.cu", "fft_dd_4.cu", "fft_dd_5.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off",
          "-I", os.path.join(ROOT, "include"), "-I", CSRC]

@@ -249,7 +249,7 @@ template <typename T> struct EngineT : Engine {
   DBuf<double2> S, Hs, L, Li, Ht, Y, Cc, tmp, jwork;
   DBuf<double> wv, dnorm, deps, dtb, hwork;
   DBuf<int> didx;
-  DBuf<double> rho_plane, occw;
+  DBuf<double> rho_plane, rho_part, occw;
   // Pulay histories (one for the subsystem SCF, one per subsystem for the refreshed SCF)
   // and freeze-and-thaw copies
   struct PulayHist {
@@ -410,7 +410,18 @@ template <typename T> struct EngineT : Engine {
     CK(cudaMemcpy(q.cols.p, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice));
     q.sp.npw = q.npw;
     q.sp.ncol = ncol;
+    q.sp.ldc = (ncol + 15) / 16 * 16;  // 128-byte scratch rows
     q.sp.nrow = (int)rows.size();
+    int m2lo = q.miller[1], m2hi = q.miller[1];
+    for (int p = 0; p < q.npw; ++p) {
+      m2lo = std::min(m2lo, q.miller[3 * p + 1]);
+      m2hi = std::max(m2hi, q.miller[3 * p + 1]);
+    }
+    const int m1lo = q.miller[0], m1hi = q.miller[3 * (q.npw - 1)];
+    q.sp.lo1 = ((m1lo % grid[0]) + grid[0]) % grid[0];
+    q.sp.span1 = m1hi - m1lo + 1;
+    q.sp.lo2 = ((m2lo % grid[1]) + grid[1]) % grid[1];
+    q.sp.span2 = m2hi - m2lo + 1;
     q.sp.col_start = q.cols.p;
     q.sp.col_m3lo = q.cols.p + (ncol + 1);
     q.sp.col_i1 = q.cols.p + (2 * ncol + 1);
@@ -817,7 +828,7 @@ template <typename T> struct EngineT : Engine {
   long long davidson_iters = 0, hpsi_bands = 0;
   void apply_h_dev(Sub<T>& s, KP<T>& q, const C* psi, C* hpsi, int nb) {
     hpsi_bands += nb;
-    scratch.ensure((size_t)nb * g.n3 * q.sp.ncol);
+    scratch.ensure((size_t)nb * g.n3 * q.sp.ldc);
     launch_hpsi_local<T>(psi, q.npw, hpsi, q.npw, nb, q.kin_d.p, s.vplane.p, scratch.p, q.sp, g, plans.fp, st);
     apply_nl(s, q, psi, hpsi, nb);
   }
@@ -900,16 +911,16 @@ template <typename T> struct EngineT : Engine {
   void apply_h_all() override {
     size_t total = 0;
     for (auto& sp : subs)
-      for (auto& q : sp->kp) total += (size_t)sp->nb * g.n3 * q.sp.ncol;
+      for (auto& q : sp->kp) total += (size_t)sp->nb * g.n3 * q.sp.ldc;
     scratch.ensure(total);
     std::vector<HpsiItemDesc<T>> items;
     size_t off = 0;
     for (auto& sp : subs)
       for (auto& q : sp->kp) {
         items.push_back(HpsiItemDesc<T>{q.sp, q.X.p, q.HX.p, q.kin_d.p, sp->vplane.p, scratch.p + off, q.npw, sp->nb});
-        off += (size_t)sp->nb * g.n3 * q.sp.ncol;
+        off += (size_t)sp->nb * g.n3 * q.sp.ldc;
       }
-    if (!launch_hpsi_batch_ct<T>(items.data(), (int)items.size(), g, plans.fp, st)) {
+    if (!launch_hpsi_batch<T>(items.data(), (int)items.size(), g, plans.fp, st)) {
       for (auto& sp : subs)
         for (auto& q : sp->kp) apply_h_dev(*sp, q, q.X.p, q.HX.p, sp->nb);
       return;
@@ -1381,8 +1392,9 @@ template <typename T> struct EngineT : Engine {
       std::vector<double> w(s.nb);
       for (int j = 0; j < s.nb; ++j) w[j] = 2.0 * s.wk[k] * q.occ[j] / omega;
       CK(cudaMemcpyAsync(occw.p, w.data(), s.nb * sizeof(double), cudaMemcpyHostToDevice, st));
-      scratch.ensure((size_t)s.nb * g.n3 * q.sp.ncol);
-      launch_density<T>(q.X.p, q.npw, s.nb, occw.p, scratch.p, rho_plane.p, k > 0, q.sp, g, plans.fp, st);
+      scratch.ensure((size_t)s.nb * g.n3 * q.sp.ldc);
+      rho_part.ensure((size_t)plane_density_groups(s.nb, g.n3) * nr);
+      launch_density<T>(q.X.p, q.npw, s.nb, occw.p, scratch.p, rho_part.p, rho_plane.p, k > 0, q.sp, g, plans.fp, st);
       CK(cudaStreamSynchronize(st));  // occw is reused by the next k
     }
     launch_transpose<double, double>(rho_plane.p, out, g.n3, (int)((long long)g.n1 * g.n2), 0, st);

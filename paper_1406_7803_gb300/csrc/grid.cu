@@ -49,7 +49,7 @@ k_fft_axis(cplx<T>* __restrict__ data, long long nlines, int N, long long I, Lin
 
 template <typename T>
 void launch_fft3d(cplx<T>* data, const GridDims& g, const FftPlans<T>& fp, int sign, cudaStream_t st) {
-  if (launch_fft3d_ct<T>(data, g, fp, sign, st)) return;
+  if (launch_fft3d_two_step<T>(data, g, fp, sign, st)) return;
   const long long nr = (long long)g.n1 * g.n2 * g.n3;
   struct Ax { int N; long long I; const LinePlan<T>* p; } ax[3] = {
       {g.n3, 1, &fp.p3}, {g.n2, g.n3, &fp.p2}, {g.n1, (long long)g.n2 * g.n3, &fp.p1}};

@@ -17,7 +17,7 @@
 // Only the sphere columns (a disk of the (x, y) plane) travel through global memory, so
 // a band-apply moves about 4 x n3 x ncol complex values plus the potential plane instead
 // of the 4 x N_r of a plain 3D transform pair.
-#include "fft.cuh"
+#include "hpsi2.cuh"
 #include "kernels.h"
 #include "prof.h"
 
@@ -149,7 +149,10 @@ void launch_hpsi_local(const cplx<T>* psi, int ldpsi, cplx<T>* hpsi, int ldh, in
                        const T* kin, const T* vplane, cplx<T>* scratch, const SphereDev& sp,
                        const GridDims& g, const FftPlans<T>& fp, cudaStream_t st) {
   if (nb <= 0) return;
-  if (launch_hpsi_local_ct<T>(psi, ldpsi, hpsi, ldh, nb, kin, vplane, scratch, sp, g, fp, st)) return;
+  if (ldpsi == ldh) {
+    const HpsiItemDesc<T> d{sp, psi, hpsi, kin, vplane, scratch, ldpsi, nb};
+    if (launch_hpsi_batch<T>(&d, 1, g, fp, st)) return;
+  }
   const dim3 gz(ceil_div(sp.ncol, kColsPerCta), nb);
   const size_t zs = zpass_smem<T>(g.n3), ps = plane_smem<T>(g);
   allow_smem(k_zinv<T>, zs);
@@ -210,11 +213,22 @@ k_plane_density(const cplx<T>* __restrict__ scratch, SphereDev sp, int nb, const
 }
 
 template <typename T>
-void launch_density(const cplx<T>* psi, int ldpsi, int nb, const double* weight, cplx<T>* scratch,
-                    double* rho_plane, int accumulate, const SphereDev& sp, const GridDims& g,
-                    const FftPlans<T>& fp, cudaStream_t st) {
+void launch_density(const cplx<T>* psi, int ldpsi, int nb, const double* weight, cplx<T>* scratch, double* part,
+                    double* rho_plane, int accumulate, const SphereDev& sp, const GridDims& g, const FftPlans<T>& fp,
+                    cudaStream_t st) {
   if (nb <= 0) return;
-  if (launch_density_ct<T>(psi, ldpsi, nb, weight, scratch, rho_plane, accumulate, sp, g, fp, st)) return;
+  if (two_step_grid<T>(g, sp)) {
+    HpsiBatch<T> B;
+    B.n = 1;
+    B.it[0] = HpsiItem<T>{sp, psi, nullptr, nullptr, nullptr, scratch, ldpsi, nb, 0, 0};
+    {
+      ProfScope prof_("k_zinv_density", st);
+      launch_zinv_cols<T>(g.n3, (unsigned)(ceil_div(sp.ncol, z_cols<T>()) * nb), B, fp.p3.tw, st);
+    }
+    ProfScope prof_("k_plane_density", st);
+    launch_plane_density<T>(g, scratch, sp, nb, weight, part, rho_plane, accumulate, fp, st);
+    return;
+  }
   const dim3 gz(ceil_div(sp.ncol, kColsPerCta), nb);
   const size_t zs = zpass_smem<T>(g.n3), ps = plane_smem<T>(g);
   allow_smem(k_zinv<T>, zs);
@@ -257,9 +271,9 @@ template void launch_hpsi_local<float>(const float2*, int, float2*, int, int, co
 template void launch_hpsi_local<double>(const double2*, int, double2*, int, int, const double*, const double*,
                                         double2*, const SphereDev&, const GridDims&, const FftPlans<double>&,
                                         cudaStream_t);
-template void launch_density<float>(const float2*, int, int, const double*, float2*, double*, int, const SphereDev&,
-                                    const GridDims&, const FftPlans<float>&, cudaStream_t);
-template void launch_density<double>(const double2*, int, int, const double*, double2*, double*, int,
+template void launch_density<float>(const float2*, int, int, const double*, float2*, double*, double*, int,
+                                    const SphereDev&, const GridDims&, const FftPlans<float>&, cudaStream_t);
+template void launch_density<double>(const double2*, int, int, const double*, double2*, double*, double*, int,
                                      const SphereDev&, const GridDims&, const FftPlans<double>&, cudaStream_t);
 template void launch_transpose<double, double>(const double*, double*, int, int, int, cudaStream_t);
 template void launch_transpose<double, float>(const double*, float*, int, int, int, cudaStream_t);

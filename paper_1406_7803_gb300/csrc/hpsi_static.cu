@@ -33,7 +33,7 @@ static __device__ __align__(256) double2 st_scratch[kStScratch];
 static __device__ __align__(256) double st_vplane[kStMaxGrid];
 static __device__ __align__(256) double st_kin[kStMaxNpw];
 static __device__ __align__(256) int st_cols[4 * kStMaxCols + 1 + kMaxPlane];
-static __device__ __align__(256) int st_ncols[2];
+static __device__ __align__(256) int st_ncols[6];
 static __device__ __align__(256) double2 st_tw[3][kMaxLine];
 
 struct StaticPtrs {
@@ -68,7 +68,7 @@ static fde_status static_setup(int dev, StaticPtrs* out) {
 }
 
 // Column map of a sphere (one CTA): cols = [start(ncol+1) | m3lo | i1 | i2 | rows];
-// ncols = {ncol, nrow}.  A column starts where (m1, m2) changes; rows are the distinct i1.
+// ncols = {ncol, nrow, lowest m1 mod n1, m1 span, lowest m2 mod n2, m2 span}.  A column starts where (m1, m2) changes; rows are the distinct i1.
 // The caller's list is checked on the way, because the transforms index shared-memory lines
 // by it: (m1, m2) keys strictly increasing from column to column (sorted, no repeats), m3
 // contiguous inside a column, every m3 in [-n3, n3), every column at most n3 long, and the
@@ -177,6 +177,10 @@ k_static_columns(const int* __restrict__ mil, int npw, int n1, int n2, int n3, i
       if (rowflag[i]) rows[r++] = i;
     ncols[0] = ncol;
     ncols[1] = r;
+    ncols[2] = ((lo1 % n1) + n1) % n1;
+    ncols[3] = hi1 - lo1 + 1;
+    ncols[4] = ((lo2 % n2) + n2) % n2;
+    ncols[5] = hi2 - lo2 + 1;
   }
 }
 
@@ -245,7 +249,7 @@ extern "C" fde_status fde_apply_h_local_static(const fde_cell_desc* cell, const 
   k_static_kin<<<ceil_div(npw, 256), 256, 0, st>>>(d_miller, npw, b[0], b[1], b[2], kfrac[0] * b[0],
                                                    kfrac[1] * b[1], kfrac[2] * b[2], P.kin);
   launch_transpose<double, double>(d_veff, P.vplane, n1 * n2, n3, 0, st);
-  int hc[2] = {0, 0};
+  int hc[6] = {0, 0, 0, 0, 0, 0};
   if (cudaMemcpyAsync(hc, P.ncols, sizeof(hc), cudaMemcpyDeviceToHost, st) != cudaSuccess) return FDE_ECUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return FDE_ECUDA;
   const int ncol = hc[0], nrow = hc[1];
@@ -256,7 +260,12 @@ extern "C" fde_status fde_apply_h_local_static(const fde_cell_desc* cell, const 
   SphereDev sp;
   sp.npw = npw;
   sp.ncol = ncol;
+  sp.ldc = ncol;  // the scratch array's limit counts n3 x ncol values
   sp.nrow = nrow;
+  sp.lo1 = hc[2];
+  sp.span1 = hc[3];
+  sp.lo2 = hc[4];
+  sp.span2 = hc[5];
   sp.col_start = P.cols;
   sp.col_m3lo = P.cols + ncol + 1;
   sp.col_i1 = sp.col_m3lo + ncol;

@@ -13,6 +13,9 @@ namespace fde {
 // contiguous run of m3 values; sphere order puts each column's run contiguously.
 struct SphereDev {
   int npw, ncol, nrow;
+  int ldc;           // columns a scratch row [i3][ldc] holds: ncol, or more so that rows are aligned
+  int lo1, span1;    // grid index of the lowest m1 and the span of m1 (rows without a column included)
+  int lo2, span2;    // the same for m2
   const int* col_start;  // [ncol + 1] offsets into the sphere
   const int* col_m3lo;   // [ncol] signed m3 of the first point
   const int* col_i1;     // [ncol] grid index i1 = m1 mod n1
@@ -29,16 +32,17 @@ template <typename T> struct FftPlans {
 };
 
 // ---- H psi local part and densities (hpsi.cu) -----------------------------------------
-// scratch: [nb][n3][ncol] complex T.  vplane: [n3][n1][n2] real T.
+// scratch: [nb][n3][ldc] complex T.  vplane: [n3][n1][n2] real T.
 template <typename T>
 void launch_hpsi_local(const cplx<T>* psi, int ldpsi, cplx<T>* hpsi, int ldh, int nb,
                        const T* kin, const T* vplane, cplx<T>* scratch, const SphereDev& sp,
                        const GridDims& g, const FftPlans<T>& fp, cudaStream_t st);
 
-// rho_plane[n3][n1][n2] (+)= sum_b weight[b] |u_b(r)|^2 for the block of nb orbitals.
+// rho_plane[n3][n1][n2] (+)= sum_b weight[b] |u_b(r)|^2 for the block of nb orbitals; part: work of
+// plane_density_groups(nb, n3) N_r doubles.
 template <typename T>
 void launch_density(const cplx<T>* psi, int ldpsi, int nb, const double* weight,
-                    cplx<T>* scratch, double* rho_plane, int accumulate, const SphereDev& sp,
+                    cplx<T>* scratch, double* part, double* rho_plane, int accumulate, const SphereDev& sp,
                     const GridDims& g, const FftPlans<T>& fp, cudaStream_t st);
 
 // One (subsystem, k) block of bands of a batched H psi launch.
@@ -48,32 +52,45 @@ template <typename T> struct HpsiItemDesc {
   cplx<T>* hpsi;
   const T* kin;
   const T* vplane;
-  cplx<T>* scratch;  // [nb][n3][ncol] of this item
+  cplx<T>* scratch;  // [nb][n3][ldc] of this item
   int ld, nb;
 };
-// Local H psi of many items in three launches (batches of up to 24 items each).
+// Local H psi of many items in three launches (batches of up to 24 items each); false (nothing
+// launched) when a length of the grid has no two-step plan (fft2.cuh): the runtime-length kernels
+// of hpsi.cu serve those grids.
 template <typename T>
-bool launch_hpsi_batch_ct(const HpsiItemDesc<T>* items, int nitems, const GridDims& g, const FftPlans<T>& fp,
-                          cudaStream_t st);
-
-// Variant of the FP32 plane pass the tuner chose for plane side n1 and z length n3 (-1: none
-// tuned yet).
+bool launch_hpsi_batch(const HpsiItemDesc<T>* items, int nitems, const GridDims& g, const FftPlans<T>& fp,
+                       cudaStream_t st);
+// The same three phases' launches on a prepared batch (hpsi2_z32.cu, hpsi2_z64.cu, hpsi2_p32.cu,
+// hpsi2_p64.cu).
+template <typename T> struct HpsiBatch;
+template <typename T>
+void launch_zinv_cols(int n3, unsigned blocks, const HpsiBatch<T>& B, const cplx<T>* tw, cudaStream_t st);
+template <typename T>
+void launch_zfwd_cols(int n3, unsigned blocks, const HpsiBatch<T>& B, T inv_nr, const cplx<T>* tw, cudaStream_t st);
+template <typename T>
+void launch_plane_pass(const GridDims& g, unsigned blocks, const HpsiBatch<T>& B, const FftPlans<T>& fp, cudaStream_t st);
+// rho_plane (+)= sum_b weight[b] |u_b|^2 from the z pass's scratch; part: plane_density_groups
+// partial densities (N_r doubles each).
+int plane_density_groups(int nb, int n3);
+template <typename T>
+void launch_plane_density(const GridDims& g, const cplx<T>* scratch, const SphereDev& sp, int nb, const double* weight,
+                          double* part, double* rho_plane, int accumulate, const FftPlans<T>& fp, cudaStream_t st);
+// Whether a grid has two-step plans and its plane kernel fits shared memory for a sphere.
+template <typename T> bool two_step_grid(const GridDims& g, const SphereDev& sp);
+// Variant of the plane pass in use for a grid shape (-1: none was tuned), and the pinned one
+// (false for values outside -1 .. 7).
 int query_plane_variant(int n1, int n3);
-// Pin the variant (0 .. count - 1) or return to tuning (-1); false for other values.
 bool pin_plane_variant(int v);
 
-// Compile-time-length variants (hpsi_ct.cuh); return false when the grid sizes are not
-// among the instantiated ones, and the runtime-length kernels run instead.
+// Full 3D transforms on two-step plans (fft3.cu); false when a length has none.
 template <typename T>
-bool launch_hpsi_local_ct(const cplx<T>* psi, int ldpsi, cplx<T>* hpsi, int ldh, int nb, const T* kin,
-                          const T* vplane, cplx<T>* scratch, const SphereDev& sp, const GridDims& g,
-                          const FftPlans<T>& fp, cudaStream_t st);
-template <typename T>
-bool launch_density_ct(const cplx<T>* psi, int ldpsi, int nb, const double* weight, cplx<T>* scratch,
-                       double* rho_plane, int accumulate, const SphereDev& sp, const GridDims& g,
-                       const FftPlans<T>& fp, cudaStream_t st);
-template <typename T>
-bool launch_fft3d_ct(cplx<T>* data, const GridDims& g, const FftPlans<T>& fp, int sign, cudaStream_t st);
+bool launch_fft3d_two_step(cplx<T>* data, const GridDims& g, const FftPlans<T>& fp, int sign, cudaStream_t st);
+template <>
+bool launch_fft3d_two_step<float>(float2* data, const GridDims& g, const FftPlans<float>& fp, int sign, cudaStream_t st);
+template <>
+bool launch_fft3d_two_step<double>(double2* data, const GridDims& g, const FftPlans<double>& fp, int sign,
+                                   cudaStream_t st);
 
 // out[j][i] = (Tout) in[i][j], in is [rows][cols]; with optional accumulate.
 template <typename Tin, typename Tout>
