@@ -4,13 +4,18 @@
 // the matrix rows cyclically in shared memory (row i in CTA i % P) and synchronise with the
 // hardware cluster barrier; the embarrassingly parallel phases run as ordinary launches.
 //
-//   k_cl_cholesky   S = L L^H (right-looking, 2 cluster barriers per column)
-//   k_tri_inverse   L^{-1}, one warp per column
-//   k_cl_tridiag    Householder reduction A = Q T Q^H (3 cluster barriers per column)
-//   k_tri_eigvals   eigenvalues of T by 32-point multisection on Sturm counts (warp each)
+//   k_cl_cholesky   S = L L^H (right-looking, one cluster barrier per column)
+//   k_tri_inverse   L^{-1}, one CTA per column
+//   k_cl_tridiag    Householder reduction A = Q T Q^H (2 cluster barriers per column)
+//   k_tri_eigvals   eigenvalues of T by 128-point multisection on Sturm counts (CTA each)
 //   k_tri_solve     inverse iteration, one thread per eigenvector
 //   k_tri_orth      modified Gram-Schmidt inside clusters of close eigenvalues
-//   k_backtransform v = H_0 ... H_{n-2} z, one warp per eigenvector
+//   k_wy_gram       inner products of the reflectors, block by block
+//   k_backtransform v = H_0 ... H_{n-2} z, one CTA per eigenvector, 16 reflectors at a time
+// At these sizes (n up to a few hundred) every kernel is bound by latency: a dependent FP64
+// operation takes some 70 cycles and a division or square root ten of them, so each step keeps its
+// chain of dependent operations short (sums as trees, reciprocals formed once and by one warp,
+// no division inside a recurrence) and its barriers few.
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -43,7 +48,9 @@ __device__ __forceinline__ double block_sum_cl(double v, double* red) {
 }
 
 struct ClusterLayout {
-  int P, rank, nloc, ld;
+  int P, rank, nloc, sh;  // CTAs (a power of two, 2^sh), own rank, rows held
+  __device__ __forceinline__ int owner(int i) const { return i & (P - 1); }
+  __device__ __forceinline__ int local(int i) const { return i >> sh; }
 };
 
 __device__ __forceinline__ ClusterLayout cluster_layout(int n) {
@@ -51,249 +58,288 @@ __device__ __forceinline__ ClusterLayout cluster_layout(int n) {
   c.P = (int)cg::this_cluster().num_blocks();
   c.rank = (int)cg::this_cluster().block_rank();
   c.nloc = (n + c.P - 1) / c.P;
-  c.ld = n;
+  c.sh = 31 - __clz(c.P);
   return c;
 }
 
 // ---- Cholesky --------------------------------------------------------------------------------
-// Shared memory: rows [nloc][n] double2, col [n] double2, red.
+// Every CTA gathers the raw column j of the trailing matrix (its owners' rows, through the cluster's
+// shared memory) with the reciprocal of its pivot, and updates its own rows
+//   A[i][k] -= (A[i][j] / d_j) conj(A[k][j]),
+// one cluster barrier a column; the columns are scaled by 1 / sqrt(d_j) at the end, all at once, so no
+// square root and one reciprocal sit in the chain of a column.  Shared memory: rows [nloc][n],
+// col [n], piv [n] (the least accepted pivots, then 1 / sqrt(d_j)).  Writes the transpose of L,
+// which k_tri_inverse reads by columns.
 __global__ void __launch_bounds__(kClThreads)
-k_cl_cholesky(const double2* __restrict__ S, int n, double2* __restrict__ L, unsigned* status, double rel_pivot) {
+k_cl_cholesky(const double2* __restrict__ S, int n, double2* __restrict__ LT, unsigned* status, double rel_pivot) {
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ __align__(16) unsigned char smem[];
   const ClusterLayout c = cluster_layout(n);
   double2* rows = reinterpret_cast<double2*>(smem);
   double2* col = rows + (size_t)c.nloc * n;
-  __shared__ double s_diag;
+  double* piv = reinterpret_cast<double*>(col + n);
+  __shared__ double s_inv;
+  __shared__ int s_bad;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int idx = tid; idx < c.nloc * n; idx += kClThreads) {
     const int li = idx / n, j = idx - li * n, i = li * c.P + c.rank;
     rows[idx] = (i < n && j <= i) ? S[(size_t)i * n + j] : make_double2(0, 0);
   }
+  for (int j = tid; j < n; j += kClThreads) piv[j] = rel_pivot * S[(size_t)j * n + j].x;
+  if (tid == 0) s_bad = 0;
   cl.sync();
   bool failed = false;
+  int bad = 0;
   for (int j = 0; j < n; ++j) {
-    const int oj = j % c.P, lj = j / c.P;
-    if (tid == 0) {
-      const double2* rj = cl.map_shared_rank(rows, oj);
-      s_diag = rj[(size_t)lj * n + j].x;
-    }
-    __syncthreads();
-    const double d = s_diag;
-    if (!(d > rel_pivot * S[(size_t)j * n + j].x)) {  // identical values in every CTA: a uniform exit
-      failed = true;
-      break;
-    }
-    const double sd = sqrt(d), inv = 1.0 / sd;
-    // scale column j of the own rows below the diagonal
-    for (int li = tid; li < c.nloc; li += kClThreads) {
-      const int i = li * c.P + c.rank;
-      if (i > j && i < n) {
-        double2& v = rows[(size_t)li * n + j];
-        v.x *= inv;
-        v.y *= inv;
+    for (int k = j + tid; k < n; k += kClThreads) {
+      const double2* rk = cl.map_shared_rank(rows, c.owner(k));
+      const double2 x = rk[(size_t)c.local(k) * n + j];
+      col[k] = x;
+      if (k == j) {  // thread 0
+        if (!(x.x > piv[j])) s_bad = 1;
+        s_inv = 1.0 / x.x;
+        piv[j] = x.x;
       }
     }
-    cl.sync();
-    if (c.rank == oj && tid == 0) rows[(size_t)lj * n + j] = make_double2(sd, 0.0);
-    // gather column j (rows > j) and update the own rows: A[i][k] -= L[i][j] conj(L[k][j])
-    for (int k = j + 1 + tid; k < n; k += kClThreads) {
-      const double2* rk = cl.map_shared_rank(rows, k % c.P);
-      col[k] = rk[(size_t)(k / c.P) * n + j];
-    }
     __syncthreads();
+    if (s_bad) {  // the same values in every CTA: a uniform exit
+      failed = true;
+      bad = j;
+      break;
+    }
+    const double inv = s_inv;
     for (int li = warp; li < c.nloc; li += kClWarps) {
       const int i = li * c.P + c.rank;
       if (i <= j || i >= n) continue;
-      const double2 a = rows[(size_t)li * n + j];
+      const double2 a = col[i];
+      const double ax = a.x * inv, ay = a.y * inv;
       double2* ri = rows + (size_t)li * n;
       for (int k = j + 1 + lane; k <= i; k += 32) {
         const double2 b = col[k];
         double2 v = ri[k];
-        v.x -= a.x * b.x + a.y * b.y;
-        v.y -= a.y * b.x - a.x * b.y;
+        v.x = fma(-ax, b.x, v.x);
+        v.y = fma(-ay, b.x, v.y);
+        v.x = fma(-ay, b.y, v.x);
+        v.y = fma(ax, b.y, v.y);
         ri[k] = v;
       }
     }
     cl.sync();
   }
   if (failed) {
-    if (c.rank == 0 && tid == 0) atomicOr(status, ST_CHOLESKY);
+    if (c.rank == 0 && tid == 0) {
+      atomicOr(status, ST_CHOLESKY);
+      status[1] = (unsigned)bad;
+    }
   } else {
+    for (int j = tid; j < n; j += kClThreads) piv[j] = 1.0 / sqrt(piv[j]);
+    __syncthreads();
     for (int idx = tid; idx < c.nloc * n; idx += kClThreads) {
       const int li = idx / n, j = idx - li * n, i = li * c.P + c.rank;
-      if (i < n) L[(size_t)i * n + j] = (j <= i) ? rows[idx] : make_double2(0, 0);
+      if (i >= n) continue;
+      double2 v = make_double2(0, 0);
+      if (j <= i) {
+        const double p = piv[j];
+        v = rows[idx];
+        v = (j == i) ? make_double2(v.x * p, 0.0) : make_double2(v.x * p, v.y * p);
+      }
+      LT[(size_t)j * n + i] = v;
     }
   }
   cl.sync();  // no CTA leaves while others may still read its shared memory
 }
 
 // ---- triangular inverse ------------------------------------------------------------------------
-// Li = L^{-1} (lower); column c by forward substitution, one warp per column.
-__global__ void k_tri_inverse(const double2* __restrict__ L, int n, double2* __restrict__ Li, const unsigned* status) {
+// Li = L^{-1} (lower); column c of the inverse by forward substitution, right-looking: one CTA per
+// column, a thread per row, the residual in registers.  Row i's value is final once columns c .. i - 1
+// have been taken off it; its thread publishes x_i = r_i / L_ii (a stored reciprocal) and every later
+// row takes L[k][i] x_i off its own.  Reads L by columns (LT, coalesced).
+constexpr int kTiThreads = 128;
+constexpr int kTiRows = 4;  // rows a thread: n up to 512
+__global__ void __launch_bounds__(kTiThreads)
+k_tri_inverse(const double2* __restrict__ LT, int n, double2* __restrict__ Li, const unsigned* status) {
   if (*status & ST_CHOLESKY) return;
-  const int lane = threadIdx.x & 31;
-  const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (c >= n) return;
-  for (int i = lane; i < c; i += 32) Li[(size_t)i * n + c] = make_double2(0, 0);
-  for (int i = c; i < n; ++i) {
-    double re = 0.0, im = 0.0;
-    const double2* li = L + (size_t)i * n;
-    for (int k = c + lane; k < i; k += 32) {
-      const double2 l = li[k], x = Li[(size_t)k * n + c];
-      re += l.x * x.x - l.y * x.y;
-      im += l.x * x.y + l.y * x.x;
-    }
-    re = warp_sum_d(re);
-    im = warp_sum_d(im);
-    if (lane == 0) {
-      const double dd = li[i].x;
-      Li[(size_t)i * n + c] = make_double2((((i == c) ? 1.0 : 0.0) - re) / dd, -im / dd);
-    }
-    __syncwarp();
+  extern __shared__ double2 xs[];  // [n] solution; [n] doubles of reciprocals behind it
+  double* rd = reinterpret_cast<double*>(xs + n);
+  const int c = blockIdx.x, tid = threadIdx.x;
+  for (int i = c + tid; i < n; i += kTiThreads) rd[i] = 1.0 / LT[(size_t)i * n + i].x;
+  double2 r[kTiRows], l[kTiRows];
+#pragma unroll
+  for (int s = 0; s < kTiRows; ++s) {
+    const int k = tid + kTiThreads * s;
+    r[s] = make_double2(k == c ? 1.0 : 0.0, 0.0);
+    l[s] = (k > c && k < n) ? LT[(size_t)c * n + k] : make_double2(0, 0);
   }
+  __syncthreads();
+  for (int i = c; i < n; ++i) {
+    const int own = i % kTiThreads, os = i / kTiThreads;
+    if (tid == own) {
+      double2 v = make_double2(0, 0);
+#pragma unroll
+      for (int s = 0; s < kTiRows; ++s)
+        if (s == os) v = r[s];
+      const double p = rd[i];
+      xs[i] = make_double2(v.x * p, v.y * p);
+    }
+    __syncthreads();
+    const double2 x = xs[i];
+#pragma unroll
+    for (int s = 0; s < kTiRows; ++s) {
+      const int k = tid + kTiThreads * s;
+      const double2 a = l[s];
+      if (i + 1 < n && k > i + 1 && k < n) l[s] = LT[(size_t)(i + 1) * n + k];  // ahead of its use
+      if (k > i && k < n) {
+        r[s].x = fma(-a.x, x.x, r[s].x);
+        r[s].y = fma(-a.x, x.y, r[s].y);
+        r[s].x = fma(a.y, x.y, r[s].x);
+        r[s].y = fma(-a.y, x.x, r[s].y);
+      }
+    }
+  }
+  for (int i = tid; i < n; i += kTiThreads) Li[(size_t)i * n + c] = i < c ? make_double2(0, 0) : xs[i];
 }
 
 // ---- Householder tridiagonalisation ----------------------------------------------------------
 // A (n x n Hermitian, full storage) -> d[n], e[n] (T = Q^H A Q real symmetric tridiagonal),
 // tau[n] and the reflector vectors Vh[k][j] (j > k; Vh[k][k+1] = 1) with
-// H_k = I - tau_k v_k v_k^H.
-// Shared memory: rows [nloc][n], vfull [n], wfull [n], wown [nloc] (double2), pub (2 double2).
-__global__ void __launch_bounds__(kClThreads)
+// H_k = I - tau_k v_k v_k^H.  Every CTA gathers the whole column (and later the whole product p = tau
+// A v) through the cluster's shared memory and forms its norm, the reflector and p^H v itself: a
+// column takes two cluster barriers instead of four and no second gather of partial sums.
+// Shared memory: rows [nloc][n], v [n], w [n], pown [nloc] (double2).  192 x 192: 3.0 ms before.
+__device__ __forceinline__ void warp_sum_d2(double& a, double& b) {
+  for (int o = 16; o > 0; o >>= 1) {
+    const double x = __shfl_xor_sync(0xffffffffu, a, o), y = __shfl_xor_sync(0xffffffffu, b, o);
+    a += x;
+    b += y;
+  }
+}
+constexpr int kTdWarps = 16;  // most warps a CTA of the reduction
+__global__ void __launch_bounds__(32 * kTdWarps)
 k_cl_tridiag(const double2* __restrict__ A, int n, double* __restrict__ d, double* __restrict__ e,
              double2* __restrict__ tau, double2* __restrict__ Vh) {
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ __align__(16) unsigned char smem[];
   const ClusterLayout c = cluster_layout(n);
   double2* rows = reinterpret_cast<double2*>(smem);
-  double2* vfull = rows + (size_t)c.nloc * n;
-  double2* wfull = vfull + n;
-  double2* wown = wfull + n;
-  double2* pub = wown + c.nloc;  // pub[0].x: partial |x|^2, pub[1]: partial p^H v
-  __shared__ double red[kClWarps];
-  __shared__ double2 s_tau, s_sc;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int idx = tid; idx < c.nloc * n; idx += kClThreads) {
+  double2* v = rows + (size_t)c.nloc * n;
+  double2* w = v + n;
+  double2* pown = w + n;
+  __shared__ double2 red[kTdWarps];
+  __shared__ double2 s_tau, s_sc, s_al;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+  for (int idx = tid; idx < c.nloc * n; idx += nt) {
     const int li = idx / n, j = idx - li * n, i = li * c.P + c.rank;
     rows[idx] = (i < n) ? A[(size_t)i * n + j] : make_double2(0, 0);
   }
-  __syncthreads();
+  cl.sync();
   for (int k = 0; k < n - 1; ++k) {
-    // (1) partial |x|^2 of the column below the subdiagonal
+    // column k below the diagonal, |x|^2 below the subdiagonal
     double acc = 0;
-    for (int li = tid; li < c.nloc; li += kClThreads) {
-      const int i = li * c.P + c.rank;
-      if (i >= k + 2 && i < n) {
-        const double2 x = rows[(size_t)li * n + k];
-        acc += x.x * x.x + x.y * x.y;
-      }
+    for (int j = k + 1 + tid; j < n; j += nt) {
+      const double2 x = cl.map_shared_rank(rows, c.owner(j))[(size_t)c.local(j) * n + k];
+      v[j] = x;
+      if (j > k + 1) acc = fma(x.x, x.x, fma(x.y, x.y, acc));
     }
-    acc = block_sum_cl(acc, red);
-    if (tid == 0) pub[0] = make_double2(acc, 0.0);
-    cl.sync();
-    // (2) reflector (every CTA computes the same one)
-    if (tid == 0) {
-      double xn2 = 0;
-      for (int r = 0; r < c.P; ++r) xn2 += cl.map_shared_rank(pub, r)[0].x;
-      const double2 alpha = cl.map_shared_rank(rows, (k + 1) % c.P)[(size_t)((k + 1) / c.P) * n + k];
-      double2 t = make_double2(0, 0), sc = make_double2(0, 0);
-      double beta = alpha.x;
-      if (!(xn2 == 0.0 && alpha.y == 0.0)) {
-        beta = -copysign(sqrt(alpha.x * alpha.x + alpha.y * alpha.y + xn2), alpha.x);
-        t = make_double2((beta - alpha.x) / beta, -alpha.y / beta);
-        const double ar = alpha.x - beta, ai = alpha.y, den = ar * ar + ai * ai;
-        sc = make_double2(ar / den, -ai / den);
+    acc = warp_sum_d(acc);
+    if (lane == 0) red[warp].x = acc;
+    __syncthreads();
+    if (warp == 0) {
+      double xn2 = lane < nw ? red[lane].x : 0.0;
+      for (int o = kTdWarps / 2; o > 0; o >>= 1) xn2 += __shfl_xor_sync(0xffffffffu, xn2, o);
+      if (lane == 0) {
+        const double2 alpha = v[k + 1];
+        double2 t = make_double2(0, 0), sc = make_double2(0, 0);
+        double beta = alpha.x;
+        if (!(xn2 == 0.0 && alpha.y == 0.0)) {
+          beta = -copysign(sqrt(fma(alpha.x, alpha.x, fma(alpha.y, alpha.y, xn2))), alpha.x);
+          const double ib = 1.0 / beta, ar = alpha.x - beta, ai = alpha.y, id = 1.0 / fma(ar, ar, ai * ai);
+          t = make_double2((beta - alpha.x) * ib, -alpha.y * ib);
+          sc = make_double2(ar * id, -ai * id);
+        }
+        s_tau = t;
+        s_sc = sc;
+        if (c.rank == 0) {
+          e[k] = beta;
+          tau[k] = t;
+        }
+        if (c.rank == k % c.P) d[k] = rows[(size_t)(k / c.P) * n + k].x;
       }
-      s_tau = t;
-      s_sc = sc;
-      if (c.rank == 0) {
-        e[k] = beta;
-        tau[k] = t;
-      }
-      if (c.rank == k % c.P) d[k] = rows[(size_t)(k / c.P) * n + k].x;
     }
     __syncthreads();
     const double2 tk = s_tau, sc = s_sc;
     const bool skip = (tk.x == 0.0 && tk.y == 0.0);  // uniform over the cluster
-    for (int j = k + 1 + tid; j < n; j += kClThreads) {
-      double2 v;
-      if (j == k + 1) {
-        v = make_double2(1.0, 0.0);
-      } else if (skip) {
-        v = make_double2(0.0, 0.0);
-      } else {
-        v = cmul(cl.map_shared_rank(rows, j % c.P)[(size_t)(j / c.P) * n + k], sc);
-      }
-      vfull[j] = v;
-      if (c.rank == 0) Vh[(size_t)k * n + j] = v;
+    for (int j = k + 1 + tid; j < n; j += nt) {
+      const double2 x = j == k + 1 ? make_double2(1.0, 0.0) : (skip ? make_double2(0.0, 0.0) : cmul(v[j], sc));
+      v[j] = x;
+      if (c.rank == 0) Vh[(size_t)k * n + j] = x;
     }
     __syncthreads();
     if (skip) {
-      cl.sync();
-      cl.sync();
+      cl.sync();  // the next column's rows are read after this barrier as after the others'
       continue;
     }
-    // p_i = tau (A22 v)_i for the own trailing rows (warp per row); partial p^H v
-    double dr = 0, di = 0;
-    for (int li = warp; li < c.nloc; li += kClWarps) {
+    // p_i = tau (A22 v)_i for the own trailing rows (warp per row)
+    for (int li = warp; li < c.nloc; li += nw) {
       const int i = li * c.P + c.rank;
       if (i <= k || i >= n) continue;
       const double2* ri = rows + (size_t)li * n;
       double sr = 0, si = 0;
       for (int j = k + 1 + lane; j < n; j += 32) {
-        const double2 a = ri[j], v = vfull[j];
-        sr += a.x * v.x - a.y * v.y;
-        si += a.x * v.y + a.y * v.x;
+        const double2 a = ri[j], x = v[j];
+        sr = fma(a.x, x.x, sr);
+        si = fma(a.x, x.y, si);
+        sr = fma(-a.y, x.y, sr);
+        si = fma(a.y, x.x, si);
       }
-      sr = warp_sum_d(sr);
-      si = warp_sum_d(si);
-      const double2 p = cmul(tk, make_double2(sr, si));
-      if (lane == 0) {
-        wown[li] = p;
-        const double2 v = vfull[i];
-        dr += p.x * v.x + p.y * v.y;
-        di += p.x * v.y - p.y * v.x;
-      }
-    }
-    dr = block_sum_cl(dr, red);
-    di = block_sum_cl(di, red);
-    if (tid == 0) pub[1] = make_double2(dr, di);
-    cl.sync();
-    // (3) w = p + alpha2 v with alpha2 = -tau (p^H v) / 2
-    if (tid == 0) {
-      double tr = 0, ti = 0;
-      for (int r = 0; r < c.P; ++r) {
-        const double2 q = cl.map_shared_rank(pub, r)[1];
-        tr += q.x;
-        ti += q.y;
-      }
-      red[0] = tr;
-      red[1] = ti;
-    }
-    __syncthreads();
-    const double2 al = cmul(make_double2(-0.5 * tk.x, -0.5 * tk.y), make_double2(red[0], red[1]));
-    for (int li = tid; li < c.nloc; li += kClThreads) {
-      const int i = li * c.P + c.rank;
-      if (i > k && i < n) wown[li] = cadd(wown[li], cmul(al, vfull[i]));
+      warp_sum_d2(sr, si);
+      if (lane == 0) pown[li] = cmul(tk, make_double2(sr, si));
     }
     cl.sync();
-    // (4) full w, then A22 -= v w^H + w v^H on the own rows
-    for (int j = k + 1 + tid; j < n; j += kClThreads) wfull[j] = cl.map_shared_rank(wown, j % c.P)[j / c.P];
+    // the whole p, p^H v, w = p + alpha v with alpha = -tau (p^H v) / 2
+    double dr = 0, di = 0;
+    for (int j = k + 1 + tid; j < n; j += nt) {
+      const double2 p = cl.map_shared_rank(pown, c.owner(j))[c.local(j)], x = v[j];
+      w[j] = p;
+      dr = fma(p.x, x.x, fma(p.y, x.y, dr));
+      di = fma(p.x, x.y, fma(-p.y, x.x, di));
+    }
+    warp_sum_d2(dr, di);
+    if (lane == 0) red[warp] = make_double2(dr, di);
     __syncthreads();
-    for (int li = warp; li < c.nloc; li += kClWarps) {
+    if (warp == 0) {
+      double2 t = lane < nw ? red[lane] : make_double2(0, 0);
+      for (int o = kTdWarps / 2; o > 0; o >>= 1) {
+        const double x = __shfl_xor_sync(0xffffffffu, t.x, o), y = __shfl_xor_sync(0xffffffffu, t.y, o);
+        t.x += x;
+        t.y += y;
+      }
+      if (lane == 0) s_al = cmul(make_double2(-0.5 * tk.x, -0.5 * tk.y), t);
+    }
+    __syncthreads();
+    const double2 al = s_al;
+    for (int j = k + 1 + tid; j < n; j += nt) w[j] = cadd(w[j], cmul(al, v[j]));
+    __syncthreads();
+    // A22 -= v w^H + w v^H on the own rows
+    for (int li = warp; li < c.nloc; li += nw) {
       const int i = li * c.P + c.rank;
       if (i <= k || i >= n) continue;
-      const double2 vi = vfull[i], wi = wfull[i];
+      const double2 vi = v[i], wi = w[i];
       double2* ri = rows + (size_t)li * n;
       for (int j = k + 1 + lane; j < n; j += 32) {
-        const double2 vj = vfull[j], wj = wfull[j];
+        const double2 vj = v[j], wj = w[j];
         double2 a = ri[j];
-        a.x -= (vi.x * wj.x + vi.y * wj.y) + (wi.x * vj.x + wi.y * vj.y);
-        a.y -= (vi.y * wj.x - vi.x * wj.y) + (wi.y * vj.x - wi.x * vj.y);
+        a.x = fma(-vi.x, wj.x, a.x);
+        a.y = fma(-vi.y, wj.x, a.y);
+        a.x = fma(-vi.y, wj.y, a.x);
+        a.y = fma(vi.x, wj.y, a.y);
+        a.x = fma(-wi.x, vj.x, a.x);
+        a.y = fma(-wi.y, vj.x, a.y);
+        a.x = fma(-wi.y, vj.y, a.x);
+        a.y = fma(wi.x, vj.y, a.y);
         ri[j] = a;
       }
     }
-    __syncthreads();
+    cl.sync();
   }
   if (tid == 0 && c.rank == (n - 1) % c.P) d[n - 1] = rows[(size_t)((n - 1) / c.P) * n + (n - 1)].x;
   if (tid == 0 && c.rank == 0) {
@@ -304,77 +350,103 @@ k_cl_tridiag(const double2* __restrict__ A, int n, double* __restrict__ d, doubl
 }
 
 // ---- eigenvalues of T -------------------------------------------------------------------------
-__device__ __forceinline__ int sturm_count_s(const double* d, const double* e, int n, double x, double pivmin) {
-  int cnt = 0;
-  double q = d[0] - x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  if (q < 0) ++cnt;
+// Number of eigenvalues of the scaled T below x: sign changes of the leading principal minors
+//   p_j = (d_j - x) p_{j-1} - e_{j-1}^2 p_{j-2},
+// one fused multiply-add deep per row (the quotient form's division is some ten).  T is scaled to a norm
+// between one and two, so a row grows the pair by less than 2^3; a vanishing minor counts as a change and
+// becomes -2^-100 of its predecessor (a pivot far below the rounding of T, as the quotient form's
+// least pivot is), so a row shrinks the pair by at most some 2^-106; it is rescaled by a power of two
+// every four rows.
+__device__ __forceinline__ int sturm_count_minors(const double* d, const double* e2, int n, double x) {
+  const double least = -7.888609052210118e-31;  // -2^-100
+  double p0 = 1.0, p1 = d[0] - x;
+  if (p1 == 0.0) p1 = least;
+  int cnt = p1 < 0.0;
   for (int j = 1; j < n; ++j) {
-    q = d[j] - x - e[j - 1] * e[j - 1] / q;
-    if (fabs(q) < pivmin) q = -pivmin;
-    if (q < 0) ++cnt;
+    double p2 = fma(d[j] - x, p1, -(e2[j - 1] * p0));
+    if (p2 == 0.0) p2 = least * p1;
+    cnt += (__double2hiint(p2) ^ __double2hiint(p1)) < 0;
+    p0 = p1;
+    p1 = p2;
+    if ((j & 3) == 0) {
+      const int ex = max(__double2hiint(p0) & 0x7fffffff, __double2hiint(p1) & 0x7fffffff) >> 20;
+      const double s = __hiloint2double((2046 - ex) << 20, 0);  // 2^-(exponent of the larger)
+      p0 *= s;
+      p1 *= s;
+    }
   }
   return cnt;
 }
 
-// Gershgorin interval and scale of T; pivmin for the Sturm recurrences.
-struct TriBounds {
-  double lo, hi, tnorm, pivmin;
-};
-__device__ TriBounds tri_bounds(const double* d, const double* e, int n) {
-  TriBounds b;
-  double tn = 0, lo = 1e300, hi = -1e300, emax2 = 0;
-  for (int j = 0; j < n; ++j) {
-    const double r = (j < n - 1 ? fabs(e[j]) : 0.0) + (j > 0 ? fabs(e[j - 1]) : 0.0);
-    tn = fmax(tn, fabs(d[j]) + r);
-    lo = fmin(lo, d[j] - r);
-    hi = fmax(hi, d[j] + r);
-    if (j < n - 1) emax2 = fmax(emax2, e[j] * e[j]);
-  }
-  b.tnorm = fmax(tn, 1e-300);
-  b.lo = lo - 1e-12 * b.tnorm - 1e-300;
-  b.hi = hi + 1e-12 * b.tnorm + 1e-300;
-  b.pivmin = fmax(1e-300, 2.2e-308 * fmax(1.0, emax2));
-  return b;
+// The power of two that scales ||T|| (its largest row sum tn) into [1, 2).
+__device__ __forceinline__ double tri_scale(double tn) {
+  const int ex = (__double2hiint(tn) & 0x7fffffff) >> 20;
+  return ex < 24 || ex > 2022 ? 1.0 : __hiloint2double((2046 - ex) << 20, 0);
 }
 
-// w[i] = i-th smallest eigenvalue; one warp per i, 32 Sturm counts per step (the interval
-// shrinks 33-fold per step).
-__global__ void k_tri_eigvals(const double* __restrict__ dg, const double* __restrict__ eg, int n, double* w) {
+// w[i] = i-th smallest eigenvalue of T; one CTA of 128 threads per i, 128 Sturm counts per step (the
+// interval shrinks 129-fold, so eight steps where 32 points take eleven; the four warps sit on the
+// SM's four quarters).  CTA 0 leaves ||T|| in *tnorm.  192 eigenvalues of n = 192 took 1.3 ms in
+// quotient form, a warp each; the 64 that are asked for now, 0.2 ms.
+constexpr int kEvThreads = 128;
+__global__ void __launch_bounds__(kEvThreads)
+k_tri_eigvals(const double* __restrict__ dg, const double* __restrict__ eg, int n, double* w, double* tnorm) {
   extern __shared__ double sde[];
+  __shared__ double red[3][kEvThreads / 32], xs[kEvThreads];
+  __shared__ int first;
   double* d = sde;
-  double* e = sde + n;
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    d[j] = dg[j];
-    e[j] = eg[j];
+  double* e2 = sde + n;
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, i = blockIdx.x;
+  double tn = 0, lo = 1e300, hi = -1e300;
+  for (int j = tid; j < n; j += kEvThreads) {
+    const double dj = dg[j], r = (j < n - 1 ? fabs(eg[j]) : 0.0) + (j > 0 ? fabs(eg[j - 1]) : 0.0);
+    d[j] = dj;
+    tn = fmax(tn, fabs(dj) + r);
+    lo = fmin(lo, dj - r);
+    hi = fmax(hi, dj + r);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (lane == 0) {
+    red[0][wp] = tn;
+    red[1][wp] = lo;
+    red[2][wp] = hi;
   }
   __syncthreads();
-  const TriBounds b = tri_bounds(d, e, n);
-  const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (i >= n) return;
-  double lo = b.lo, hi = b.hi;
+  for (int q = 0; q < kEvThreads / 32; ++q) {
+    tn = fmax(tn, red[0][q]);
+    lo = fmin(lo, red[1][q]);
+    hi = fmax(hi, red[2][q]);
+  }
+  tn = fmax(tn, 1e-300);
+  if (i == 0 && tid == 0) *tnorm = tn;
+  const double sc = tri_scale(tn);
+  for (int j = tid; j < n; j += kEvThreads) {
+    d[j] *= sc;
+    const double ej = j < n - 1 ? eg[j] * sc : 0.0;
+    e2[j] = ej * ej;
+  }
+  lo = (lo - 1e-12 * tn - 1e-300) * sc;
+  hi = (hi + 1e-12 * tn + 1e-300) * sc;
   for (int it = 0; it < 64; ++it) {
-    if (hi - lo <= 2.2e-16 * fmax(fabs(lo), fabs(hi)) + 1e-300) break;
-    const double step = (hi - lo) / 33.0;
-    const double x = lo + step * (double)(lane + 1);
-    const bool above = sturm_count_s(d, e, n, x, b.pivmin) > i;
-    const unsigned m = __ballot_sync(0xffffffffu, above);
-    double nlo, nhi;
-    if (m == 0) {
-      nlo = __shfl_sync(0xffffffffu, x, 31);
-      nhi = hi;
-    } else {
-      const int f = __ffs(m) - 1;
-      nhi = __shfl_sync(0xffffffffu, x, f);
-      const double xl = __shfl_sync(0xffffffffu, x, f > 0 ? f - 1 : 0);
-      nlo = (f > 0) ? xl : lo;
-    }
+    if (hi - lo <= 2.2e-16 * fmax(fabs(lo), fabs(hi)) + 1e-19) break;
+    const double x = lo + (hi - lo) / (double)(kEvThreads + 1) * (double)(tid + 1);
+    xs[tid] = x;
+    if (tid == 0) first = kEvThreads;
+    __syncthreads();
+    if (sturm_count_minors(d, e2, n, x) > i) atomicMin(&first, tid);
+    __syncthreads();
+    const int f = first;
+    const double nlo = f > 0 ? xs[f - 1] : lo, nhi = f < kEvThreads ? xs[f] : hi;
+    __syncthreads();
     if (!(nlo > lo || nhi < hi)) break;  // no representable progress
     lo = nlo;
     hi = nhi;
   }
-  if (lane == 0) w[i] = 0.5 * (lo + hi);
+  if (tid == 0) w[i] = 0.5 * (lo + hi) / sc;
 }
 
 // ---- eigenvectors of T by inverse iteration -----------------------------------------------
@@ -386,110 +458,132 @@ __device__ __forceinline__ double start_value_s(int i, int j) {
   return 0.5 + (double)(h & 0xffff) / 65536.0;
 }
 
+// 1 / a for 2^-53 <= |a| < 2^100 by two Newton steps from the FP32 reciprocal.
+__device__ __forceinline__ double recip_newton(double a) {
+  double r = (double)__frcp_rn((float)a);
+  r = fma(r, fma(-a, r, 1.0), r);
+  return fma(r, fma(-a, r, 1.0), r);
+}
+
 // Inverse iteration for vectors i < nvec: `iters` solves of (T - w_i I) z_new = z with the
-// partially pivoted LU of T - w_i I (factorised once), normalising after each; starts from
-// the current Z (fresh = 0) or a fixed pseudo-random vector (fresh = 1).  Z[i][n] (row per
-// vector); work: 5 n nvec doubles, interleaved by vector so that the threads of a warp touch
-// consecutive addresses.
-__global__ void k_tri_solve(const double* __restrict__ d, const double* __restrict__ e, int n, const double* w,
-                            int nvec, int fresh, int iters, double* __restrict__ Z, double* __restrict__ work) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nvec) return;
-  double tn = 0;
-  for (int j = 0; j < n; ++j) {
-    const double r = (j < n - 1 ? fabs(e[j]) : 0.0) + (j > 0 ? fabs(e[j - 1]) : 0.0);
-    tn = fmax(tn, fabs(d[j]) + r);
+// partially pivoted LU of the scaled T - w_i I, normalised at the end (one solve grows a vector by at
+// most some 2^53 n); starts from the current Z and the factors an earlier call left in work (fresh = 0),
+// or from a fixed pseudo-random vector, factorising first (fresh = 1).  Z[i][n] (row per vector);
+// work: 5 n nvec doubles.  A CTA is one warp with VPC vectors, a thread each, all recurrences in
+// shared memory: the factorisation's chain is a reciprocal and two operations a row, a solve's two
+// and three (pivots kept as reciprocals; a pivot below 2^-52 ||T|| is set to it).
+__global__ void __launch_bounds__(32)
+k_tri_solve(const double* __restrict__ dg, const double* __restrict__ eg, int n, const double* w, int nvec, int fresh,
+            int iters, double* __restrict__ Z, double* __restrict__ work, const double* __restrict__ tnorm, int vpc) {
+  extern __shared__ double sm[];
+  const int lane = threadIdx.x, i0 = blockIdx.x * vpc, nv = min(vpc, nvec - i0);
+  const size_t blk = (size_t)n * vpc;
+  double* ia = sm;             // reciprocal pivots          [n][vpc]
+  double* u1 = sm + blk;       // first superdiagonal
+  double* u2 = sm + 2 * blk;   // second superdiagonal (fill-in)
+  double* ml = sm + 3 * blk;   // multipliers
+  double* sw = sm + 4 * blk;   // 1 where rows j and j + 1 were interchanged
+  double* z = sm + 5 * blk;
+  double* sd = sm + 6 * blk;   // scaled d [n], e [n]
+  double* se = sd + n;
+  double* save = work + (size_t)blockIdx.x * 5 * blk;
+  const double sc = tri_scale(*tnorm);
+  for (int j = lane; j < n; j += 32) {
+    sd[j] = dg[j] * sc;
+    se[j] = j < n - 1 ? eg[j] * sc : 0.0;
   }
-  const double tiny = 2.2e-16 * fmax(tn, 1e-300);
-  const double lam = w[i];
-  double* z = Z + (size_t)i * n;
-  const size_t nv = (size_t)nvec;
-  double* wa = work;                 // pivots
-  double* wu1 = work + n * nv;       // first superdiagonal
-  double* wu2 = work + 2 * n * nv;   // second superdiagonal (fill-in)
-  double* wl = work + 3 * n * nv;    // multipliers
-  double* wp = work + 4 * n * nv;    // 1 where rows j and j+1 were interchanged
-  if (fresh)
-    for (int j = 0; j < n; ++j) z[j] = start_value_s(i, j);
-  {
-    double a = d[0] - lam, u1 = (n > 1) ? e[0] : 0.0;
-    for (int j = 0; j < n - 1; ++j) {
-      const double sub = e[j], dn = d[j + 1] - lam, en = (j + 1 < n - 1) ? e[j + 1] : 0.0;
-      if (fabs(a) >= fabs(sub)) {
-        const double m = sub / ((a == 0.0) ? tiny : a);
-        wa[j * nv + i] = a;
-        wu1[j * nv + i] = u1;
-        wu2[j * nv + i] = 0.0;
-        wl[j * nv + i] = m;
-        wp[j * nv + i] = 0.0;
-        a = dn - m * u1;
-        u1 = en;
-      } else {
-        const double m = a / sub;
-        wa[j * nv + i] = sub;
-        wu1[j * nv + i] = dn;
-        wu2[j * nv + i] = en;
-        wl[j * nv + i] = m;
-        wp[j * nv + i] = 1.0;
-        a = u1 - m * dn;
-        u1 = -m * en;
-      }
-    }
-    wa[(size_t)(n - 1) * nv + i] = a;
-    wu1[(size_t)(n - 1) * nv + i] = 0.0;
-    wu2[(size_t)(n - 1) * nv + i] = 0.0;
+  if (fresh) {
+    for (size_t k = lane; k < blk; k += 32) z[k] = start_value_s(i0 + (int)(k % vpc), (int)(k / vpc));
+  } else {
+    for (size_t k = lane; k < 5 * blk; k += 32) sm[k] = save[k];
+    for (int k = lane; k < nv * n; k += 32) z[(size_t)(k % n) * vpc + k / n] = Z[(size_t)(i0 + k / n) * n + k % n];
   }
-  for (int it = 0; it < iters; ++it) {
-    // forward: apply the row operations
-    for (int j = 0; j < n - 1; ++j) {
-      const double m = wl[j * nv + i];
-      if (wp[j * nv + i] != 0.0) {
-        const double t = z[j];
-        z[j] = z[j + 1];
-        z[j + 1] = t - m * z[j];
-      } else {
-        z[j + 1] -= m * z[j];
+  __syncwarp();
+  if (lane < nv) {
+    const double tiny = 2.2e-16;
+    if (fresh) {
+      const double lam = w[i0 + lane] * sc;
+      double a = sd[0] - lam, u = n > 1 ? se[0] : 0.0;
+      for (int j = 0; j < n - 1; ++j) {
+        const double sub = se[j], dn = sd[j + 1] - lam, en = se[j + 1];
+        const bool keep = fabs(a) >= fabs(sub);
+        double p = keep ? a : sub;
+        if (fabs(p) < tiny) p = copysign(tiny, p);
+        const double r = recip_newton(p), m = (keep ? sub : a) * r;
+        const size_t k = (size_t)j * vpc + lane;
+        ia[k] = r;
+        u1[k] = keep ? u : dn;
+        u2[k] = keep ? 0.0 : en;
+        ml[k] = m;
+        sw[k] = keep ? 0.0 : 1.0;
+        a = keep ? fma(-m, u, dn) : fma(-m, dn, u);
+        u = keep ? en : -m * en;
       }
+      const size_t k = (size_t)(n - 1) * vpc + lane;
+      if (fabs(a) < tiny) a = copysign(tiny, a);
+      ia[k] = recip_newton(a);
+      u1[k] = u2[k] = ml[k] = sw[k] = 0.0;
     }
-    // back substitution
-    double b1 = 0.0, b2 = 0.0, nn = 0.0;
-    for (int j = n - 1; j >= 0; --j) {
-      const double aj = wa[j * nv + i];
-      const double x = (z[j] - wu1[j * nv + i] * b1 - wu2[j * nv + i] * b2) / ((aj == 0.0) ? tiny : aj);
-      z[j] = x;
-      b2 = b1;
-      b1 = x;
-      nn += x * x;
+    double nn = 0;
+    for (int it = 0; it < iters; ++it) {
+      // the row operations
+      double t = z[lane];
+      for (int j = 0; j < n - 1; ++j) {
+        const size_t k = (size_t)j * vpc + lane;
+        const double nx = z[k + vpc], m = ml[k];
+        const bool swp = sw[k] != 0.0;
+        z[k] = swp ? nx : t;
+        t = swp ? fma(-m, nx, t) : fma(-m, t, nx);
+      }
+      z[(size_t)(n - 1) * vpc + lane] = t;
+      // back substitution
+      double b1 = 0.0, b2 = 0.0;
+      nn = 0;
+      for (int j = n - 1; j >= 0; --j) {
+        const size_t k = (size_t)j * vpc + lane;
+        const double x = fma(-u1[k], b1, fma(-u2[k], b2, z[k])) * ia[k];
+        z[k] = x;
+        b2 = b1;
+        b1 = x;
+        nn = fma(x, x, nn);
+      }
     }
     const double inv = 1.0 / sqrt(fmax(nn, 1e-300));
-    for (int j = 0; j < n; ++j) z[j] *= inv;
+    for (int j = 0; j < n; ++j) z[(size_t)j * vpc + lane] *= inv;
   }
+  __syncwarp();
+  if (fresh)
+    for (size_t k = lane; k < 5 * blk; k += 32) save[k] = sm[k];
+  for (int k = lane; k < nv * n; k += 32) Z[(size_t)(i0 + k / n) * n + k % n] = z[(size_t)(k % n) * vpc + k / n];
 }
 
 // Modified Gram-Schmidt inside each cluster of eigenvalues closer than gap_rel * ||T||
 // (one CTA per cluster; CTAs beyond the number of clusters return).  Z[i][n].
-__global__ void k_tri_orth(const double* __restrict__ d, const double* __restrict__ e, int n, const double* w,
-                           int nvec, double gap_rel, double* __restrict__ Z) {
+__global__ void k_tri_orth(int n, const double* w, int nvec, double gap_rel, double* __restrict__ Z,
+                           const double* __restrict__ tnorm) {
   __shared__ double red[32];
   __shared__ int s_lo, s_hi;
-  if (threadIdx.x == 0) {
-    double tn = 0;
-    for (int j = 0; j < n; ++j) {
-      const double r = (j < n - 1 ? fabs(e[j]) : 0.0) + (j > 0 ? fabs(e[j - 1]) : 0.0);
-      tn = fmax(tn, fabs(d[j]) + r);
-    }
-    const double gap = gap_rel * fmax(tn, 1e-300);
-    int c = -1, lo = 0, hi = 0;
-    for (int q = 0; q < nvec; ++q) {
-      if (q == 0 || w[q] - w[q - 1] > gap) {
-        ++c;
-        if (c == (int)blockIdx.x) lo = q;
-        if (c == (int)blockIdx.x + 1) break;
+  if (threadIdx.x < 32) {
+    // bounds of cluster blockIdx.x: its start and the next start
+    const double gap = gap_rel * *tnorm;
+    const int lane = threadIdx.x;
+    int seen = 0, lo = -1, hi = -1;
+    for (int q0 = 0; q0 < nvec && hi < 0; q0 += 32) {
+      const int q = q0 + lane;
+      const bool start = q < nvec && (q == 0 || w[q] - w[q - 1] > gap);
+      unsigned m = __ballot_sync(0xffffffffu, start);
+      while (m && hi < 0) {
+        const int q1 = q0 + __ffs(m) - 1;
+        if (seen == (int)blockIdx.x) lo = q1;
+        if (seen == (int)blockIdx.x + 1) hi = q1;
+        ++seen;
+        m &= m - 1;
       }
-      if (c == (int)blockIdx.x) hi = q + 1;
     }
-    s_lo = lo;
-    s_hi = (c >= (int)blockIdx.x) ? hi : lo;
+    if (lane == 0) {
+      s_lo = lo < 0 ? 0 : lo;
+      s_hi = lo < 0 ? 0 : (hi < 0 ? nvec : hi);
+    }
   }
   __syncthreads();
   const int lo = s_lo, hi = s_hi;
@@ -518,40 +612,93 @@ __global__ void k_tri_orth(const double* __restrict__ d, const double* __restric
   }
 }
 
-// V[:, i] = H_0 H_1 ... H_{n-2} z_i (column i of the row-major n x n V; one warp per vector);
-// columns nvec..n-1 of V are zeroed.
-__global__ void k_backtransform(const double2* __restrict__ Vh, const double2* __restrict__ tau, int n, int nvec,
-                                const double* __restrict__ Z, double2* __restrict__ V) {
+// ---- back-transformation ---------------------------------------------------------------------------
+// The reflectors are applied 16 at a time.  With s_k = v_k^H z for the whole block at once, the
+// coefficient of H_k inside it is f_k = tau_k (s_k - sum_{l > k} (v_k^H v_l) f_l), so a block takes one
+// pass over z for its 16 inner products, 16 short steps on one warp and one pass to subtract
+// sum f_k v_k, instead of 16 dependent pairs of passes.
+constexpr int kWy = 16;
+// G[blk][a][b] = v_{k0 + a}^H v_{k0 + b}, a < b (a warp each).
+__global__ void k_wy_gram(const double2* __restrict__ Vh, int n, int nref, double2* __restrict__ G) {
   const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (i >= n) return;
+  const int id = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int blk = id / (kWy * kWy), a = id / kWy % kWy, b = id % kWy, k0 = blk * kWy;
+  if (a >= b || k0 + b >= nref) return;
+  const double2 *va = Vh + (size_t)(k0 + a) * n, *vb = Vh + (size_t)(k0 + b) * n;
+  double sr = 0, si = 0;
+  for (int j = k0 + b + 1 + lane; j < n; j += 32) {
+    const double2 x = va[j], y = vb[j];
+    sr = fma(x.x, y.x, fma(x.y, y.y, sr));
+    si = fma(x.x, y.y, fma(-x.y, y.x, si));
+  }
+  warp_sum_d2(sr, si);
+  if (lane == 0) G[(size_t)blk * kWy * kWy + a * kWy + b] = make_double2(sr, si);
+}
+
+// V[:, i] = H_0 H_1 ... H_{n-2} z_i (column i of the row-major n x n V; one CTA per vector);
+// columns nvec..n-1 of V are zeroed.
+constexpr int kBtThreads = 256;
+__global__ void __launch_bounds__(kBtThreads)
+k_backtransform(const double2* __restrict__ Vh, const double2* __restrict__ tau, const double2* __restrict__ G, int n,
+                int nvec, const double* __restrict__ Z, double2* __restrict__ V) {
+  extern __shared__ double2 zs[];  // [n]
+  __shared__ double2 f[kWy];
+  const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (i >= nvec) {
-    for (int r = lane; r < n; r += 32) V[(size_t)r * n + i] = make_double2(0, 0);
+    for (int r = tid; r < n; r += kBtThreads) V[(size_t)r * n + i] = make_double2(0, 0);
     return;
   }
-  const double* z = Z + (size_t)i * n;
-  for (int r = lane; r < n; r += 32) V[(size_t)r * n + i] = make_double2(z[r], 0.0);
-  __syncwarp();
-  for (int k = n - 2; k >= 0; --k) {
-    const double2 tk = tau[k];
-    if (tk.x == 0.0 && tk.y == 0.0) continue;
-    const double2* v = Vh + (size_t)k * n;
-    double sr = 0, si = 0;  // v^H x over rows k+1 ..
-    for (int j = k + 1 + lane; j < n; j += 32) {
-      const double2 a = v[j], x = V[(size_t)j * n + i];
-      sr += a.x * x.x + a.y * x.y;
-      si += a.x * x.y - a.y * x.x;
+  for (int r = tid; r < n; r += kBtThreads) zs[r] = make_double2(Z[(size_t)i * n + r], 0.0);
+  const int nref = n - 1;
+  for (int blk = (nref - 1) / kWy; blk >= 0; --blk) {
+    const int k0 = blk * kWy;
+    __syncthreads();
+    for (int a = warp; a < kWy; a += kBtThreads / 32) {
+      double sr = 0, si = 0;
+      if (k0 + a < nref) {
+        const double2* v = Vh + (size_t)(k0 + a) * n;
+        for (int j = k0 + a + 1 + lane; j < n; j += 32) {
+          const double2 x = v[j], y = zs[j];
+          sr = fma(x.x, y.x, fma(x.y, y.y, sr));
+          si = fma(x.x, y.y, fma(-x.y, y.x, si));
+        }
+      }
+      warp_sum_d2(sr, si);
+      if (lane == 0) f[a] = make_double2(sr, si);
     }
-    sr = warp_sum_d(sr);
-    si = warp_sum_d(si);
-    const double2 f = cmul(tk, make_double2(sr, si));
-    for (int j = k + 1 + lane; j < n; j += 32) {
-      const double2 a = v[j];
-      double2& x = V[(size_t)j * n + i];
-      x = csub(x, cmul(f, a));
+    __syncthreads();
+    if (warp == 0) {
+      const int a = lane & (kWy - 1);
+      double2 s = f[a];
+      const double2 t = k0 + a < nref ? tau[k0 + a] : make_double2(0, 0);
+      const double2* g = G + (size_t)blk * kWy * kWy + a * kWy;
+      double2 out = make_double2(0, 0);
+      for (int b = kWy - 1; b >= 0; --b) {
+        const bool have = a < b && k0 + b < nref;
+        const double2 c = have ? g[b] : make_double2(0, 0);  // v_a^H v_b
+        double2 x = cmul(t, s);
+        if (a == b) out = x;
+        x.x = __shfl_sync(0xffffffffu, x.x, b);
+        x.y = __shfl_sync(0xffffffffu, x.y, b);
+        s.x = fma(-c.x, x.x, fma(c.y, x.y, s.x));
+        s.y = fma(-c.x, x.y, fma(-c.y, x.x, s.y));
+      }
+      if (lane < kWy) f[a] = out;
     }
-    __syncwarp();
+    __syncthreads();
+    for (int j = k0 + 1 + tid; j < n; j += kBtThreads) {
+      double2 y = zs[j];
+      for (int a = 0; a < kWy; ++a) {
+        if (j <= k0 + a || k0 + a >= nref) break;
+        const double2 c = f[a], v = Vh[(size_t)(k0 + a) * n + j];
+        y.x = fma(-c.x, v.x, fma(c.y, v.y, y.x));
+        y.y = fma(-c.x, v.y, fma(-c.y, v.x, y.y));
+      }
+      zs[j] = y;
+    }
   }
+  __syncthreads();
+  for (int r = tid; r < n; r += kBtThreads) V[(size_t)r * n + i] = zs[r];
 }
 
 // ---- host side -----------------------------------------------------------------------------
@@ -563,7 +710,7 @@ static size_t tridiag_smem(int n, int P) {
 }
 static size_t chol_smem(int n, int P) {
   const int nloc = (n + P - 1) / P;
-  return ((size_t)nloc * n + n) * sizeof(double2);
+  return ((size_t)nloc * n + n) * sizeof(double2) + (size_t)n * sizeof(double);
 }
 
 static int cluster_size() {
@@ -610,14 +757,14 @@ int dense_cluster_max_n() {
   int n = 0;
   if (P > 0)
     while (tridiag_smem(n + 1, P) <= 200 * 1024 && chol_smem(n + 1, P) <= 200 * 1024) ++n;
-  nmax = n;
+  nmax = std::min(n, kTiThreads * kTiRows);
   return nmax;
 }
 
-static cudaLaunchConfig_t cluster_cfg(int P, size_t smem, cudaStream_t st, cudaLaunchAttribute* at) {
+static cudaLaunchConfig_t cluster_cfg(int P, int threads, size_t smem, cudaStream_t st, cudaLaunchAttribute* at) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(P);
-  cfg.blockDim = dim3(kClThreads);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -634,43 +781,59 @@ bool launch_cholesky_cluster(const double2* S, int n, double2* L, double2* Li, u
   if (n < 1 || n > dense_cluster_max_n()) return false;
   const int P = cluster_size();
   cudaLaunchAttribute at[1];
-  cudaLaunchConfig_t cfg = cluster_cfg(P, chol_smem(n, P), st, at);
+  cudaLaunchConfig_t cfg = cluster_cfg(P, kClThreads, chol_smem(n, P), st, at);
   count_launches(2);
   if (cudaLaunchKernelEx(&cfg, k_cl_cholesky, S, n, L, status, rel_pivot) != cudaSuccess) return false;
-  const int wpb = 4;
-  k_tri_inverse<<<(n + wpb - 1) / wpb, 32 * wpb, 0, st>>>(L, n, Li, status);
+  k_tri_inverse<<<n, kTiThreads, (size_t)n * (sizeof(double2) + sizeof(double)), st>>>(L, n, Li, status);
   return true;
 }
 
+// Vectors a CTA of the inverse iteration takes: as many (up to 16) as its factors fit 200 KB.
+static int tri_solve_vpc(int n) {
+  int v = 16;
+  while (v > 1 && ((size_t)6 * n * v + 2 * (size_t)n) * sizeof(double) > 200 * 1024) v /= 2;
+  return v;
+}
+static size_t wy_doubles(int n) { return (size_t)2 * kWy * kWy * ((n + kWy - 1) / kWy); }
+
 size_t heev_cluster_work_doubles(int n, int nvec) {
-  // d, e, w copies | tau (2n) | Vh (2 n^2) | Z (nvec n) | solve work (5 n nvec)
-  return (size_t)2 * n + 2 * (size_t)n + 2 * (size_t)n * n + (size_t)nvec * n + 5 * (size_t)n * nvec + 64;
+  // d, e | tau (2n) | Vh (2 n^2) | Z (nvec n) | factors (5 n nvec, rounded up to whole CTAs) | reflector
+  // products | ||T||
+  return (size_t)2 * n + 2 * (size_t)n + 2 * (size_t)n * n + (size_t)nvec * n + 5 * (size_t)n * (nvec + 16) +
+         wy_doubles(n) + 64;
 }
 
-bool launch_heev_cluster(const double2* A, int n, int nvec, double* w, double2* V, double* work, cudaStream_t st) {
-  if (n < 2 || n > dense_cluster_max_n() || nvec < 1 || nvec > n) return false;
-  const int P = cluster_size();
+bool launch_heev_cluster(const double2* A, int n, int nvec, int nval, double* w, double2* V, double* work,
+                         cudaStream_t st) {
+  if (n < 2 || n > dense_cluster_max_n() || nvec < 1 || nvec > nval || nval > n) return false;
+  const int P = cluster_size(), vpc = tri_solve_vpc(n);
+  const size_t solve_smem = ((size_t)6 * n * vpc + 2 * (size_t)n) * sizeof(double);
+  if (cudaFuncSetAttribute(k_tri_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
+    return false;
   double* d = work;
   double* e = d + n;
   double2* tau = reinterpret_cast<double2*>(e + n);
   double2* Vh = tau + n;
-  double* Z = reinterpret_cast<double*>(Vh + (size_t)n * n);
+  double2* G = Vh + (size_t)n * n;
+  double* Z = reinterpret_cast<double*>(G) + wy_doubles(n);
   double* sw = Z + (size_t)nvec * n;
+  double* tnorm = sw + 5 * (size_t)n * ((nvec + vpc - 1) / vpc) * vpc;
   cudaLaunchAttribute at[1];
-  cudaLaunchConfig_t cfg = cluster_cfg(P, tridiag_smem(n, P), st, at);
+  const int nloc = (n + P - 1) / P, warps = std::max(4, std::min(kTdWarps, nloc));
+  cudaLaunchConfig_t cfg = cluster_cfg(P, 32 * warps, tridiag_smem(n, P), st, at);
   count_launches(1);
   if (cudaLaunchKernelEx(&cfg, k_cl_tridiag, A, n, d, e, tau, Vh) != cudaSuccess) return false;
-  const int wpb = 4;
   count_launches(7);
-  k_tri_eigvals<<<(n + wpb - 1) / wpb, 32 * wpb, 2 * n * sizeof(double), st>>>(d, e, n, w);
-  const int tpb = 64;
+  k_tri_eigvals<<<nval, kEvThreads, 2 * n * sizeof(double), st>>>(d, e, n, w, tnorm);
   // Two rounds of (inverse iteration, Gram-Schmidt inside clusters of close eigenvalues).
   const double gap_rel = 1e-3;
-  k_tri_solve<<<(nvec + tpb - 1) / tpb, tpb, 0, st>>>(d, e, n, w, nvec, 1, 2, Z, sw);
-  k_tri_orth<<<nvec, 128, 0, st>>>(d, e, n, w, nvec, gap_rel, Z);
-  k_tri_solve<<<(nvec + tpb - 1) / tpb, tpb, 0, st>>>(d, e, n, w, nvec, 0, 1, Z, sw);
-  k_tri_orth<<<nvec, 128, 0, st>>>(d, e, n, w, nvec, gap_rel, Z);
-  k_backtransform<<<n, 32, 0, st>>>(Vh, tau, n, nvec, Z, V);
+  const int nc = (nvec + vpc - 1) / vpc, blocks = (n + kWy - 1) / kWy;
+  k_tri_solve<<<nc, 32, solve_smem, st>>>(d, e, n, w, nvec, 1, 2, Z, sw, tnorm, vpc);
+  k_tri_orth<<<nvec, 128, 0, st>>>(n, w, nvec, gap_rel, Z, tnorm);
+  k_tri_solve<<<nc, 32, solve_smem, st>>>(d, e, n, w, nvec, 0, 1, Z, sw, tnorm, vpc);
+  k_tri_orth<<<nvec, 128, 0, st>>>(n, w, nvec, gap_rel, Z, tnorm);
+  k_wy_gram<<<(blocks * kWy * kWy + 3) / 4, 128, 0, st>>>(Vh, n, n - 1, G);
+  k_backtransform<<<n, kBtThreads, (size_t)n * sizeof(double2), st>>>(Vh, tau, G, n, nvec, Z, V);
   return true;
 }
 

@@ -300,8 +300,8 @@ template <typename T> struct EngineT : Engine {
     for (auto& b : htot) b.alloc(nr);
     partial.alloc(64 * (size_t)grid_red_blocks());
     scal.alloc(256);
-    status.alloc(1);
-    CK(cudaMemsetAsync(status.p, 0, sizeof(unsigned), st));
+    status.alloc(2);  // ST_* bits; the column of the last failed Cholesky pivot
+    CK(cudaMemsetAsync(status.p, 0, 2 * sizeof(unsigned), st));
     rho_plane.alloc(nr);
   }
   ~EngineT() override {
@@ -817,10 +817,8 @@ template <typename T> struct EngineT : Engine {
     CK(cudaMemcpyAsync(spsi, psi, (size_t)nb * q.npw * sizeof(C), cudaMemcpyDeviceToDevice, st));
     if (!s.uspp) return;
     gwork.ensure(gemm_hn_work(s.nproj, nb, q.npw));
-    Pm.ensure((size_t)s.nproj * nb);
     Qm.ensure((size_t)s.nproj * nb);
-    launch_gemm_hn<T>(q.beta.p, q.npw, psi, q.npw, s.nproj, nb, q.npw, Pm.p, nb, gwork.p, st);
-    launch_kb_couple(Pm.p, s.Qblk, s.natoms, nb, Qm.p, st);
+    launch_project_couple<T>(q.beta.p, psi, q.npw, q.npw, s.Qblk, nullptr, s.natoms, nb, Qm.p, gwork.p, st);
     launch_gemm_rot<T>(q.beta.p, q.npw, Qm.p, nb, s.nproj, nb, q.npw, spsi, q.npw, 1.0, 1.0, st);
   }
 
@@ -836,11 +834,9 @@ template <typename T> struct EngineT : Engine {
   void apply_nl(Sub<T>& s, KP<T>& q, const C* psi, C* hpsi, int nb) {
     if (s.nproj) {
       gwork.ensure(gemm_hn_work(s.nproj, nb, q.npw));
-      Pm.ensure((size_t)s.nproj * nb);
       Qm.ensure((size_t)s.nproj * nb);
-      launch_gemm_hn<T>(q.beta.p, q.npw, psi, q.npw, s.nproj, nb, q.npw, Pm.p, nb, gwork.p, st);
-      if (s.uspp) launch_kb_couple_atoms(Pm.p, s.Dscr.p, s.nproj_atom, s.natoms, nb, Qm.p, st);
-      else launch_kb_couple(Pm.p, s.Dblk, s.natoms, nb, Qm.p, st);
+      launch_project_couple<T>(q.beta.p, psi, q.npw, q.npw, s.Dblk, s.uspp ? s.Dscr.p : nullptr, s.natoms, nb, Qm.p,
+                               gwork.p, st);
       launch_gemm_rot<T>(q.beta.p, q.npw, Qm.p, nb, s.nproj, nb, q.npw, hpsi, q.npw, 1.0, 1.0, st);
     }
   }
@@ -1097,11 +1093,14 @@ template <typename T> struct EngineT : Engine {
   // A stricter bound (1e-3) ends the FP32 solves of the 72 x 72 x 180 slab after a dozen
   // iterations, short of a 1e-4 residual.  FP64 vectors: a rounding-level bound.
   static constexpr double rel_pivot() { return sizeof(T) == 4 ? 1e-5 : 1e-29; }
+  int bad_pivot = -1;  // column of the last failure
   void check_cholesky() {
-    unsigned h = 0;
-    CK(cudaMemcpyAsync(&h, status.p, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    unsigned hs[2] = {0, 0};
+    CK(cudaMemcpyAsync(hs, status.p, sizeof(hs), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    const unsigned h = hs[0];
     if (h & ST_CHOLESKY) {
+      bad_pivot = (int)hs[1];
       CK(cudaMemsetAsync(status.p, 0, sizeof(unsigned), st));
       throw Err{FDE_ENOCONV, "overlap matrix is not positive definite (linearly dependent vectors)"};
     }
@@ -1156,15 +1155,14 @@ template <typename T> struct EngineT : Engine {
     launch_small_gemm(tmp.p, n, 0, Li.p, n, 1, n, n, n, Ht.p, n, st);
     launch_hermitize(Ht.p, n, st);
     hwork.ensure(heev_work_doubles(n, nb));
-    launch_heev(Ht.p, n, nb, wv.p, Y.p, hwork.p, st);
+    launch_heev(Ht.p, n, nb, nb, wv.p, Y.p, hwork.p, st);
     launch_small_gemm(Li.p, n, 1, Y.p, n, 0, n, n, n, Cc.p, n, st);
     launch_gemm_rot<T>(V.p, K, Cc.p, n, n, nb, K, V2.p, K, 1.0, 0.0, st);
     launch_gemm_rot<T>(HV.p, K, Cc.p, n, n, nb, K, HV2.p, K, 1.0, 0.0, st);
     if (use_s) launch_gemm_rot<T>(SV.p, K, Cc.p, n, n, nb, K, SV2.p, K, 1.0, 0.0, st);
-    eps.resize(n);
-    CK(cudaMemcpyAsync(eps.data(), wv.p, n * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
     eps.resize(nb);
+    CK(cudaMemcpyAsync(eps.data(), wv.p, nb * sizeof(double), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
   }
 
   // Orthogonalise the m rows B against the nb current orbitals (rows 0..nb of V; in the S
@@ -1186,6 +1184,21 @@ template <typename T> struct EngineT : Engine {
     launch_scale_rows<T>(Bk, K, m, K, dtb.p, st);
     if (HBk) launch_scale_rows<T>(HBk, K, m, K, dtb.p, st);
     if (SBk) launch_scale_rows<T>(SBk, K, m, K, dtb.p, st);
+  }
+
+  // Replaces the search direction whose pivot failed last by the last one, V and its images alike, and
+  // counts it out of n; false when the failing row is one of the nb orbitals or the only direction.
+  bool drop_direction(int nb, int* n, int K) {
+    const int b = bad_pivot;
+    if (b < nb || b >= *n || *n - 1 <= nb) return false;
+    --*n;
+    if (b < *n) {
+      const size_t row = (size_t)K * sizeof(C), from = (size_t)*n * K, to = (size_t)b * K;
+      CK(cudaMemcpyAsync(V.p + to, V.p + from, row, cudaMemcpyDeviceToDevice, st));
+      CK(cudaMemcpyAsync(HV.p + to, HV.p + from, row, cudaMemcpyDeviceToDevice, st));
+      if (use_s) CK(cudaMemcpyAsync(SV.p + to, SV.p + from, row, cudaMemcpyDeviceToDevice, st));
+    }
+    return true;
   }
 
   // Block eigensolver (LOBPCG form of block Davidson): the search space of every iteration is
@@ -1310,14 +1323,23 @@ template <typename T> struct EngineT : Engine {
         rayleigh_ritz(q, n, nb, eps);
       } catch (Err& e) {
         if (e.st != FDE_ENOCONV) throw;
-        if (np == 0) break;  // dependent search directions: keep the current orbitals
-        n = nb + m;          // drop the previous directions and retry once
-        try {
-          rayleigh_ritz(q, n, nb, eps);
-        } catch (Err& e2) {
-          if (e2.st != FDE_ENOCONV) throw;
-          break;
+        // dependent search directions: the previous directions go first, then, one at a time, the
+        // residuals that depend on the others (residuals of a block that misses a band all point to
+        // it); with too many of them the solve ends with the current orbitals
+        bool again = true;
+        int left = m / 2;
+        if (np > 0) n = nb + m;
+        else again = drop_direction(nb, &n, K), --left;
+        while (again) {
+          try {
+            rayleigh_ritz(q, n, nb, eps);
+            break;
+          } catch (Err& e2) {
+            if (e2.st != FDE_ENOCONV) throw;
+            again = left-- > 0 && drop_direction(nb, &n, K);
+          }
         }
+        if (!again) break;
       }
       // update directions P = [W P] C[nb:n, :nb] (and their H- and S-images)
       launch_gemm_rot<T>(V.p + (size_t)nb * K, K, Cc.p + (size_t)nb * n, n, n - nb, nb, K, Pb.p, K, 1.0, 0.0, st);
@@ -2398,7 +2420,7 @@ fde_status fde_dense_eigh(fde_ctx* c, int n, const double* d_A, int nvec, double
     a.alloc((size_t)n * n);
     wk.alloc(fde::heev_work_doubles(n, nvec));
     CK(cudaMemcpyAsync(a.p, d_A, (size_t)n * n * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
-    fde::launch_heev(a.p, n, nvec, d_w, (double2*)d_V, wk.p, c->stream);
+    fde::launch_heev(a.p, n, nvec, n, d_w, (double2*)d_V, wk.p, c->stream);
     CK(cudaStreamSynchronize(c->stream));
     return FDE_OK;
   });

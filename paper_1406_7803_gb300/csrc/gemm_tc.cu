@@ -12,16 +12,20 @@
 // Precision.  TF32 keeps 10 mantissa bits.  Each operand is split x = hi + lo with hi = x
 // truncated to TF32 (exact) and lo = x - hi (exact in FP32); D += Ahi Bhi + Ahi Blo + Alo Bhi
 // (three MMAs per k-step) carries ~21 bits, the accuracy of the FP32 CUDA-core product.
-// passes = 1 keeps only Ahi Bhi.
+// passes = 1 keeps only Ahi Bhi.  The cross passes have an accumulator of their own: the tensor cores
+// truncate the sum at every addition, so adding 2^-11-sized terms to the large sum cost it two of
+// every three truncations -- the diagonal of an orthonormal block's Gram matrix came out 2e-5 low,
+// above the least pivot the eigensolver accepts, and near-dependent search directions failed its
+// Cholesky factorisation.
 //
 // Data flow per CTA (256 threads, one 128 x 64 complex output tile, one K-chunk):
-//   registers <- global (8-byte loads, one k-tile of 16 complex ahead) ; split, rotate and
+//   registers <- global (8-byte loads, two k-tiles of 16 complex ahead) ; split, rotate and
 //   store into the 128-byte-swizzled K-major shared-memory layout the MMA descriptors
 //   describe ; fence.proxy.async ; one elected thread issues 4 k-steps x passes MMAs of
 //   M = 128, N = 128, K = 8 and commits them to the stage's mbarrier ; one stage per CTA,
 //   two CTAs per SM.
-//   Epilogue: tcgen05.ld of the 128 x 128 FP32 accumulator, FP64 partial tile to global;
-//   k_gemm_hn_reduce (linalg.cu) sums the K-splits in a fixed order.
+//   Epilogue: tcgen05.ld of the 128 x 128 FP32 accumulators, FP32 partial tile to global;
+//   k_gemm_hn_reduce or k_gemm_hn_couple (linalg.cu) sums the K-splits in FP64 in a fixed order.
 // Every wait is bounded; on timeout the kernel sets ST_TIMEOUT, waits (bounded) for its
 // issued MMAs, frees its tensor memory and returns.
 #include <stdint.h>
@@ -40,13 +44,14 @@ constexpr int kTcThreads = 256;
 constexpr int kTcM = 128;      // output rows (A rows) per CTA
 constexpr int kTcN = 64;       // complex output columns (B rows) per CTA
 constexpr int kTcKc = 16;      // complex K per k-tile (32 floats = one 128-byte row)
+constexpr int kTcAcc = 2 * kTcN;  // tensor-memory columns of one accumulator
 constexpr int kTile = 16384;   // bytes of one 128-row x 128-byte operand tile
 constexpr int kStage = 4 * kTile;  // A hi, A lo, B hi, B lo
-// One shared-memory stage per CTA and two CTAs per SM: twice the warps issuing the next
-// k-tile's loads (the kernel is latency-bound) for the same buffering per SM.
+// One shared-memory stage per CTA and two CTAs per SM (66 KB and 256 tensor-memory columns each): the
+// kernel is bound by the latency of the next k-tiles' loads, so the SM needs many warps issuing them.
 constexpr int kStages = 1;
 constexpr int kCtasPerSm = 2;
-constexpr int kTmemCols = 128;
+constexpr int kTmemCols = 256;  // the hi hi sums and, 128 columns on, the sums of the two cross passes
 constexpr long long kSpin = kTcSpin;
 
 __device__ unsigned g_tc_status;
@@ -77,12 +82,15 @@ __device__ __forceinline__ void st2(uint32_t addr, float a, float b) {
   asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
 }
 
+constexpr int kDsPitch = kTcN + 1;  // complex values per row of the staged accumulator
+constexpr int kDsBytes = kTcM * kDsPitch * (int)sizeof(float2);
+
 constexpr int kAld = kTcM * kTcKc / kTcThreads;  // A elements per thread per k-tile (8)
 constexpr int kBld = kTcN * kTcKc / kTcThreads;  // B elements per thread per k-tile (4)
 
 __global__ void __launch_bounds__(kTcThreads, kCtasPerSm)
 k_gemm_hn_tc(const float2* __restrict__ A, int lda, const float2* __restrict__ B, int ldb, int m, int n, int K,
-             int kchunk, int passes, double2* __restrict__ part) {
+             int kchunk, int passes, float2* __restrict__ part) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bars[kStages];
   __shared__ uint32_t tmem_slot;
@@ -110,8 +118,8 @@ k_gemm_hn_tc(const float2* __restrict__ A, int lda, const float2* __restrict__ B
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
 
-  float2 ra[kAld], rb[kBld];
-  auto load = [&](int t) {
+  float2 ra[2][kAld], rb[2][kBld];  // two k-tiles of operands in flight
+  auto load = [&](int t, float2 (&ra)[kAld], float2 (&rb)[kBld]) {
     const int k0 = kb + t * kTcKc;
 #pragma unroll
     for (int q = 0; q < kAld; ++q) {
@@ -126,7 +134,7 @@ k_gemm_hn_tc(const float2* __restrict__ A, int lda, const float2* __restrict__ B
       rb[q] = (j < n && k < ke) ? __ldg(B + (size_t)j * ldb + k) : make_float2(0.f, 0.f);
     }
   };
-  auto store = [&](uint32_t st) {
+  auto store = [&](uint32_t st, const float2 (&ra)[kAld], const float2 (&rb)[kBld]) {
 #pragma unroll
     for (int q = 0; q < kAld; ++q) {
       const int idx = tid + kTcThreads * q, r = idx >> 4, c = 2 * (idx & 15);
@@ -149,8 +157,9 @@ k_gemm_hn_tc(const float2* __restrict__ A, int lda, const float2* __restrict__ B
   };
 
   int issued = 0;  // k-tiles whose MMAs were committed (meaningful in thread 0)
-  if (nt > 0) load(0);
-  for (int t = 0; t < nt; ++t) {
+  // one k-tile: wait for the stage, store the operands loaded two tiles ago, issue the MMAs, load the
+  // tile after next; false when the stage wait ran out
+  const auto step = [&](int t, float2 (&xa)[kAld], float2 (&xb)[kBld]) {
     const int s = t % kStages;
     const uint32_t st = base + (uint32_t)s * kStage;
     if (t >= kStages) {
@@ -158,9 +167,9 @@ k_gemm_hn_tc(const float2* __restrict__ A, int lda, const float2* __restrict__ B
       if (tid == 0 && !mbar_wait(su32(&bars[s]), (unsigned)(((t - kStages) / kStages) & 1), g_tc_stage_spin))
         abort_flag = 1;
       __syncthreads();
-      if (abort_flag) break;
+      if (abort_flag) return false;
     }
-    store(st);
+    store(st, xa, xb);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (tid == 0) {
@@ -172,14 +181,21 @@ k_gemm_hn_tc(const float2* __restrict__ A, int lda, const float2* __restrict__ B
         mma_tf32(tmem, ah, bh, (t > 0 || kk > 0) ? 1u : 0u);
         if (passes > 1) {
           const uint64_t al = sdesc(st + kTile + off), bl = sdesc(st + 3 * kTile + off);
-          mma_tf32(tmem, ah, bl, 1u);
-          mma_tf32(tmem, al, bh, 1u);
+          mma_tf32(tmem + kTcAcc, ah, bl, (t > 0 || kk > 0) ? 1u : 0u);
+          mma_tf32(tmem + kTcAcc, al, bh, 1u);
         }
       }
       mma_commit(su32(&bars[s]));
       ++issued;
     }
-    if (t + 1 < nt) load(t + 1);
+    if (t + 2 < nt) load(t + 2, xa, xb);
+    return true;
+  };
+  if (nt > 0) load(0, ra[0], rb[0]);
+  if (nt > 1) load(1, ra[1], rb[1]);
+  for (int t = 0; t < nt; t += 2) {
+    if (!step(t, ra[0], rb[0])) break;
+    if (t + 1 < nt && !step(t + 1, ra[1], rb[1])) break;
   }
 
   // wait for the last commit of each stage: every issued MMA has completed
@@ -196,31 +212,45 @@ k_gemm_hn_tc(const float2* __restrict__ A, int lda, const float2* __restrict__ B
   if (!ok && tid == 0) atomicOr(&g_tc_status, drained ? ST_TIMEOUT : (ST_TIMEOUT | ST_TMEM_HELD));
   tc_fence_after();
   if (ok) {
-    // warp w reads accumulator lanes 32 (w % 4) .. + 31 (its rows); warps 0-3 take the
-    // complex columns 0..31, warps 4-7 the columns 32..63
+    // Accumulator -> shared memory (the stage buffer is free: every MMA has completed) -> whole rows of
+    // the partial tile (a lane holds a row: written from there, each 8-byte value was a transaction of
+    // its own).  Warp w reads lanes 32 (w % 4) .. + 31; warps 0-3 take the complex columns 0..31,
+    // warps 4-7 the columns 32..63.  Ds[r][j] = (re, im), row pitch 65 complex.
+    float2* Ds = reinterpret_cast<float2*>(smem_raw + (base - su32(smem_raw)));
     const int q = warp & 3, h = warp >> 2;
-    const int r = 32 * q + lane, i = i0 + r;
+    const int r = 32 * q + lane;
     const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16);
-    double2* P = part + ((size_t)blockIdx.z * m + (size_t)(i < m ? i : 0)) * n;
+    if (i0 + 32 * q < m) {
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const int jc = 32 * h + 16 * half;
-      float re[16], im[16];
-      if (nt > 0) {
-        tmem_ld16(trow + (uint32_t)jc, re);
-        tmem_ld16(trow + (uint32_t)(kTcN + jc), im);
-      } else {
+      for (int half = 0; half < 2; ++half) {
+        const int jc = 32 * h + 16 * half;
+        float re[16], im[16];
+        if (nt > 0) {
+          tmem_ld16(trow + (uint32_t)jc, re);
+          tmem_ld16(trow + (uint32_t)(kTcN + jc), im);
+          if (passes > 1) {
+            float cr[16], ci[16];
+            tmem_ld16(trow + (uint32_t)(kTcAcc + jc), cr);
+            tmem_ld16(trow + (uint32_t)(kTcAcc + kTcN + jc), ci);
 #pragma unroll
-        for (int x = 0; x < 16; ++x) re[x] = im[x] = 0.f;
-      }
-      if (i < m) {
+            for (int x = 0; x < 16; ++x) {
+              re[x] += cr[x];
+              im[x] += ci[x];
+            }
+          }
+        } else {
 #pragma unroll
-        for (int x = 0; x < 16; ++x) {
-          const int j = j0 + jc + x;
-          if (j < n) P[j] = make_double2((double)re[x], (double)im[x]);
+          for (int x = 0; x < 16; ++x) re[x] = im[x] = 0.f;
         }
+#pragma unroll
+        for (int x = 0; x < 16; ++x) Ds[r * kDsPitch + jc + x] = make_float2(re[x], im[x]);
       }
     }
+    __syncthreads();
+    const int mr = min(kTcM, m - i0), nc = min(kTcN, n - j0);
+    float2* P = part + ((size_t)blockIdx.z * m + i0) * n + j0;
+    for (int rr = warp; rr < mr; rr += kTcThreads / 32)
+      for (int j = lane; j < nc; j += 32) P[(size_t)rr * n + j] = Ds[rr * kDsPitch + j];
   }
   tc_fence_before();
   __syncthreads();
@@ -439,21 +469,22 @@ k_gemm_rot_tc(const float2* __restrict__ X, int ldx, const double2* __restrict__
 
 }  // namespace
 
-// K-splits of the tensor-core product: about two resident CTAs per SM over the grid, at
-// least eight k-tiles per split.
+// K-splits of the tensor-core product: two CTAs for every SM over the grid, at least two k-tiles per
+// split.  (Eight k-tiles, the least before, left seven CTAs to run eight load latencies
+// in a row on the 898 plane waves of a small cell: 18 us for three bands.)
 int gemm_hn_tc_splits(int m, int n, int K) {
   const int tiles = ceil_div(m, kTcM) * ceil_div(n, kTcN);
   int s = ceil_div(2 * 152, tiles);
-  const int smax = std::max(1, ceil_div(K, 8 * kTcKc));
+  const int smax = std::max(1, ceil_div(K, 2 * kTcKc));
   return std::max(1, std::min(s, smax));
 }
 
-size_t gemm_hn_tc_smem() { return (size_t)kStages * kStage + 1024; }
+size_t gemm_hn_tc_smem() { return (size_t)std::max(kStages * kStage, kDsBytes) + 1024; }
 
 // Partial tiles of C = A^H B into part[nsplit][m][n]; returns the number of splits (0 if the
 // kernel could not be configured; nothing is launched then).
 int launch_gemm_hn_tc(const float2* A, int lda, const float2* B, int ldb, int m, int n, int K, int passes,
-                      double2* part, cudaStream_t st) {
+                      float2* part, cudaStream_t st) {
   static int attr = 0;  // 1 configured, -1 failed
   if (attr == 0)
     attr = cudaFuncSetAttribute(k_gemm_hn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,

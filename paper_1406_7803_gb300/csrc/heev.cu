@@ -328,8 +328,8 @@ size_t heev_work_doubles(int n, int nvec) {
 }
 
 // The cluster-distributed solver (dense.cu) when n fits it, else this one-CTA kernel.
-void launch_heev(double2* A, int n, int nvec, double* w, double2* V, double* work, cudaStream_t st) {
-  if (launch_heev_cluster(A, n, nvec, w, V, work, st)) return;
+void launch_heev(double2* A, int n, int nvec, int nval, double* w, double2* V, double* work, cudaStream_t st) {
+  if (launch_heev_cluster(A, n, nvec, nval, w, V, work, st)) return;
   count_launches(1);
   k_heev<<<1, kHeevThreads, 0, st>>>(A, n, nvec, w, V, work);
 }

@@ -106,10 +106,10 @@ size_t gemm_hn_work(int m, int n, int K);
 void set_gemm_hn_path(int path);
 int gemm_hn_path();
 // The tensor-core kernel itself (gemm_tc.cu): partial tiles into part[nsplit][m][n];
-// returns nsplit, or 0 when the kernel could not be configured (nothing launched).
+// (FP32 values); returns nsplit, or 0 when the kernel could not be configured (nothing launched).
 int gemm_hn_tc_splits(int m, int n, int K);
 int launch_gemm_hn_tc(const float2* A, int lda, const float2* B, int ldb, int m, int n, int K, int passes,
-                      double2* part, cudaStream_t st);
+                      float2* part, cudaStream_t st);
 // Y = alpha U^T-combination of the rows of X + beta Y on the tensor cores (gemm_tc.cu), with
 // the same passes as launch_gemm_hn_tc; false when the kernel could not be configured.
 bool launch_gemm_rot_tc(const float2* X, int ldx, const double2* U, int ldu, int m, int n, int K, float2* Y,
@@ -119,7 +119,7 @@ unsigned gemm_tc_take_status(cudaStream_t st);
 bool set_tc_stage_spin(long long polls);
 void disable_tensor_cores();
 bool tensor_cores_disabled();
-void launch_gemm_hn_reduce(const double2* part, int nsplit, int m, int n, double2* C, int ldc, cudaStream_t st);
+void launch_gemm_hn_reduce(const float2* part, int nsplit, int m, int n, double2* C, int ldc, cudaStream_t st);
 template <typename T>
 void launch_gemm_hn(const cplx<T>* A, int lda, const cplx<T>* B, int ldb, int m, int n, int K,
                     double2* C, int ldc, double2* work, cudaStream_t st);
@@ -133,29 +133,49 @@ template <typename T>
 void launch_gemm_rot(const cplx<T>* X, int ldx, const double2* U, int ldu, int m, int n, int K,
                      cplx<T>* Y, int ldy, double alpha, double beta, cudaStream_t st, bool tensor = false);
 
+template <>
+void launch_gemm_hn<float>(const float2* A, int lda, const float2* B, int ldb, int m, int n, int K, double2* C, int ldc,
+                           double2* work, cudaStream_t st);
+template <>
+void launch_gemm_hn<double>(const double2* A, int lda, const double2* B, int ldb, int m, int n, int K, double2* C,
+                            int ldc, double2* work, cudaStream_t st);
+template <>
+void launch_gemm_rot<float>(const float2* X, int ldx, const double2* U, int ldu, int m, int n, int K, float2* Y, int ldy,
+                            double alpha, double beta, cudaStream_t st, bool tensor);
+template <>
+void launch_gemm_rot<double>(const double2* X, int ldx, const double2* U, int ldu, int m, int n, int K, double2* Y,
+                             int ldy, double alpha, double beta, cudaStream_t st, bool tensor);
+
 // Per-atom block of the projector coupling (np x np, row-major, np <= 8).
 struct KbBlock {
   double d[64];
   int np;
 };
-// Q[a np + i][b] = sum_j D[i][j] P[a np + j][b] for natoms atoms and nb columns (FP64 complex,
-// leading dimension nb).
-void launch_kb_couple(const double2* P, const KbBlock& D, int natoms, int nb, double2* Q, cudaStream_t st);
-// The same with its own np x np block for every atom: D [natoms][np][np] (device).
-void launch_kb_couple_atoms(const double2* P, const double* D, int np, int natoms, int nb, double2* Q, cudaStream_t st);
+// Q[a np + i][b] = sum_j D[i][j] <beta_{a np + j}|psi_b> for natoms atoms and nb bands (FP64 complex,
+// leading dimension nb): the block D for every atom, or, with Datom [natoms][np][np] (device), each
+// atom's own.  beta [natoms np][ld], psi [nb][ld], rows of length K; work: gemm_hn_work double2.
+template <typename T>
+void launch_project_couple(const cplx<T>* beta, const cplx<T>* psi, int ld, int K, const KbBlock& D, const double* Datom,
+                           int natoms, int nb, double2* Q, double2* work, cudaStream_t st);
+template <>
+void launch_project_couple<float>(const float2* beta, const float2* psi, int ld, int K, const KbBlock& D,
+                                  const double* Datom, int natoms, int nb, double2* Q, double2* work, cudaStream_t st);
+template <>
+void launch_project_couple<double>(const double2* beta, const double2* psi, int ld, int K, const KbBlock& D,
+                                   const double* Datom, int natoms, int nb, double2* Q, double2* work, cudaStream_t st);
 
 // Cholesky S = L L^H (n x n, FP64 complex, lower, in place into L) and Linv = L^{-1};
-// sets status bit ST_CHOLESKY on a pivot not above rel_pivot S_jj (the squared norm of a
+// sets bit ST_CHOLESKY of status[0] and leaves the column in status[1] on a pivot not above rel_pivot S_jj (the squared norm of a
 // vector's part orthogonal to the earlier ones, relative to its own squared norm: below the
 // rounding level of the vectors' precision they are numerically dependent).
 void launch_cholesky_inv(const double2* S, int n, double2* L, double2* Linv, unsigned* status, double rel_pivot,
                          cudaStream_t st);
 
-// Hermitian eigenproblem (FP64): A (n x n) -> eigenvalues w[n] ascending and the eigenvectors
-// of the lowest nvec eigenvalues in the columns of V (other columns zero), by
+// Hermitian eigenproblem (FP64): A (n x n) -> the lowest nval eigenvalues w[0 .. nval) ascending (w holds
+// n) and the eigenvectors of the lowest nvec eigenvalues in the columns of V (other columns zero), by
 // tridiagonalisation, bisection and inverse iteration (dense.cu, heev.cu).
 size_t heev_work_doubles(int n, int nvec);
-void launch_heev(double2* A, int n, int nvec, double* w, double2* V, double* work, cudaStream_t st);
+void launch_heev(double2* A, int n, int nvec, int nval, double* w, double2* V, double* work, cudaStream_t st);
 
 // Row-wise helpers on [nb][K] blocks.
 template <typename T>
