@@ -406,27 +406,31 @@ template <typename T> struct EngineT : Engine {
     all.insert(all.end(), ci1.begin(), ci1.end());
     all.insert(all.end(), ci2.begin(), ci2.end());
     all.insert(all.end(), rows.begin(), rows.end());
-    q.cols.alloc(all.size());
-    CK(cudaMemcpy(q.cols.p, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice));
-    q.sp.npw = q.npw;
-    q.sp.ncol = ncol;
-    q.sp.ldc = (ncol + 15) / 16 * 16;  // 128-byte scratch rows
-    q.sp.nrow = (int)rows.size();
     int m2lo = q.miller[1], m2hi = q.miller[1];
     for (int p = 0; p < q.npw; ++p) {
       m2lo = std::min(m2lo, q.miller[3 * p + 1]);
       m2hi = std::max(m2hi, q.miller[3 * p + 1]);
     }
     const int m1lo = q.miller[0], m1hi = q.miller[3 * (q.npw - 1)];
+    const int span2 = m2hi - m2lo + 1, pos0 = (int)all.size();
+    for (int c = 0; c < ncol; ++c)
+      all.push_back((q.miller[3 * cs[c]] - m1lo) * (span2 | 1) + q.miller[3 * cs[c] + 1] - m2lo);
+    q.cols.alloc(all.size());
+    CK(cudaMemcpy(q.cols.p, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice));
+    q.sp.npw = q.npw;
+    q.sp.ncol = ncol;
+    q.sp.ldc = (ncol + 15) / 16 * 16;  // 128-byte scratch rows
+    q.sp.nrow = (int)rows.size();
     q.sp.lo1 = ((m1lo % grid[0]) + grid[0]) % grid[0];
     q.sp.span1 = m1hi - m1lo + 1;
     q.sp.lo2 = ((m2lo % grid[1]) + grid[1]) % grid[1];
-    q.sp.span2 = m2hi - m2lo + 1;
+    q.sp.span2 = span2;
     q.sp.col_start = q.cols.p;
     q.sp.col_m3lo = q.cols.p + (ncol + 1);
     q.sp.col_i1 = q.cols.p + (2 * ncol + 1);
     q.sp.col_i2 = q.cols.p + (3 * ncol + 1);
     q.sp.row_i1 = q.cols.p + (4 * ncol + 1);
+    q.sp.col_pos = q.cols.p + pos0;
     std::vector<T> kt(q.npw);
     for (int p = 0; p < q.npw; ++p) kt[p] = (T)q.kin[p];
     q.kin_d.alloc(q.npw);

@@ -174,6 +174,33 @@ __host__ __device__ constexpr Split split_of(int n) {
 }
 inline bool split_side_ok(int n) { return n <= 160 && split_of(n).a > 0; }
 
+// Plan of a plane side N = R1 R2 (R1 >= R2).  Where N has coprime factors the two steps run on the
+// prime-factor indices -- input n = (R2 r + R1 j) mod N, output k with k = q mod R1, k = p mod R2 -- and
+// there are no twiddles between them: W_N^{nk} = W_R1^{rq} W_R2^{jp}.  That saves 14 % of the
+// arithmetic of 72 = 9 x 8 and the loads of its 56 twiddles.  Other sides take the Cooley-Tukey
+// indices n = j + R2 r, k = q + R1 p.
+template <int R1_, int R2_> struct SidePlan {
+  static constexpr int R1 = R1_, R2 = R2_, N = R1 * R2;
+  static constexpr int gcd(int a, int b) { return b ? gcd(b, a % b) : a; }
+  static constexpr bool kCoprime = gcd(R1, R2) == 1;
+  // unit of q and of p in k (prime-factor form)
+  static constexpr int E1 = kCoprime ? crt_index(R1, R2, 1 % R1, 0) : 0, E2 = kCoprime ? crt_index(R1, R2, 0, 1 % R2) : 0;
+  // input index of element r of item j is in0(j) + R2 r, modulo N (each term below N)
+  __host__ __device__ static constexpr int in0(int j) { return kCoprime ? R1 * j : j; }
+  // output index of element p of item q is out0(q) + out(p), modulo N (each term below N)
+  __host__ __device__ static constexpr int out0(int q) { return kCoprime ? q * E1 % N : q; }
+  __host__ __device__ static constexpr int out(int p) { return kCoprime ? p * E2 % N : R1 * p; }
+  __host__ __device__ static constexpr int wrap(int k) { return k >= N ? k - N : k; }
+  __host__ __device__ static constexpr int output(int q, int p) {
+    return kCoprime ? wrap(out0(q) + out(p)) : q + R1 * p;  // the latter never wraps
+  }
+};
+// Sides as X(N, R1, R2).
+#define FDE_PLANE_SIDES(X)                                                                                       \
+  X(24, 8, 3) X(30, 6, 5) X(32, 8, 4) X(36, 9, 4) X(40, 8, 5) X(45, 9, 5) X(48, 16, 3) X(50, 10, 5) X(54, 9, 6)   \
+  X(60, 12, 5) X(64, 8, 8) X(72, 9, 8) X(75, 15, 5) X(80, 16, 5) X(90, 10, 9) X(96, 12, 8) X(100, 10, 10)         \
+  X(108, 12, 9) X(120, 15, 8) X(128, 16, 8) X(135, 15, 9) X(144, 16, 9) X(150, 15, 10) X(160, 16, 10)
+
 __host__ __device__ constexpr int round_up(int n, int m) { return (n + m - 1) / m * m; }
 
 // x * W^e or x * conj(W^e) from the table tw[e] = exp(-2 pi i e / N).

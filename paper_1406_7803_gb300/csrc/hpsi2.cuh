@@ -182,137 +182,175 @@ struct PlaneDims {
   int W;          // X pitch of the column stage (odd)
 };
 
-template <typename T, int R1, int R2>
+// Offset of the span's first index from element 0 of item j: element r sits at d = wrap(base + R2 r) of
+// the span, inside it when d < span.
+template <typename Plan> __device__ __forceinline__ int span_base(int j, int lo) {
+  const int b = Plan::in0(j) - lo;
+  return b < 0 ? b + Plan::N : b;
+}
+
+template <typename T, typename Plan>
 __device__ __forceinline__ void plane_y_inv(cplx<T>* P, const cplx<T>* X, const PlaneDims& D, int pitch, int nt,
                                             const cplx<T>* __restrict__ tw) {
   using C = cplx<T>;
-  constexpr int N = R1 * R2;
+  constexpr int R1 = Plan::R1, R2 = Plan::R2;
   const unsigned inv = (1u << 20) / (unsigned)D.n1s + 1u;  // w / n1s = w inv >> 20 for w < 2^20 / n1s
   for (int w = threadIdx.x; w < D.n1s * R2; w += nt) {
     const int j = (int)(((unsigned)w * inv) >> 20), r = w - j * D.n1s;
+    const int base = span_base<Plan>(j, D.lo2);
+    const C* x = X + r * D.W;
     C v[R1];
 #pragma unroll
     for (int q = 0; q < R1; ++q) {
-      const int d = run_offset(j + q * R2, D.lo2, N);
-      v[q] = d < D.n2s ? X[r * D.W + d] : mk<T>(0, 0);
+      const int d = Plan::wrap(base + q * R2);
+      v[q] = d < D.n2s ? x[d] : mk<T>(0, 0);
     }
     dft_r<R1>(v, +1);
+    C* o = P + r * pitch;
+    const int oj = Plan::out(j);
 #pragma unroll
-    for (int q = 0; q < R1; ++q) P[r * pitch + q + R1 * j] = v[q];
+    for (int q = 0; q < R1; ++q) o[Plan::wrap(Plan::out0(q) + oj)] = v[q];
   }
   __syncthreads();
   for (int w = threadIdx.x; w < D.n1s * R1; w += nt) {
     const int q = (int)(((unsigned)w * inv) >> 20), r = w - q * D.n1s;
+    C* o = P + r * pitch;
     C v[R2];
 #pragma unroll
     for (int j = 0; j < R2; ++j) {
-      v[j] = P[r * pitch + q + R1 * j];
-      if (j) v[j] = twist(v[j], tw[j * q], +1);
+      v[j] = o[Plan::output(q, j)];
+      if (!Plan::kCoprime && j) v[j] = twist(v[j], tw[j * q], +1);
     }
     dft_r<R2>(v, +1);
 #pragma unroll
-    for (int p = 0; p < R2; ++p) P[r * pitch + q + R1 * p] = v[p];
+    for (int p = 0; p < R2; ++p) o[Plan::output(q, p)] = v[p];
   }
 }
 
-template <typename T, int R1, int R2>
+template <typename T, typename Plan>
 __device__ __forceinline__ void plane_y_fwd(cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, int nt,
                                             const cplx<T>* __restrict__ tw) {
   using C = cplx<T>;
-  constexpr int N = R1 * R2;
+  constexpr int R1 = Plan::R1, R2 = Plan::R2;
   const unsigned inv = (1u << 20) / (unsigned)D.n1s + 1u;
   for (int w = threadIdx.x; w < D.n1s * R1; w += nt) {
     const int q = (int)(((unsigned)w * inv) >> 20), r = w - q * D.n1s;
+    C* o = P + r * pitch;
     C v[R2];
 #pragma unroll
-    for (int p = 0; p < R2; ++p) v[p] = P[r * pitch + q + R1 * p];
+    for (int p = 0; p < R2; ++p) v[p] = o[Plan::output(q, p)];
     dft_r<R2>(v, -1);
 #pragma unroll
-    for (int j = 0; j < R2; ++j) P[r * pitch + q + R1 * j] = j ? twist(v[j], tw[j * q], -1) : v[j];
+    for (int j = 0; j < R2; ++j) o[Plan::output(q, j)] = (!Plan::kCoprime && j) ? twist(v[j], tw[j * q], -1) : v[j];
   }
   __syncthreads();
   for (int w = threadIdx.x; w < D.n1s * R2; w += nt) {
     const int j = (int)(((unsigned)w * inv) >> 20), r = w - j * D.n1s;
+    const C* o = P + r * pitch;
+    const int oj = Plan::out(j);
     C v[R1];
 #pragma unroll
-    for (int q = 0; q < R1; ++q) v[q] = P[r * pitch + q + R1 * j];
+    for (int q = 0; q < R1; ++q) v[q] = o[Plan::wrap(Plan::out0(q) + oj)];
     dft_r<R1>(v, -1);
+    const int base = span_base<Plan>(j, D.lo2);
+    C* x = X + r * D.W;
 #pragma unroll
     for (int q = 0; q < R1; ++q) {
-      const int d = run_offset(j + q * R2, D.lo2, N);
-      if (d < D.n2s) X[r * D.W + d] = v[q];
+      const int d = Plan::wrap(base + q * R2);
+      if (d < D.n2s) x[d] = v[q];
     }
   }
 }
 
-// Step 1 of the inverse x transforms of the columns c0 .. c0 + nc - 1: rows of P into X[slot][c],
-// slot = j R1 + q.
-template <typename T, int R1, int R2>
-__device__ __forceinline__ void plane_x_in(const cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, int c0, int lb,
-                                           int nc, int nt) {
-  using C = cplx<T>;
-  constexpr int N = R1 * R2;
-  for (int w = threadIdx.x; w < R2 * lb; w += nt) {
-    const int j = w / lb, c = w - j * lb;
-    if (c >= nc) continue;
-    C v[R1];
+// The x steps of all columns, lb at a time (lb max(R1, R2) <= nt: one item a thread and step).  What a
+// thread's item needs -- the rows of its step-1 inputs, the potential's rows of its outputs, its
+// twiddles -- depends on the item alone, so it is found once and kept over the batches.
+// Step 1: rows of P into X[slot][c], slot = j R1 + q.  Step 2, the potential and the forward's first step:
+// X in place.  The forward's second step: X back into the rows of P.
+template <typename T, typename Plan>
+struct XItem {
+  int row[Plan::R1];  // step 1: offset in P of the item's element r, or -1 outside the span
+  __device__ __forceinline__ void rows(const PlaneDims& D, int j, int c, int pitch) {
+    const int base = span_base<Plan>(j, D.lo1);
 #pragma unroll
-    for (int q = 0; q < R1; ++q) {
-      const int d = run_offset(j + q * R2, D.lo1, N);
-      v[q] = d < D.n1s ? P[d * pitch + c0 + c] : mk<T>(0, 0);
+    for (int q = 0; q < Plan::R1; ++q) {
+      const int d = Plan::wrap(base + q * Plan::R2);
+      row[q] = d < D.n1s ? d * pitch + c : -1;
     }
-    dft_r<R1>(v, +1);
-#pragma unroll
-    for (int q = 0; q < R1; ++q) X[(j * R1 + q) * lb + c] = v[q];
   }
-}
-// Step 2 of the inverse, the potential, step 1 of the forward: item q of column c, in place.
-template <typename T, int R1, int R2>
-__device__ __forceinline__ void plane_x_mul(cplx<T>* X, int c0, int lb, int nc, int nt, const cplx<T>* __restrict__ tw,
-                                            const T* __restrict__ vp, int n2) {
+};
+template <typename T, typename Plan>
+__device__ __forceinline__ void plane_x_in(const cplx<T>* P, cplx<T>* X, const XItem<T, Plan>& I, int j, int c, int c0,
+                                           int lb) {
   using C = cplx<T>;
-  for (int w = threadIdx.x; w < R1 * lb; w += nt) {
-    const int q = w / lb, c = w - q * lb;
-    if (c >= nc) continue;
-    C v[R2], t[R2];
+  constexpr int R1 = Plan::R1;
+  C v[R1];
 #pragma unroll
-    for (int j = 0; j < R2; ++j) {
-      v[j] = X[(j * R1 + q) * lb + c];
-      if (j) {
-        t[j] = tw[j * q];
-        v[j] = twist(v[j], t[j], +1);
+  for (int q = 0; q < R1; ++q) v[q] = I.row[q] >= 0 ? P[I.row[q] + c0] : mk<T>(0, 0);
+  dft_r<R1>(v, +1);
+#pragma unroll
+  for (int q = 0; q < R1; ++q) X[(j * R1 + q) * lb + c] = v[q];
+}
+template <typename T, typename Plan>
+__device__ __forceinline__ void plane_x_out(cplx<T>* P, const cplx<T>* X, const XItem<T, Plan>& I, int j, int c, int c0,
+                                            int lb) {
+  using C = cplx<T>;
+  constexpr int R1 = Plan::R1;
+  C v[R1];
+#pragma unroll
+  for (int q = 0; q < R1; ++q) v[q] = X[(j * R1 + q) * lb + c];
+  dft_r<R1>(v, -1);
+#pragma unroll
+  for (int q = 0; q < R1; ++q)
+    if (I.row[q] >= 0) P[I.row[q] + c0] = v[q];
+}
+template <typename T, typename Plan>
+__device__ __forceinline__ void plane_x_all(cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, int n2, int lb,
+                                            const cplx<T>* __restrict__ tw, const T* __restrict__ vp) {
+  using C = cplx<T>;
+  constexpr int R1 = Plan::R1, R2 = Plan::R2;
+  const int tid = threadIdx.x, j = tid / lb, c = tid - j * lb;  // the same pair serves both item kinds
+  const bool in1 = j < R2, in2 = j < R1;
+  XItem<T, Plan> I;
+  if (in1) I.rows(D, j, c, pitch);
+  int vo[R2];
+  C t[Plan::kCoprime ? 1 : R2];
+#pragma unroll
+  for (int p = 0; p < R2; ++p) {
+    vo[p] = Plan::output(j, p) * n2 + c;
+    if constexpr (!Plan::kCoprime)
+      if (p && in2) t[p] = tw[p * j];
+  }
+#pragma unroll 1
+  for (int c0 = 0; c0 < n2; c0 += lb) {
+    const bool have = c < n2 - c0;
+    if (in1 && have) plane_x_in<T, Plan>(P, X, I, j, c, c0, lb);
+    __syncthreads();
+    if (in2 && have) {
+      C v[R2];
+#pragma unroll
+      for (int p = 0; p < R2; ++p) {
+        v[p] = X[(p * R1 + j) * lb + c];
+        if constexpr (!Plan::kCoprime)
+          if (p) v[p] = twist(v[p], t[p], +1);
+      }
+      dft_r<R2>(v, +1);
+#pragma unroll
+      for (int p = 0; p < R2; ++p) {
+        const T s = vp[vo[p] + c0];
+        v[p].x *= s;
+        v[p].y *= s;
+      }
+      dft_r<R2>(v, -1);
+#pragma unroll
+      for (int p = 0; p < R2; ++p) {
+        if constexpr (!Plan::kCoprime)
+          if (p) v[p] = cmul(v[p], t[p]);
+        X[(p * R1 + j) * lb + c] = v[p];
       }
     }
-    dft_r<R2>(v, +1);
-#pragma unroll
-    for (int p = 0; p < R2; ++p) {
-      const T s = vp[(q + R1 * p) * n2 + c0 + c];
-      v[p].x *= s;
-      v[p].y *= s;
-    }
-    dft_r<R2>(v, -1);
-#pragma unroll
-    for (int j = 0; j < R2; ++j) X[(j * R1 + q) * lb + c] = j ? cmul(v[j], t[j]) : v[j];
-  }
-}
-// Step 2 of the forward x transforms: X back into the rows of P.
-template <typename T, int R1, int R2>
-__device__ __forceinline__ void plane_x_out(cplx<T>* P, const cplx<T>* X, const PlaneDims& D, int pitch, int c0, int lb,
-                                            int nc, int nt) {
-  using C = cplx<T>;
-  constexpr int N = R1 * R2;
-  for (int w = threadIdx.x; w < R2 * lb; w += nt) {
-    const int j = w / lb, c = w - j * lb;
-    if (c >= nc) continue;
-    C v[R1];
-#pragma unroll
-    for (int q = 0; q < R1; ++q) v[q] = X[(j * R1 + q) * lb + c];
-    dft_r<R1>(v, -1);
-#pragma unroll
-    for (int q = 0; q < R1; ++q) {
-      const int d = run_offset(j + q * R2, D.lo1, N);
-      if (d < D.n1s) P[d * pitch + c0 + c] = v[q];
-    }
+    __syncthreads();
+    if (in1 && have) plane_x_out<T, Plan>(P, X, I, j, c, c0, lb);
   }
 }
 
@@ -323,17 +361,14 @@ __device__ __forceinline__ PlaneDims plane_dims(const SphereDev& sp) {
 // Sphere columns of one plane into X[row][m2 - lo2] (slots without a column are zero), and back.
 template <typename T>
 __device__ __forceinline__ void plane_columns_in(cplx<T>* X, const cplx<T>* __restrict__ S, const SphereDev& sp,
-                                                 const PlaneDims& D, int n1, int n2, int nt) {
+                                                 const PlaneDims& D, int nt) {
   for (int i = threadIdx.x; i < D.n1s * D.W; i += nt) X[i] = mk<T>(0, 0);
   __syncthreads();
-  for (int c = threadIdx.x; c < sp.ncol; c += nt)
-    X[run_offset(sp.col_i1[c], D.lo1, n1) * D.W + run_offset(sp.col_i2[c], D.lo2, n2)] = S[c];
+  for (int c = threadIdx.x; c < sp.ncol; c += nt) X[sp.col_pos[c]] = S[c];
 }
 template <typename T>
-__device__ __forceinline__ void plane_columns_out(const cplx<T>* X, cplx<T>* __restrict__ S, const SphereDev& sp,
-                                                  const PlaneDims& D, int n1, int n2, int nt) {
-  for (int c = threadIdx.x; c < sp.ncol; c += nt)
-    S[c] = X[run_offset(sp.col_i1[c], D.lo1, n1) * D.W + run_offset(sp.col_i2[c], D.lo2, n2)];
+__device__ __forceinline__ void plane_columns_out(const cplx<T>* X, cplx<T>* __restrict__ S, const SphereDev& sp, int nt) {
+  for (int c = threadIdx.x; c < sp.ncol; c += nt) S[c] = X[sp.col_pos[c]];
 }
 
 // Columns a batch of the x transforms takes: as many as let about NT threads hold one butterfly
@@ -346,13 +381,12 @@ __host__ __device__ constexpr int plane_batch(int n2, int rmax, int nt) {
   return (n2 + nb - 1) / nb;
 }
 
-template <typename T, int R1X, int R2X, int R1Y, int R2Y, int NT, int MINB>
+template <typename T, typename PX, typename PY, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
 k_plane_pass(const __grid_constant__ HpsiBatch<T> B, int n3, const cplx<T>* __restrict__ tw1,
              const cplx<T>* __restrict__ tw2, int psize) {
   using C = cplx<T>;
-  constexpr int N1 = R1X * R2X, N2 = R1Y * R2Y, PITCH = N2 | 1;
-  constexpr int LB = plane_batch(N2, R1X > R2X ? R1X : R2X, NT);
+  constexpr int PITCH = PY::N | 1, LB = plane_batch(PY::N, PX::R1, NT);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* P = reinterpret_cast<C*>(smem_raw);
   C* X = P + psize;
@@ -361,25 +395,16 @@ k_plane_pass(const __grid_constant__ HpsiBatch<T> B, int n3, const cplx<T>* __re
   const int local = blockIdx.x - I.pstart;
   const int b = local / n3, i3 = local - b * n3;
   C* S = I.scratch + ((size_t)b * n3 + i3) * sp.ldc;
-  const T* vp = I.vplane + (size_t)i3 * N1 * N2;
   const PlaneDims D = plane_dims<T>(sp);
-  plane_columns_in<T>(X, S, sp, D, N1, N2, NT);
+  plane_columns_in<T>(X, S, sp, D, NT);
   __syncthreads();
-  plane_y_inv<T, R1Y, R2Y>(P, X, D, PITCH, NT, tw2);
+  plane_y_inv<T, PY>(P, X, D, PITCH, NT, tw2);
   __syncthreads();
-#pragma unroll 1
-  for (int c0 = 0; c0 < N2; c0 += LB) {
-    const int nc = N2 % LB == 0 ? LB : min(LB, N2 - c0);
-    plane_x_in<T, R1X, R2X>(P, X, D, PITCH, c0, LB, nc, NT);
-    __syncthreads();
-    plane_x_mul<T, R1X, R2X>(X, c0, LB, nc, NT, tw1, vp, N2);
-    __syncthreads();
-    plane_x_out<T, R1X, R2X>(P, X, D, PITCH, c0, LB, nc, NT);
-  }
+  plane_x_all<T, PX>(P, X, D, PITCH, PY::N, LB, tw1, I.vplane + (size_t)i3 * PX::N * PY::N);
   __syncthreads();
-  plane_y_fwd<T, R1Y, R2Y>(P, X, D, PITCH, NT, tw2);
+  plane_y_fwd<T, PY>(P, X, D, PITCH, NT, tw2);
   __syncthreads();
-  plane_columns_out<T>(X, S, sp, D, N1, N2, NT);
+  plane_columns_out<T>(X, S, sp, NT);
 }
 
 // ---- band densities --------------------------------------------------------------------------------
@@ -407,61 +432,64 @@ __device__ __forceinline__ float2 rho_add(float2 a, float2 b) {
 __device__ __forceinline__ double rho_weight(double w, double) { return w; }
 __device__ __forceinline__ dd rho_weight(double w, float) { return dd_from_double(w); }
 
-template <typename T, int R1, int R2>
-__device__ __forceinline__ void plane_x_rho(const cplx<T>* X, int c0, int lb, int nc, int nt,
+template <typename T, typename Plan>
+__device__ __forceinline__ void plane_x_rho(const cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, int n2, int lb,
                                             const cplx<T>* __restrict__ tw, double weight, bool first,
-                                            typename RhoAcc<T>::t* rho, int n2) {
+                                            typename RhoAcc<T>::t* rho) {
   using C = cplx<T>;
+  constexpr int R1 = Plan::R1, R2 = Plan::R2;
   const auto wt = rho_weight(weight, T(0));
-  for (int w = threadIdx.x; w < R1 * lb; w += nt) {
-    const int q = w / lb, c = w - q * lb;
-    if (c >= nc) continue;
-    C v[R2];
+  const int tid = threadIdx.x, j = tid / lb, c = tid - j * lb;
+  const bool in1 = j < R2, in2 = j < R1;
+  XItem<T, Plan> I;
+  if (in1) I.rows(D, j, c, pitch);
+#pragma unroll 1
+  for (int c0 = 0; c0 < n2; c0 += lb) {
+    const bool have = c < n2 - c0;
+    if (in1 && have) plane_x_in<T, Plan>(P, X, I, j, c, c0, lb);
+    __syncthreads();
+    if (in2 && have) {
+      C v[R2];
 #pragma unroll
-    for (int j = 0; j < R2; ++j) {
-      v[j] = X[(j * R1 + q) * lb + c];
-      if (j) v[j] = twist(v[j], tw[j * q], +1);
-    }
-    dft_r<R2>(v, +1);
+      for (int p = 0; p < R2; ++p) {
+        v[p] = X[(p * R1 + j) * lb + c];
+        if constexpr (!Plan::kCoprime)
+          if (p) v[p] = twist(v[p], tw[p * j], +1);
+      }
+      dft_r<R2>(v, +1);
 #pragma unroll
-    for (int p = 0; p < R2; ++p) {
-      auto* o = rho + (q + R1 * p) * n2 + c0 + c;
-      const auto d = rho_term(wt, v[p]);
-      *o = first ? d : rho_add(*o, d);
+      for (int p = 0; p < R2; ++p) {
+        auto* o = rho + Plan::output(j, p) * n2 + c0 + c;
+        const auto d = rho_term(wt, v[p]);
+        *o = first ? d : rho_add(*o, d);
+      }
     }
+    __syncthreads();
   }
 }
 
 // Bands [nb g / groups, nb (g + 1) / groups) of group g.
-template <typename T, int R1X, int R2X, int R1Y, int R2Y, int NT, int MINB>
+template <typename T, typename PX, typename PY, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
 k_plane_rho(const cplx<T>* __restrict__ scratch, SphereDev sp, int nb, const double* __restrict__ weight,
             typename RhoAcc<T>::t* __restrict__ part, int n3, const cplx<T>* __restrict__ tw1,
             const cplx<T>* __restrict__ tw2, int psize) {
   using C = cplx<T>;
-  constexpr int N1 = R1X * R2X, N2 = R1Y * R2Y, PITCH = N2 | 1;
-  constexpr int LB = plane_batch(N2, R1X > R2X ? R1X : R2X, NT);
+  constexpr int PITCH = PY::N | 1, LB = plane_batch(PY::N, PX::R1, NT);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* P = reinterpret_cast<C*>(smem_raw);
   C* X = P + psize;
   const int i3 = blockIdx.x, g = blockIdx.y;
   const int b0 = (int)((long long)nb * g / gridDim.y), b1 = (int)((long long)nb * (g + 1) / gridDim.y);
   const PlaneDims D = plane_dims<T>(sp);
-  auto* rho = part + ((size_t)g * n3 + i3) * N1 * N2;
+  auto* rho = part + ((size_t)g * n3 + i3) * PX::N * PY::N;
 #pragma unroll 1
   for (int b = b0; b < b1; ++b) {
-    plane_columns_in<T>(X, scratch + ((size_t)b * n3 + i3) * sp.ldc, sp, D, N1, N2, NT);
+    plane_columns_in<T>(X, scratch + ((size_t)b * n3 + i3) * sp.ldc, sp, D, NT);
     __syncthreads();
-    plane_y_inv<T, R1Y, R2Y>(P, X, D, PITCH, NT, tw2);
+    plane_y_inv<T, PY>(P, X, D, PITCH, NT, tw2);
     __syncthreads();
-#pragma unroll 1
-    for (int c0 = 0; c0 < N2; c0 += LB) {
-      const int nc = N2 % LB == 0 ? LB : min(LB, N2 - c0);
-      plane_x_in<T, R1X, R2X>(P, X, D, PITCH, c0, LB, nc, NT);
-      __syncthreads();
-      plane_x_rho<T, R1X, R2X>(X, c0, LB, nc, NT, tw1, weight[b], b == b0, rho, N2);
-      __syncthreads();
-    }
+    plane_x_rho<T, PX>(P, X, D, PITCH, PY::N, LB, tw1, weight[b], b == b0, rho);
   }
 }
 

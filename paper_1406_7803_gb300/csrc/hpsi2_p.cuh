@@ -6,32 +6,40 @@
 
 namespace fde {
 
-constexpr int kPlaneThreads2 = 256;
+constexpr int kPlaneThreads2 = 256;  // planes with different sides
 
 // Planes with different sides: the steps of every length as functions of their own, chosen by the
 // sides when the kernel runs (two lengths to a kernel would be 576 kernels a precision).
 template <typename T, int R1, int R2>
 __device__ __noinline__ void any_y_inv(cplx<T>* P, const cplx<T>* X, const PlaneDims& D, int pitch, const cplx<T>* tw) {
-  plane_y_inv<T, R1, R2>(P, X, D, pitch, kPlaneThreads2, tw);
+  plane_y_inv<T, SidePlan<R1, R2>>(P, X, D, pitch, kPlaneThreads2, tw);
 }
 template <typename T, int R1, int R2>
 __device__ __noinline__ void any_y_fwd(cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, const cplx<T>* tw) {
-  plane_y_fwd<T, R1, R2>(P, X, D, pitch, kPlaneThreads2, tw);
+  plane_y_fwd<T, SidePlan<R1, R2>>(P, X, D, pitch, kPlaneThreads2, tw);
 }
-// All columns: inverse x, the potential, forward x.
 template <typename T, int R1, int R2>
 __device__ __noinline__ void any_x_all(cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, int n2, int lb,
                                        const cplx<T>* tw, const T* vp) {
-#pragma unroll 1
-  for (int c0 = 0; c0 < n2; c0 += lb) {
-    const int nc = min(lb, n2 - c0);
-    plane_x_in<T, R1, R2>(P, X, D, pitch, c0, lb, nc, kPlaneThreads2);
-    __syncthreads();
-    plane_x_mul<T, R1, R2>(X, c0, lb, nc, kPlaneThreads2, tw, vp, n2);
-    __syncthreads();
-    plane_x_out<T, R1, R2>(P, X, D, pitch, c0, lb, nc, kPlaneThreads2);
-  }
+  plane_x_all<T, SidePlan<R1, R2>>(P, X, D, pitch, n2, lb, tw, vp);
 }
+template <typename T, int R1, int R2>
+__device__ __noinline__ void any_x_rho(const cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, int n2, int lb,
+                                       const cplx<T>* tw, double weight, bool first, typename RhoAcc<T>::t* rho) {
+  plane_x_rho<T, SidePlan<R1, R2>>(P, X, D, pitch, n2, lb, tw, weight, first, rho);
+}
+#define FDE_ANY(SIDE, CALL)      \
+  switch (SIDE) {                \
+    FDE_PLANE_SIDES(CALL)        \
+  }
+#define FDE_Y_INV(N, R1, R2) \
+  case N: any_y_inv<T, R1, R2>(P, X, D, pitch, tw2); break;
+#define FDE_Y_FWD(N, R1, R2) \
+  case N: any_y_fwd<T, R1, R2>(P, X, D, pitch, tw2); break;
+#define FDE_X_ALL(N, R1, R2) \
+  case N: any_x_all<T, R1, R2>(P, X, D, pitch, n2, lb, tw1, vp); break;
+#define FDE_X_RHO(N, R1, R2) \
+  case N: any_x_rho<T, R1, R2>(P, X, D, pitch, n2, lb, tw1, weight[b], b == b0, rho); break;
 
 template <typename T>
 __global__ void __launch_bounds__(kPlaneThreads2, 2)
@@ -49,107 +57,15 @@ k_plane_pass_any(const __grid_constant__ HpsiBatch<T> B, int n1, int n2, int n3,
   C* S = I.scratch + ((size_t)b * n3 + i3) * sp.ldc;
   const T* vp = I.vplane + (size_t)i3 * n1 * n2;
   const PlaneDims D = plane_dims<T>(sp);
-  plane_columns_in<T>(X, S, sp, D, n1, n2, kPlaneThreads2);
+  plane_columns_in<T>(X, S, sp, D, kPlaneThreads2);
   __syncthreads();
-  switch (n2) {
-#define FDE_CASE(N, R2, R1)                      \
-  case N:                                        \
-    any_y_inv<T, R1, R2>(P, X, D, pitch, tw2);   \
-    break;
-    FDE_SPLIT_SIDES(FDE_CASE)
-#undef FDE_CASE
-  }
+  FDE_ANY(n2, FDE_Y_INV)
   __syncthreads();
-  switch (n1) {
-#define FDE_CASE(N, R2, R1)                                       \
-  case N:                                                         \
-    any_x_all<T, R1, R2>(P, X, D, pitch, n2, lb, tw1, vp);        \
-    break;
-    FDE_SPLIT_SIDES(FDE_CASE)
-#undef FDE_CASE
-  }
+  FDE_ANY(n1, FDE_X_ALL)
   __syncthreads();
-  switch (n2) {
-#define FDE_CASE(N, R2, R1)                      \
-  case N:                                        \
-    any_y_fwd<T, R1, R2>(P, X, D, pitch, tw2);   \
-    break;
-    FDE_SPLIT_SIDES(FDE_CASE)
-#undef FDE_CASE
-  }
+  FDE_ANY(n2, FDE_Y_FWD)
   __syncthreads();
-  plane_columns_out<T>(X, S, sp, D, n1, n2, kPlaneThreads2);
-}
-
-// Shared memory of the plane pass: P for the widest span of the batch, X for one batch of columns
-// and for the column stage.
-template <typename T> static size_t plane_smem2(int n1, int n2, int span1, int span2, int lb) {
-  const size_t p = (size_t)span1 * (n2 | 1);
-  const size_t x = std::max((size_t)n1 * lb, (size_t)span1 * (span2 | 1));
-  return (p + x) * sizeof(cplx<T>);
-}
-constexpr size_t kPlaneSmemMax = 232448;  // 227 KB a CTA can have
-static inline int side_rmax(int n) { return split_of(n).b; }
-
-template <typename T> bool two_step_grid(const GridDims& g, const SphereDev& sp) {
-  if (!split_side_ok(g.n1) || !split_side_ok(g.n2) || split_of(g.n3).a == 0) return false;
-  const int lb = plane_batch(g.n2, side_rmax(g.n1), kPlaneThreads2);
-  return plane_smem2<T>(g.n1, g.n2, sp.span1, sp.span2, lb) <= kPlaneSmemMax;
-}
-
-template <typename K> static inline void allow_smem2(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-template <typename T, int R1, int R2>
-static void plane_square(unsigned blocks, const HpsiBatch<T>& B, int n3, const FftPlans<T>& fp, size_t sm, int psize,
-                         cudaStream_t st) {
-  constexpr int N = R1 * R2;
-  constexpr int MINB = sizeof(T) == 8 ? 2 : (N <= 100 ? 4 : 3);
-  auto* k = k_plane_pass<T, R1, R2, R1, R2, kPlaneThreads2, MINB>;
-  allow_smem2(k, sm);
-  count_launches(1);
-  k<<<blocks, kPlaneThreads2, sm, st>>>(B, n3, fp.p1.tw, fp.p2.tw, psize);
-}
-
-template <typename T>
-void launch_plane_pass(const GridDims& g, unsigned blocks, const HpsiBatch<T>& B, const FftPlans<T>& fp,
-                       cudaStream_t st) {
-  int s1 = 0, s2 = 0;
-  for (int i = 0; i < B.n; ++i) {
-    s1 = std::max(s1, B.it[i].sp.span1);
-    s2 = std::max(s2, B.it[i].sp.span2);
-  }
-  const int lb = plane_batch(g.n2, side_rmax(g.n1), kPlaneThreads2);
-  const size_t sm = plane_smem2<T>(g.n1, g.n2, s1, s2, lb);
-  const int psize = s1 * (g.n2 | 1);
-  if (g.n1 == g.n2) {
-    switch (g.n1) {
-#define FDE_CASE(N, R2, R1)                                          \
-  case N:                                                            \
-    plane_square<T, R1, R2>(blocks, B, g.n3, fp, sm, psize, st);     \
-    return;
-      FDE_SPLIT_SIDES(FDE_CASE)
-#undef FDE_CASE
-    }
-    return;
-  }
-  allow_smem2(k_plane_pass_any<T>, sm);
-  count_launches(1);
-  k_plane_pass_any<T><<<blocks, kPlaneThreads2, sm, st>>>(B, g.n1, g.n2, g.n3, fp.p1.tw, fp.p2.tw, psize, lb);
-}
-
-template <typename T, int R1, int R2>
-__device__ __noinline__ void any_x_rho(const cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, int n2, int lb,
-                                       const cplx<T>* tw, double weight, bool first, typename RhoAcc<T>::t* rho) {
-#pragma unroll 1
-  for (int c0 = 0; c0 < n2; c0 += lb) {
-    const int nc = min(lb, n2 - c0);
-    plane_x_in<T, R1, R2>(P, X, D, pitch, c0, lb, nc, kPlaneThreads2);
-    __syncthreads();
-    plane_x_rho<T, R1, R2>(X, c0, lb, nc, kPlaneThreads2, tw, weight, first, rho, n2);
-    __syncthreads();
-  }
+  plane_columns_out<T>(X, S, sp, kPlaneThreads2);
 }
 
 template <typename T>
@@ -168,26 +84,98 @@ k_plane_rho_any(const cplx<T>* __restrict__ scratch, SphereDev sp, int nb, const
   auto* rho = part + ((size_t)g * n3 + i3) * n1 * n2;
 #pragma unroll 1
   for (int b = b0; b < b1; ++b) {
-    plane_columns_in<T>(X, scratch + ((size_t)b * n3 + i3) * sp.ldc, sp, D, n1, n2, kPlaneThreads2);
+    plane_columns_in<T>(X, scratch + ((size_t)b * n3 + i3) * sp.ldc, sp, D, kPlaneThreads2);
     __syncthreads();
-    switch (n2) {
-#define FDE_CASE(N, R2, R1)                      \
-  case N:                                        \
-    any_y_inv<T, R1, R2>(P, X, D, pitch, tw2);   \
-    break;
-      FDE_SPLIT_SIDES(FDE_CASE)
-#undef FDE_CASE
-    }
+    FDE_ANY(n2, FDE_Y_INV)
     __syncthreads();
-    switch (n1) {
-#define FDE_CASE(N, R2, R1)                                                            \
-  case N:                                                                              \
-    any_x_rho<T, R1, R2>(P, X, D, pitch, n2, lb, tw1, weight[b], b == b0, rho);        \
-    break;
-      FDE_SPLIT_SIDES(FDE_CASE)
-#undef FDE_CASE
-    }
+    FDE_ANY(n1, FDE_X_RHO)
   }
+}
+
+// Shared memory of the plane pass: P for the widest span of the batch, X for one batch of columns
+// and for the column stage.
+template <typename T> static size_t plane_smem2(int n1, int n2, int span1, int span2, int lb) {
+  const size_t p = (size_t)span1 * (n2 | 1);
+  const size_t x = std::max((size_t)n1 * lb, (size_t)span1 * (span2 | 1));
+  return (p + x) * sizeof(cplx<T>);
+}
+constexpr size_t kPlaneSmemMax = 232448;  // 227 KB a CTA can have
+
+// Threads and least resident CTAs of a square plane's kernel.  A CTA has threads for one row of items of
+// the y steps (0.46 N rows hold columns at the cutoffs the grids are made for) and for whole batches
+// of columns, so that few rounds run with a handful of threads: 72 x 72, 33 rows of 9 items and two
+// batches of 36 columns, 352 threads.
+struct PlaneShape {
+  int nt, minb;
+};
+template <typename T> __host__ __device__ constexpr PlaneShape plane_shape(int n) {
+  if (sizeof(T) == 8) return n == 72 ? PlaneShape{352, 2} : PlaneShape{n <= 24 ? 192 : 256, 2};
+  if (n <= 24) return PlaneShape{192, 4};
+  if (n == 72) return PlaneShape{352, 3};
+  if (n <= 90) return PlaneShape{256, 4};
+  if (n <= 96) return PlaneShape{288, 3};
+  if (n <= 108) return PlaneShape{256, 3};
+  return PlaneShape{n == 144 ? 384 : 320, 2};
+}
+__host__ __device__ constexpr int side_rmax(int n) {
+  switch (n) {
+#define FDE_CASE(N, R1, R2) \
+  case N:                   \
+    return R1;
+    FDE_PLANE_SIDES(FDE_CASE)
+#undef FDE_CASE
+  }
+  return 1;
+}
+template <typename T> static int plane_lb(int n1, int n2) {
+  return plane_batch(n2, side_rmax(n1), n1 == n2 ? plane_shape<T>(n1).nt : kPlaneThreads2);
+}
+
+template <typename T> bool two_step_grid(const GridDims& g, const SphereDev& sp) {
+  if (!split_side_ok(g.n1) || !split_side_ok(g.n2) || split_of(g.n3).a == 0) return false;
+  return plane_smem2<T>(g.n1, g.n2, sp.span1, sp.span2, plane_lb<T>(g.n1, g.n2)) <= kPlaneSmemMax;
+}
+
+template <typename K> static inline void allow_smem2(K kernel, size_t bytes) {
+  if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+template <typename T, int R1, int R2>
+static void plane_square(unsigned blocks, const HpsiBatch<T>& B, int n3, const FftPlans<T>& fp, size_t sm, int psize,
+                         cudaStream_t st) {
+  constexpr PlaneShape S = plane_shape<T>(R1 * R2);
+  using Plan = SidePlan<R1, R2>;
+  auto* k = k_plane_pass<T, Plan, Plan, S.nt, S.minb>;
+  allow_smem2(k, sm);
+  count_launches(1);
+  k<<<blocks, S.nt, sm, st>>>(B, n3, fp.p1.tw, fp.p2.tw, psize);
+}
+
+template <typename T>
+void launch_plane_pass(const GridDims& g, unsigned blocks, const HpsiBatch<T>& B, const FftPlans<T>& fp,
+                       cudaStream_t st) {
+  int s1 = 0, s2 = 0;
+  for (int i = 0; i < B.n; ++i) {
+    s1 = std::max(s1, B.it[i].sp.span1);
+    s2 = std::max(s2, B.it[i].sp.span2);
+  }
+  const int lb = plane_lb<T>(g.n1, g.n2);
+  const size_t sm = plane_smem2<T>(g.n1, g.n2, s1, s2, lb);
+  const int psize = s1 * (g.n2 | 1);
+  if (g.n1 == g.n2) {
+    switch (g.n1) {
+#define FDE_CASE(N, R1, R2)                                          \
+  case N:                                                            \
+    plane_square<T, R1, R2>(blocks, B, g.n3, fp, sm, psize, st);     \
+    return;
+      FDE_PLANE_SIDES(FDE_CASE)
+#undef FDE_CASE
+    }
+    return;
+  }
+  allow_smem2(k_plane_pass_any<T>, sm);
+  count_launches(1);
+  k_plane_pass_any<T><<<blocks, kPlaneThreads2, sm, st>>>(B, g.n1, g.n2, g.n3, fp.p1.tw, fp.p2.tw, psize, lb);
 }
 
 // rho_plane (+)= the groups' partial sums, in group order.
@@ -207,12 +195,12 @@ template <typename T, int R1, int R2>
 static void rho_square(dim3 grid, const cplx<T>* scr, const SphereDev& sp, int nb, const double* weight,
                        typename RhoAcc<T>::t* part, int n3, const FftPlans<T>& fp, size_t sm, int psize,
                        cudaStream_t st) {
-  constexpr int N = R1 * R2;
-  constexpr int MINB = sizeof(T) == 8 ? 2 : (N <= 100 ? 4 : 3);
-  auto* k = k_plane_rho<T, R1, R2, R1, R2, kPlaneThreads2, MINB>;
+  constexpr PlaneShape S = plane_shape<T>(R1 * R2);
+  using Plan = SidePlan<R1, R2>;
+  auto* k = k_plane_rho<T, Plan, Plan, S.nt, S.minb>;
   allow_smem2(k, sm);
   count_launches(1);
-  k<<<grid, kPlaneThreads2, sm, st>>>(scr, sp, nb, weight, part, n3, fp.p1.tw, fp.p2.tw, psize);
+  k<<<grid, S.nt, sm, st>>>(scr, sp, nb, weight, part, n3, fp.p1.tw, fp.p2.tw, psize);
 }
 
 // Groups of bands of a plane density: enough CTAs for four on each of 152 SMs.
@@ -225,17 +213,17 @@ void launch_plane_density(const GridDims& g, const cplx<T>* scr, const SphereDev
   static_assert(sizeof(A) == sizeof(double), "partial sums take the space of a double");
   A* part = reinterpret_cast<A*>(part_);
   const int groups = plane_density_groups(nb, g.n3);
-  const int lb = plane_batch(g.n2, side_rmax(g.n1), kPlaneThreads2);
+  const int lb = plane_lb<T>(g.n1, g.n2);
   const size_t sm = plane_smem2<T>(g.n1, g.n2, sp.span1, sp.span2, lb);
   const int psize = sp.span1 * (g.n2 | 1);
   const dim3 grid(g.n3, groups);
   if (g.n1 == g.n2) {
     switch (g.n1) {
-#define FDE_CASE(N, R2, R1)                                                                        \
+#define FDE_CASE(N, R1, R2)                                                                        \
   case N:                                                                                          \
     rho_square<T, R1, R2>(grid, scr, sp, nb, weight, part, g.n3, fp, sm, psize, st);               \
     break;
-      FDE_SPLIT_SIDES(FDE_CASE)
+      FDE_PLANE_SIDES(FDE_CASE)
 #undef FDE_CASE
     }
   } else {

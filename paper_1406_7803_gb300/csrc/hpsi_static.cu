@@ -32,7 +32,7 @@ constexpr long long kStScratch = 1 << 20;  // complex values of the column scrat
 static __device__ __align__(256) double2 st_scratch[kStScratch];
 static __device__ __align__(256) double st_vplane[kStMaxGrid];
 static __device__ __align__(256) double st_kin[kStMaxNpw];
-static __device__ __align__(256) int st_cols[4 * kStMaxCols + 1 + kMaxPlane];
+static __device__ __align__(256) int st_cols[5 * kStMaxCols + 1 + kMaxPlane];
 static __device__ __align__(256) int st_ncols[6];
 static __device__ __align__(256) double2 st_tw[3][kMaxLine];
 
@@ -67,7 +67,7 @@ static fde_status static_setup(int dev, StaticPtrs* out) {
   return FDE_OK;
 }
 
-// Column map of a sphere (one CTA): cols = [start(ncol+1) | m3lo | i1 | i2 | rows];
+// Column map of a sphere (one CTA): cols = [start(ncol+1) | m3lo | i1 | i2 | place in the span | rows];
 // ncols = {ncol, nrow, lowest m1 mod n1, m1 span, lowest m2 mod n2, m2 span}.  A column starts where (m1, m2) changes; rows are the distinct i1.
 // The caller's list is checked on the way, because the transforms index shared-memory lines
 // by it: (m1, m2) keys strictly increasing from column to column (sorted, no repeats), m3
@@ -160,7 +160,8 @@ k_static_columns(const int* __restrict__ mil, int npw, int n1, int n2, int n3, i
   int* m3lo = cols + ncol + 1;
   int* ci1 = m3lo + ncol;
   int* ci2 = ci1 + ncol;
-  int* rows = ci2 + ncol;
+  int* pos = ci2 + ncol;
+  int* rows = pos + ncol;
   for (int c = threadIdx.x; c < ncol; c += blockDim.x) {
     const int p = start[c];
     const int m1 = mil[3 * p], m2 = mil[3 * p + 1];
@@ -168,6 +169,7 @@ k_static_columns(const int* __restrict__ mil, int npw, int n1, int n2, int n3, i
     const int i1 = ((m1 % n1) + n1) % n1;
     ci1[c] = i1;
     ci2[c] = ((m2 % n2) + n2) % n2;
+    pos[c] = (m1 - lo1) * ((hi2 - lo2 + 1) | 1) + m2 - lo2;
     rowflag[i1] = 1;
   }
   __syncthreads();
@@ -270,7 +272,8 @@ extern "C" fde_status fde_apply_h_local_static(const fde_cell_desc* cell, const 
   sp.col_m3lo = P.cols + ncol + 1;
   sp.col_i1 = sp.col_m3lo + ncol;
   sp.col_i2 = sp.col_i1 + ncol;
-  sp.row_i1 = sp.col_i2 + ncol;
+  sp.col_pos = sp.col_i2 + ncol;
+  sp.row_i1 = sp.col_pos + ncol;
   FftPlans<double> fp;
   fp.p1 = lp[0];
   fp.p2 = lp[1];

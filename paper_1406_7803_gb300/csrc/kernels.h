@@ -21,6 +21,7 @@ struct SphereDev {
   const int* col_i1;     // [ncol] grid index i1 = m1 mod n1
   const int* col_i2;     // [ncol] grid index i2 = m2 mod n2
   const int* row_i1;     // [nrow] distinct i1 holding at least one column
+  const int* col_pos;    // [ncol] place in the span: (m1 - lowest m1) (span2 | 1) + m2 - lowest m2
 };
 
 struct GridDims {
