@@ -29,21 +29,20 @@ template <typename C> __device__ __forceinline__ void dft3(C* v, int sign) {
   using T = decltype(v[0].x);
   constexpr T h = T(0.86602540378443864676);  // sin(2 pi / 3)
   constexpr T half = T(0.5);
-  C t1 = cadd(v[1], v[2]);
-  C t2 = cmuli(cscale(csub(v[1], v[2]), h), sign);
-  C m = csub(v[0], cscale(t1, half));
-  v[0] = cadd(v[0], t1);
-  v[1] = cadd(m, t2);
-  v[2] = csub(m, t2);
+  const C t = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+  const C m = caxmy(t, half, v[0]);
+  v[0] = cadd(v[0], t);
+  v[1] = caddi(m, d, h, sign);
+  v[2] = caddi(m, d, h, -sign);
 }
 
 template <typename C> __device__ __forceinline__ void dft4(C* v, int sign) {
-  C a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
-  C c = cadd(v[1], v[3]), d = cmuli(csub(v[1], v[3]), sign);
+  const C a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
+  const C c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
   v[0] = cadd(a, c);
   v[2] = csub(a, c);
-  v[1] = cadd(b, d);
-  v[3] = csub(b, d);
+  v[1] = caddi(b, d, sign);
+  v[3] = caddi(b, d, -sign);
 }
 
 template <typename C> __device__ __forceinline__ void dft5(C* v, int sign) {
@@ -52,17 +51,17 @@ template <typename C> __device__ __forceinline__ void dft5(C* v, int sign) {
   constexpr T c2 = T(-0.80901699437494742410);  // cos(4 pi / 5)
   constexpr T s1 = T(0.95105651629515357212);   // sin(2 pi / 5)
   constexpr T s2 = T(0.58778525229247312917);   // sin(4 pi / 5)
-  C t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
-  C t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
-  C a1 = cadd(v[0], cadd(cscale(t1, c1), cscale(t2, c2)));
-  C a2 = cadd(v[0], cadd(cscale(t1, c2), cscale(t2, c1)));
-  C b1 = cmuli(cadd(cscale(t3, s1), cscale(t4, s2)), sign);
-  C b2 = cmuli(csub(cscale(t3, s2), cscale(t4, s1)), sign);
+  const C t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
+  const C t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
+  const C a1 = caxpy(t2, c2, caxpy(t1, c1, v[0]));
+  const C a2 = caxpy(t2, c1, caxpy(t1, c2, v[0]));
+  const C b1 = caxpy(t4, s2, cscale(t3, s1));
+  const C b2 = caxmy(t4, s1, cscale(t3, s2));
   v[0] = cadd(v[0], cadd(t1, t2));
-  v[1] = cadd(a1, b1);
-  v[4] = csub(a1, b1);
-  v[2] = cadd(a2, b2);
-  v[3] = csub(a2, b2);
+  v[1] = caddi(a1, b1, sign);
+  v[4] = caddi(a1, b1, -sign);
+  v[2] = caddi(a2, b2, sign);
+  v[3] = caddi(a2, b2, -sign);
 }
 
 template <int R, typename C> __device__ __forceinline__ void dftR(C* v, int sign) {

@@ -30,15 +30,16 @@ template <typename C> __device__ __forceinline__ void dft8(C* v, int sign) {
   C e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
   dft4(e, sign);
   dft4(o, sign);
-  const C t1 = o[1], t3 = o[3];
-  o[1] = cscale(cadd(t1, cmuli(t1, sign)), h);  // (1 + sign i) / sqrt 2
-  o[2] = cmuli(o[2], sign);                     // sign i
-  o[3] = cscale(csub(cmuli(t3, sign), t3), h);  // (-1 + sign i) / sqrt 2
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    v[k] = cadd(e[k], o[k]);
-    v[k + 4] = csub(e[k], o[k]);
-  }
+  const C p = caddi(o[1], o[1], sign);        // (1 + sign i) o_1
+  const C q = caddi(o[3], o[3], -sign);       // (1 - sign i) o_3; W_8^3 o_3 = -h q
+  v[0] = cadd(e[0], o[0]);
+  v[4] = csub(e[0], o[0]);
+  v[1] = caxpy(p, h, e[1]);
+  v[5] = caxmy(p, h, e[1]);
+  v[2] = caddi(e[2], o[2], sign);
+  v[6] = caddi(e[2], o[2], -sign);
+  v[3] = caxmy(q, h, e[3]);
+  v[7] = caxpy(q, h, e[3]);
 }
 
 // A x A points with the inner roots exp(sign 2 pi i k / A^2), k = 0 .. (A - 1)^2, in wc / ws.
