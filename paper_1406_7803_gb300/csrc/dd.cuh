@@ -114,4 +114,22 @@ struct __align__(16) ddc {
 };
 template <> struct cx<dd> { using t = ddc; };
 
+// a b + c d (or a b - c d) with one renormalisation: the two leading products are split exactly and
+// summed with their rounding error, every smaller term joins the low part.  19 operations where two
+// products and an accurate sum take 34, at the same error of some 2^-46 of |a b| + |c d|.
+__device__ __forceinline__ dd dd_dot2(dd a, dd b, dd c, dd d) {
+  const float p = __fmul_rn(a.hi, b.hi), q = __fmul_rn(c.hi, d.hi);
+  float e = __fmaf_rn(a.hi, b.hi, -p), f = __fmaf_rn(c.hi, d.hi, -q);
+  e = __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, e));
+  f = __fmaf_rn(c.lo, d.hi, __fmaf_rn(c.hi, d.lo, f));
+  const dd s = dd_two_sum(p, q);
+  return dd_fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(e, f)));
+}
+__device__ __forceinline__ ddc cmul(ddc a, ddc b) {
+  ddc z;
+  z.x = dd_dot2(a.x, b.x, -a.y, b.y);
+  z.y = dd_dot2(a.x, b.y, a.y, b.x);
+  return z;
+}
+
 }  // namespace fde

@@ -583,9 +583,12 @@ template <typename T> struct EngineT : Engine {
     if (!on_device) CK(cudaStreamSynchronize(st));
   }
   void sum_densities() {
-    CK(cudaMemcpyAsync(rho_tot.p, subs[0]->rho.p, nr * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    for (size_t I = 1; I < subs.size(); ++I)
-      grid_combine<double>(rho_tot.p, subs[I]->rho.p, nullptr, nullptr, 0.0, rho_tot.p, nr, st);
+    for (size_t I = 0; I < subs.size(); I += 64) {
+      GridList l{};
+      const int n = (int)std::min<size_t>(64, subs.size() - I);
+      for (int k = 0; k < n; ++k) l.p[k] = subs[I + k]->rho.p;
+      grid_sum(l, n, I > 0, rho_tot.p, nr, st);
+    }
   }
   void get_density(int i, double* d_rho) override {
     REQ(d_rho, FDE_EINVAL, "null output");
@@ -743,17 +746,10 @@ template <typename T> struct EngineT : Engine {
       }
       grid_assemble_pair<T>(RT, Da, Db, Dz, hb ? 1 : 0, F, g, cell, nullptr, st);
       launch_fft3d<T>(F, g, plans.fp, +1, st);
-      grid_finish_pair<T>(F, vloc.p, pa ? A.veff.p : nullptr, pb ? B->veff.p : nullptr, nr, st);
-      if (pa) {
-        grid_nonfinite(A.veff.p, nr, status.p, st);
-        to_plane(A);
-        refresh_screening(A);
-      }
-      if (pb) {
-        grid_nonfinite(B->veff.p, nr, status.p, st);
-        to_plane(*B);
-        refresh_screening(*B);
-      }
+      grid_finish_pair<T>(F, vloc.p, pa ? A.veff.p : nullptr, pb ? B->veff.p : nullptr, pa ? A.vplane.p : nullptr,
+                          pb ? B->vplane.p : nullptr, g, status.p, st);
+      if (pa) refresh_screening(A);
+      if (pb) refresh_screening(*B);
     }
     EnergyParts ep;
     if (want_e) {

@@ -196,11 +196,12 @@ template <int R1_, int R2_> struct SidePlan {
     return kCoprime ? wrap(out0(q) + out(p)) : q + R1 * p;  // the latter never wraps
   }
 };
-// Sides as X(N, R1, R2).
-#define FDE_PLANE_SIDES(X)                                                                                       \
-  X(24, 8, 3) X(30, 6, 5) X(32, 8, 4) X(36, 9, 4) X(40, 8, 5) X(45, 9, 5) X(48, 16, 3) X(50, 10, 5) X(54, 9, 6)   \
-  X(60, 12, 5) X(64, 8, 8) X(72, 9, 8) X(75, 15, 5) X(80, 16, 5) X(90, 10, 9) X(96, 12, 8) X(100, 10, 10)         \
-  X(108, 12, 9) X(120, 15, 8) X(128, 16, 8) X(135, 15, 9) X(144, 16, 9) X(150, 15, 10) X(160, 16, 10)
+// Sides as X(N, R1, R2), in the groups of FDE_SPLIT_SIDES.
+#define FDE_PLANE_SIDES0(X) X(24, 8, 3) X(30, 6, 5) X(32, 8, 4) X(36, 9, 4) X(40, 8, 5) X(45, 9, 5) X(48, 16, 3)
+#define FDE_PLANE_SIDES1(X) X(50, 10, 5) X(54, 9, 6) X(60, 12, 5) X(64, 8, 8) X(72, 9, 8) X(75, 15, 5)
+#define FDE_PLANE_SIDES2(X) X(80, 16, 5) X(90, 10, 9) X(96, 12, 8) X(100, 10, 10) X(108, 12, 9) X(120, 15, 8)
+#define FDE_PLANE_SIDES3(X) X(128, 16, 8) X(135, 15, 9) X(144, 16, 9) X(150, 15, 10) X(160, 16, 10)
+#define FDE_PLANE_SIDES(X) FDE_PLANE_SIDES0(X) FDE_PLANE_SIDES1(X) FDE_PLANE_SIDES2(X) FDE_PLANE_SIDES3(X)
 
 __host__ __device__ constexpr int round_up(int n, int m) { return (n + m - 1) / m * m; }
 

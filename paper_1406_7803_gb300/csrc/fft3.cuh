@@ -48,12 +48,13 @@ template <typename C> __device__ __forceinline__ void ax_put(void* p, int i, ddc
   reinterpret_cast<double2*>(p)[i] = make_double2(dd_to_double(v.x), dd_to_double(v.y));
 }
 
-// Strided axis: element e of line l = (o, t) at (o N + e) stride + t, t < stride.
-template <typename T, int R1, int R2, typename IN, typename OUT>
-__global__ void __launch_bounds__(ax_threads<cplx<T>, R1, R2>())
+// Strided axis: element e of line l = (o, t) at (o N + e) stride + t, t < stride; on the side's plan
+// (prime-factor indices where it has coprime factors: no twiddles).
+template <typename T, typename Plan, typename IN, typename OUT>
+__global__ void __launch_bounds__(ax_threads<cplx<T>, Plan::R1, Plan::R2>())
 k_fft_strided(void* __restrict__ data, int nlines, int stride, const cplx<T>* __restrict__ tw, bool conj) {
   using C = cplx<T>;
-  constexpr int N = R1 * R2, L = ax_lines<C>(), NT = ax_threads<C, R1, R2>();
+  constexpr int R1 = Plan::R1, R2 = Plan::R2, N = Plan::N, L = ax_lines<C>(), NT = ax_threads<C, R1, R2>();
   __shared__ __align__(16) C X[N * L];
   const int c = threadIdx.x % L, i = threadIdx.x / L;
   const int l = blockIdx.x * L + c;
@@ -64,7 +65,8 @@ k_fft_strided(void* __restrict__ data, int nlines, int stride, const cplx<T>* __
   if (live && i < R2) {
     C v[R1];
 #pragma unroll
-    for (int r = 0; r < R1; ++r) v[r] = ax_conj(ax_get<C>(data, base + (i + r * R2) * stride, IN()), conj);
+    for (int r = 0; r < R1; ++r)
+      v[r] = ax_conj(ax_get<C>(data, base + Plan::wrap(Plan::in0(i) + r * R2) * stride, IN()), conj);
     dft_r<R1>(v, -1);
 #pragma unroll
     for (int q = 0; q < R1; ++q) X[(q * R2 + i) * L + c] = v[q];
@@ -75,11 +77,11 @@ k_fft_strided(void* __restrict__ data, int nlines, int stride, const cplx<T>* __
 #pragma unroll
     for (int j = 0; j < R2; ++j) {
       v[j] = X[(i * R2 + j) * L + c];
-      if (j) v[j] = cmul(v[j], tw[j * i]);
+      if (!Plan::kCoprime && j) v[j] = cmul(v[j], tw[j * i]);
     }
     dft_r<R2>(v, -1);
 #pragma unroll
-    for (int p = 0; p < R2; ++p) ax_put<C>(data, base + (i + R1 * p) * stride, ax_conj(v[p], conj), OUT());
+    for (int p = 0; p < R2; ++p) ax_put<C>(data, base + Plan::output(i, p) * stride, ax_conj(v[p], conj), OUT());
   }
 }
 
@@ -140,8 +142,8 @@ k_fft_contig(void* __restrict__ data, int nlines, const cplx<T>* __restrict__ tw
 #define FDE_STRIDED_CASE(N, R1, R2)                                                                               \
   case N:                                                                                                         \
     count_launches(1);                                                                                            \
-    k_fft_strided<T, R1, R2, IN, OUT><<<blocks, ax_threads<cplx<T>, R1, R2>(), 0, st>>>(data, (int)nlines,       \
-                                                                                         stride, tw, sign > 0);  \
+    k_fft_strided<T, SidePlan<R1, R2>, IN, OUT><<<blocks, ax_threads<cplx<T>, R1, R2>(), 0, st>>>(               \
+        data, (int)nlines, stride, tw, sign > 0);                                                                 \
     return true;
 #define FDE_CONTIG_CASE(N, R1, R2)                                                                                \
   case N:                                                                                                         \

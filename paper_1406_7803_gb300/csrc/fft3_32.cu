@@ -4,7 +4,7 @@
 namespace fde {
 
 namespace {
-FDE_AXIS_LAUNCHERS(FDE_SPLIT_SIDES, FDE_SPLIT_LINES)
+FDE_AXIS_LAUNCHERS(FDE_PLANE_SIDES, FDE_SPLIT_LINES)
 }
 
 template <>

@@ -1,5 +1,5 @@
 // fft_dd_0.cu -- double-float axis passes of one group of lengths (fft_dd.cuh).
-#define FDE_DD_SIDES FDE_SPLIT_SIDES0
+#define FDE_DD_SIDES FDE_PLANE_SIDES0
 #define FDE_DD_LINES FDE_SPLIT_SIDES0
 #define FDE_DD_AXIS dd_axis_0
 #include "fft_dd.cuh"

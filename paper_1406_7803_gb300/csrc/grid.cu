@@ -88,7 +88,7 @@ __device__ __forceinline__ Gpt gvec(long long idx, const GridDims& g, const Cell
   return p;
 }
 
-constexpr int kRedBlocks = 304;  // 2 x 152 SMs
+constexpr int kRedBlocks = 912;  // 6 x 152 SMs
 constexpr int kRedThreads = 256;
 
 __device__ __forceinline__ void block_sum_store(double v, double* out_slot) {
@@ -376,72 +376,113 @@ __global__ void k_nonfinite(const double* __restrict__ a, long long n, unsigned*
 // a(G) = (C(G) + conj C(-G)) / 2 and b(G) = (C(G) - conj C(-G)) / (2 i).  The potential build
 // packs the subsystem densities, gradient components and divergence arguments in pairs, so
 // that it needs half the FP64 transforms while computing the same quantities.
-__device__ __forceinline__ long long neg_index(long long idx, const GridDims& g) {
-  const int id = (int)idx;
-  const int i3 = id % g.n3;
-  const int r = id / g.n3;
-  const int i2 = r % g.n2, i1 = r / g.n2;
-  const int j1 = i1 ? g.n1 - i1 : 0, j2 = i2 ? g.n2 - i2 : 0, j3 = i3 ? g.n3 - i3 : 0;
-  return (long long)((j1 * g.n2 + j2) * g.n3 + j3);
-}
 __device__ __forceinline__ double2 to_d2(double2 v) { return v; }
 __device__ __forceinline__ double2 to_d2(float2 v) { return make_double2((double)v.x, (double)v.y); }
-__device__ __forceinline__ void unpack2(double2 c, double2 cn, double2* a, double2* b) {
-  *a = make_double2(0.5 * (c.x + cn.x), 0.5 * (c.y - cn.y));
-  *b = make_double2(0.5 * (c.y + cn.y), -0.5 * (c.x - cn.x));
-}
-// u + i v for complex u, v
-__device__ __forceinline__ double2 pack2(double2 u, double2 v) { return make_double2(u.x - v.y, u.y + v.x); }
-// i g f
-__device__ __forceinline__ double2 ig_mul(double gc, double2 f) { return make_double2(-gc * f.y, gc * f.x); }
-
 __global__ void k_pack2(const double* __restrict__ a, const double* __restrict__ b, double2* __restrict__ c,
                         long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     c[i] = make_double2(a[i], b ? b[i] : 0.0);
 }
 
+// The reciprocal-space passes take the points G and -G together: the fields of a packed pair unpack
+// from the same two grid values at both, their products with the components of G differ in sign
+// alone, and G^2 and 4 pi / G^2 are the same.  They are bound by FP64 operations (64 cycles of an SM
+// quarter a warp instruction), so the components of G come from tables (a conversion and a product
+// each otherwise) and every product is formed once for the pair.  72 x 72 x 180: unpacking 108 us
+// and assembling 155 us with a thread per point.
+constexpr int kAxisMax = 320;
+struct GTables {
+  double x[kAxisMax], y[kAxisMax], z[kAxisMax];
+};
+__device__ __forceinline__ double axis_g(int i, int n, double b) { return (double)(i < (n + 1) / 2 ? i : i - n) * b; }
+// The components of G along the (orthorhombic) axes, by grid index; all threads of the CTA.
+__device__ __forceinline__ void fill_tables(GTables& t, const GridDims& g, const CellDev& c) {
+  for (int i = threadIdx.x; i < g.n1; i += blockDim.x) t.x[i] = axis_g(i, g.n1, c.b[0][0]);
+  for (int i = threadIdx.x; i < g.n2; i += blockDim.x) t.y[i] = axis_g(i, g.n2, c.b[1][1]);
+  for (int i = threadIdx.x; i < g.n3; i += blockDim.x) t.z[i] = axis_g(i, g.n3, c.b[2][2]);
+  __syncthreads();
+}
+// Points with i1 <= n1 / 2 whose partner does not come before them: one of every pair G, -G.
+struct GPair {
+  int idx, jn;
+  double gx, gy, gz, g2;
+  bool nyq;
+};
+__device__ __forceinline__ bool pair_point(int idx, const GridDims& g, const GTables& t, GPair* p) {
+  const int i3 = idx % g.n3, r = idx / g.n3;
+  const int i2 = r % g.n2, i1 = r / g.n2;
+  const int j1 = i1 ? g.n1 - i1 : 0, j2 = i2 ? g.n2 - i2 : 0, j3 = i3 ? g.n3 - i3 : 0;
+  p->idx = idx;
+  p->jn = (j1 * g.n2 + j2) * g.n3 + j3;
+  if (p->jn < idx) return false;
+  p->gx = t.x[i1];
+  p->gy = t.y[i2];
+  p->gz = t.z[i3];
+  p->g2 = p->gx * p->gx + p->gy * p->gy + p->gz * p->gz;
+  p->nyq = (2 * i1 == g.n1) || (2 * i2 == g.n2) || (2 * i3 == g.n3);
+  return true;
+}
+__device__ __forceinline__ int pair_end(const GridDims& g) { return (g.n1 / 2 + 1) * g.n2 * g.n3; }
+
 // From C = FFT(rho_a + i rho_b) (unscaled): RT (+)= rho_a(G) + rho_b(G); Hartree sums
 // sum 4 pi |rho_x(G)|^2 / G^2 of both into partial rows 0 and 1; packed gradient transforms
 // Pa = iGx a + i iGy a, Pb = iGx b + i iGy b, Pz = iGz a + i iGz b (Nyquist planes zero).
-// Without b, C is rho_a's transform itself, Pb is not written and Pz carries iGz a alone.
-__global__ void k_unpack_density(const double2* __restrict__ C, int has_b, double2* __restrict__ RT, int accumulate,
-                                 double2* __restrict__ Pa, double2* __restrict__ Pb, double2* __restrict__ Pz,
-                                 GridDims g, CellDev c, double inv_nr, double* partial) {
-  const long long nr = (long long)g.n1 * g.n2 * g.n3;
+// Without b, C is rho_a's transform itself (the pair's second field is zero), Pb is not written and Pz
+// carries iGz a alone.
+template <bool SUMS>
+__global__ void __launch_bounds__(kRedThreads)
+k_unpack_density(const double2* __restrict__ C, int has_b, double2* __restrict__ RT, int accumulate,
+                 double2* __restrict__ Pa, double2* __restrict__ Pb, double2* __restrict__ Pz, GridDims g, CellDev c,
+                 double inv_nr, double* partial) {
+  __shared__ GTables tab;
+  fill_tables(tab, g, c);
+  const int end = pair_end(g);
+  const double s = 0.5 * inv_nr;
   double ea = 0, eb = 0;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < nr; idx += (long long)gridDim.x * blockDim.x) {
-    const Gpt p = gvec(idx, g, c);
-    const double2 cv = C[idx];
-    double2 a, b;
-    if (has_b) {
-      unpack2(cv, C[neg_index(idx, g)], &a, &b);
-    } else {
-      a = cv;
-      b = make_double2(0, 0);
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < end; idx += gridDim.x * blockDim.x) {
+    GPair p;
+    if (!pair_point(idx, g, tab, &p)) continue;
+    const double2 u = C[p.idx], v = C[p.jn];
+    const double2 a = make_double2(s * (u.x + v.x), s * (u.y - v.y));
+    const double2 b = has_b ? make_double2(s * (u.y + v.y), s * (v.x - u.x)) : make_double2(0, 0);
+    double2 t = make_double2(a.x + b.x, a.y + b.y), tn = cconj(t);
+    if (accumulate) {
+      const double2 r = RT[p.idx], rn = RT[p.jn];
+      t = cadd(t, r);
+      tn = cadd(tn, rn);
     }
-    a.x *= inv_nr; a.y *= inv_nr;
-    b.x *= inv_nr; b.y *= inv_nr;
-    double2 t = make_double2(a.x + b.x, a.y + b.y);
-    if (accumulate) t = make_double2(RT[idx].x + t.x, RT[idx].y + t.y);
-    RT[idx] = t;
-    if (p.g2 > 0 && !p.nyq) {
-      const double f = 4.0 * M_PI / p.g2;
+    RT[p.idx] = t;
+    RT[p.jn] = tn;
+    if (SUMS && p.g2 > 0 && !p.nyq) {
+      const double f = (p.idx == p.jn ? 4.0 : 8.0) * M_PI / p.g2;
       ea += f * (a.x * a.x + a.y * a.y);
       eb += f * (b.x * b.x + b.y * b.y);
     }
     if (Pa) {
       if (p.nyq) {
-        Pa[idx] = Pz[idx] = make_double2(0, 0);
-        if (has_b) Pb[idx] = make_double2(0, 0);
+        const double2 z = make_double2(0, 0);
+        Pa[p.idx] = Pa[p.jn] = Pz[p.idx] = Pz[p.jn] = z;
+        if (has_b) Pb[p.idx] = Pb[p.jn] = z;
       } else {
-        Pa[idx] = pack2(ig_mul(p.gx, a), ig_mul(p.gy, a));
-        if (has_b) Pb[idx] = pack2(ig_mul(p.gx, b), ig_mul(p.gy, b));
-        Pz[idx] = pack2(ig_mul(p.gz, a), ig_mul(p.gz, b));
+        // i G a at G and -G: the products with a's parts, summed and subtracted
+        const double xx = p.gx * a.x, xy = p.gx * a.y, yx = p.gy * a.x, yy = p.gy * a.y;
+        Pa[p.idx] = make_double2(-xy - yx, xx - yy);
+        Pa[p.jn] = make_double2(yx - xy, -xx - yy);
+        const double zx = p.gz * a.x, zy = p.gz * a.y;
+        double wx = 0, wy = 0;
+        if (has_b) {
+          const double ux = p.gx * b.x, uy = p.gx * b.y, vx = p.gy * b.x, vy = p.gy * b.y;
+          Pb[p.idx] = make_double2(-uy - vx, ux - vy);
+          Pb[p.jn] = make_double2(vx - uy, -ux - vy);
+          wx = p.gz * b.x;
+          wy = p.gz * b.y;
+        }
+        Pz[p.idx] = make_double2(-zy - wx, zx - wy);
+        Pz[p.jn] = make_double2(wx - zy, -zx - wy);
       }
     }
   }
-  if (partial) {
+  if (SUMS) {
     block_sum_store(ea, partial + blockIdx.x);
     block_sum_store(eb, partial + kRedBlocks + blockIdx.x);
   }
@@ -538,58 +579,111 @@ __global__ void k_pw_pair(const double* __restrict__ ra, const double* __restric
 // Reciprocal-space part of the potentials of a pair: F = Va + i Vb with
 // Vx(G) = v_H(G) - i G . d_x(G), v_H = 4 pi RT / G^2 (RT = rho_tot(G), scaled), the d_x
 // unpacked from the forward transforms Da (x, y of a), Db (x, y of b), Dz (z of a and b),
-// unscaled; without gradients Va = Vb = v_H.  Hartree sum of rho_tot into partial row 0.
-template <typename TD>
-__global__ void k_assemble_pair(const double2* __restrict__ RT, const cplx<TD>* __restrict__ Da,
-                                const cplx<TD>* __restrict__ Db, const cplx<TD>* __restrict__ Dz, int has_b,
-                                cplx<TD>* __restrict__ F, GridDims g, CellDev c, double inv_nr, double* partial) {
-  const long long nr = (long long)g.n1 * g.n2 * g.n3;
+// unscaled; without gradients Va = Vb = v_H.  Hartree sum of rho_tot into partial row 0 (SUMS).
+// FP32 grids are widened and the result narrowed on the bit patterns (dd.cuh).
+__device__ __forceinline__ double2 wide2(double2 v) { return v; }
+__device__ __forceinline__ double2 wide2(float2 v) {
+  return make_double2(float_to_double_bits(v.x), float_to_double_bits(v.y));
+}
+template <typename TD, bool SUMS>
+__global__ void __launch_bounds__(kRedThreads)
+k_assemble_pair(const double2* __restrict__ RT, const cplx<TD>* __restrict__ Da, const cplx<TD>* __restrict__ Db,
+                const cplx<TD>* __restrict__ Dz, int has_b, cplx<TD>* __restrict__ F, GridDims g, CellDev c,
+                double inv_nr, double* partial) {
+  __shared__ GTables tab;
+  fill_tables(tab, g, c);
+  const int end = pair_end(g);
+  const double s = 0.5 * inv_nr;
   double eh = 0;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < nr; idx += (long long)gridDim.x * blockDim.x) {
-    const Gpt p = gvec(idx, g, c);
-    double2 vh = make_double2(0, 0);
-    if (p.g2 > 0 && !p.nyq) {
-      const double f = 4.0 * M_PI / p.g2;
-      const double2 r = RT[idx];
-      vh = make_double2(f * r.x, f * r.y);
-      eh += f * (r.x * r.x + r.y * r.y);
-    }
-    double2 va = vh, vb = vh;
-    if (Da && !p.nyq) {
-      const long long jn = neg_index(idx, g);
-      double2 ax, ay, az, bx = make_double2(0, 0), by = make_double2(0, 0), bz = make_double2(0, 0);
-      unpack2(to_d2(Da[idx]), to_d2(Da[jn]), &ax, &ay);
-      if (has_b) {
-        unpack2(to_d2(Db[idx]), to_d2(Db[jn]), &bx, &by);
-        unpack2(to_d2(Dz[idx]), to_d2(Dz[jn]), &az, &bz);
-      } else {
-        const double2 t = to_d2(Dz[idx]), tn = to_d2(Dz[jn]);
-        az = make_double2(0.5 * (t.x + tn.x), 0.5 * (t.y - tn.y));
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < end; idx += gridDim.x * blockDim.x) {
+    GPair p;
+    if (!pair_point(idx, g, tab, &p)) continue;
+    double2 va = make_double2(0, 0), vb = va;
+    if (!p.nyq) {
+      if (p.g2 > 0) {
+        const double f = 4.0 * M_PI / p.g2;
+        const double2 r = RT[p.idx];
+        va = make_double2(f * r.x, f * r.y);
+        if (SUMS) eh += (p.idx == p.jn ? 1.0 : 2.0) * f * (r.x * r.x + r.y * r.y);
       }
-      // i G . d / N_r
-      const double dar = p.gx * ax.x + p.gy * ay.x + p.gz * az.x, dai = p.gx * ax.y + p.gy * ay.y + p.gz * az.y;
-      const double dbr = p.gx * bx.x + p.gy * by.x + p.gz * bz.x, dbi = p.gx * bx.y + p.gy * by.y + p.gz * bz.y;
-      va = make_double2(vh.x + dai * inv_nr, vh.y - dar * inv_nr);
-      vb = make_double2(vh.x + dbi * inv_nr, vh.y - dbr * inv_nr);
+      vb = va;
+      if (Da) {
+        // G . d of both fields at G (twice the unpacked values): x and y of a in Da, of b in Db, z in Dz
+        const double2 u = wide2(Da[p.idx]), un = wide2(Da[p.jn]), z = wide2(Dz[p.idx]), zn = wide2(Dz[p.jn]);
+        const double dar = p.gx * (u.x + un.x) + p.gy * (u.y + un.y) + p.gz * (z.x + zn.x);
+        const double dai = p.gx * (u.y - un.y) + p.gy * (un.x - u.x) + p.gz * (z.y - zn.y);
+        va = make_double2(va.x + dai * s, va.y - dar * s);
+        if (has_b) {
+          const double2 w = wide2(Db[p.idx]), wn = wide2(Db[p.jn]);
+          const double dbr = p.gx * (w.x + wn.x) + p.gy * (w.y + wn.y) + p.gz * (z.y + zn.y);
+          const double dbi = p.gx * (w.y - wn.y) + p.gy * (wn.x - w.x) + p.gz * (zn.x - z.x);
+          vb = make_double2(vb.x + dbi * s, vb.y - dbr * s);
+        }
+      }
     }
     if (F) {
-      const double2 o = has_b ? pack2(va, vb) : va;
-      F[idx] = mk<TD>((TD)o.x, (TD)o.y);
+      // V(-G) = conj V(G)
+      if (has_b) {
+        F[p.idx] = mk<TD>(narrow<TD>(va.x - vb.y), narrow<TD>(va.y + vb.x));
+        F[p.jn] = mk<TD>(narrow<TD>(va.x + vb.y), narrow<TD>(vb.x - va.y));
+      } else {
+        F[p.idx] = mk<TD>(narrow<TD>(va.x), narrow<TD>(va.y));
+        F[p.jn] = mk<TD>(narrow<TD>(va.x), narrow<TD>(-va.y));
+      }
     }
   }
-  if (partial) block_sum_store(eh, partial + blockIdx.x);
+  if (SUMS) block_sum_store(eh, partial + blockIdx.x);
 }
 
-// veff_x = vloc + Re/Im F (inverse-transformed reciprocal part) + w_x for the pair's
-// subsystems (either output may be NULL).
+// veff_x = vloc + Re/Im F (inverse-transformed reciprocal part) + w_x for the pair's subsystems (either
+// output may be NULL), checked for non-finite values, with the plane-major copy [i3][i1][i2] of the plane
+// pass of H psi in the working precision (transposed through shared memory): one pass over the grid
+// where the sum, the check and the transposition of each subsystem took five.
 template <typename TD>
-__global__ void k_finish_pair(const cplx<TD>* __restrict__ F, const double* __restrict__ vloc, double* va,
-                              double* vb, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const double2 f = to_d2(F[i]);
-    const double vl = vloc[i];
-    if (va) va[i] = vl + f.x + va[i];
-    if (vb) vb[i] = vl + f.y + vb[i];
+__global__ void __launch_bounds__(256)
+k_finish_pair(const cplx<TD>* __restrict__ F, const double* __restrict__ vloc, double* __restrict__ va,
+              double* __restrict__ vb, TD* __restrict__ pa, TD* __restrict__ pb, int rows, int n3, unsigned* status) {
+  __shared__ TD ta[32][33], tb[32][33];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+  bool bad = false;
+  for (int j = y; j < 32; j += 8) {
+    const int r = r0 + j, c = c0 + x;
+    if (r < rows && c < n3) {
+      const int i = r * n3 + c;
+      const cplx<TD> f = F[i];
+      const double vl = vloc[i];
+      if (va) {
+        const double v = vl + widen(f.x) + va[i];
+        va[i] = v;
+        bad |= !isfinite(v);
+        ta[j][x] = narrow<TD>(v);
+      }
+      if (vb) {
+        const double v = vl + widen(f.y) + vb[i];
+        vb[i] = v;
+        bad |= !isfinite(v);
+        tb[j][x] = narrow<TD>(v);
+      }
+    }
+  }
+  if (bad) atomicOr(status, ST_NONFINITE);
+  __syncthreads();
+  for (int j = y; j < 32; j += 8) {
+    const int c = c0 + j, r = r0 + x;
+    if (r < rows && c < n3) {
+      if (va) pa[(size_t)c * rows + r] = ta[x][j];
+      if (vb) pb[(size_t)c * rows + r] = tb[x][j];
+    }
+  }
+}
+
+// out (+)= sum of n grids.
+__global__ void k_sum_grids(GridList l, int n, int accumulate, double* __restrict__ out, long long nr) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nr; i += (long long)gridDim.x * blockDim.x) {
+    double v = accumulate ? out[i] : l.p[0][i];
+    for (int k = accumulate ? 0 : 1; k < n; ++k) v += l.p[k][i];
+    out[i] = v;
   }
 }
 
@@ -749,8 +843,11 @@ void grid_unpack_density(const double2* C, int has_b, double2* RT, int accumulat
                          double2* Pz, const GridDims& g, const CellDev& c, double* partial, cudaStream_t st) {
   count_launches(1);
   ProfScope prof_("k_unpack_density", st);
-  k_unpack_density<<<kRedBlocks, kRedThreads, 0, st>>>(C, has_b, RT, accumulate, Pa, Pb, Pz, g, c,
-                                                       1.0 / ((double)g.n1 * g.n2 * g.n3), partial);
+  const double inv = 1.0 / ((double)g.n1 * g.n2 * g.n3);
+  if (partial)
+    k_unpack_density<true><<<kRedBlocks, kRedThreads, 0, st>>>(C, has_b, RT, accumulate, Pa, Pb, Pz, g, c, inv, partial);
+  else
+    k_unpack_density<false><<<kRedBlocks, kRedThreads, 0, st>>>(C, has_b, RT, accumulate, Pa, Pb, Pz, g, c, inv, nullptr);
 }
 void grid_pw_total(const double* rho, const GradPacks& gp, int xc_mode, int kedf, double rho_cut, double* vpart,
                    double* hx, double* hy, double* hz, long long nr, double* partial, bool fp32, cudaStream_t st) {
@@ -778,14 +875,25 @@ void grid_assemble_pair(const double2* RT, const cplx<TD>* Da, const cplx<TD>* D
                         cplx<TD>* F, const GridDims& g, const CellDev& c, double* partial, cudaStream_t st) {
   count_launches(1);
   ProfScope prof_("k_assemble_pair", st);
-  k_assemble_pair<TD><<<kRedBlocks, kRedThreads, 0, st>>>(RT, Da, Db, Dz, has_b, F, g, c,
-                                                          1.0 / ((double)g.n1 * g.n2 * g.n3), partial);
+  const double inv = 1.0 / ((double)g.n1 * g.n2 * g.n3);
+  if (partial)
+    k_assemble_pair<TD, true><<<kRedBlocks, kRedThreads, 0, st>>>(RT, Da, Db, Dz, has_b, F, g, c, inv, partial);
+  else
+    k_assemble_pair<TD, false><<<kRedBlocks, kRedThreads, 0, st>>>(RT, Da, Db, Dz, has_b, F, g, c, inv, nullptr);
 }
 template <typename TD>
-void grid_finish_pair(const cplx<TD>* F, const double* vloc, double* va, double* vb, long long n, cudaStream_t st) {
+void grid_finish_pair(const cplx<TD>* F, const double* vloc, double* va, double* vb, TD* pa, TD* pb, const GridDims& g,
+                      unsigned* status, cudaStream_t st) {
+  const int rows = g.n1 * g.n2;
   count_launches(1);
   ProfScope prof_("k_finish_pair", st);
-  k_finish_pair<TD><<<gs(n), 256, 0, st>>>(F, vloc, va, vb, n);
+  k_finish_pair<TD><<<dim3(ceil_div(g.n3, 32), ceil_div(rows, 32)), 256, 0, st>>>(F, vloc, va, vb, pa, pb, rows, g.n3,
+                                                                                  status);
+}
+void grid_sum(const GridList& l, int n, bool accumulate, double* out, long long nr, cudaStream_t st) {
+  count_launches(1);
+  ProfScope prof_("k_combine", st);
+  k_sum_grids<<<gs(nr), 256, 0, st>>>(l, n, accumulate ? 1 : 0, out, nr);
 }
 int grid_red_blocks() { return kRedBlocks; }
 
@@ -800,7 +908,8 @@ int grid_red_blocks() { return kRedBlocks; }
                                 cudaStream_t);                                                                 \
   template void grid_assemble_pair<T>(const double2*, const cplx<T>*, const cplx<T>*, const cplx<T>*, int,      \
                                       cplx<T>*, const GridDims&, const CellDev&, double*, cudaStream_t);        \
-  template void grid_finish_pair<T>(const cplx<T>*, const double*, double*, double*, long long, cudaStream_t);
+  template void grid_finish_pair<T>(const cplx<T>*, const double*, double*, double*, T*, T*, const GridDims&,   \
+                                    unsigned*, cudaStream_t);
 FDE_GRID_INST(float)
 FDE_GRID_INST(double)
 

@@ -62,7 +62,14 @@ void grid_pw_pair(const double* ra, const double* rb, const double2* Pa, const d
 template <typename TD>
 void grid_assemble_pair(const double2* RT, const cplx<TD>* Da, const cplx<TD>* Db, const cplx<TD>* Dz, int has_b,
                         cplx<TD>* F, const GridDims& g, const CellDev& c, double* partial, cudaStream_t st);
+// pa, pb: plane-major copies [n3][n1][n2] of the potentials va, vb (each given with its potential).
 template <typename TD>
-void grid_finish_pair(const cplx<TD>* F, const double* vloc, double* va, double* vb, long long n, cudaStream_t st);
+void grid_finish_pair(const cplx<TD>* F, const double* vloc, double* va, double* vb, TD* pa, TD* pb, const GridDims& g,
+                      unsigned* status, cudaStream_t st);
+// out = sum of n grids (out += with accumulate).
+struct GridList {
+  const double* p[64];
+};
+void grid_sum(const GridList& l, int n, bool accumulate, double* out, long long nr, cudaStream_t st);
 
 }  // namespace fde

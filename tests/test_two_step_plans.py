@@ -12,8 +12,17 @@ import numpy as np
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1406_7803_gb300", "csrc")
-PLANS = [tuple(map(int, m)) for m in re.findall(r"X\((\d+), (\d+), (\d+)\)", open(os.path.join(CSRC, "fft2.cuh")).read())]
-SIDES = [p[0] for p in PLANS if p[0] <= 160]
+TEXT = open(os.path.join(CSRC, "fft2.cuh")).read()
+
+
+def plans(prefix):
+    lines = re.findall(r"#define %s\d\(X\)((?:.*\\\n)*.*)" % prefix, TEXT)
+    return [tuple(map(int, m)) for line in lines for m in re.findall(r"X\((\d+), (\d+), (\d+)\)", line)]
+
+
+LINES = plans("FDE_SPLIT_SIDES") + plans("FDE_SPLIT_LONG")   # (N, A, B), A <= B: z lines
+PLANES = plans("FDE_PLANE_SIDES")                            # (N, R1, R2), R1 >= R2: plane sides, strided axes
+SIDES = [p[0] for p in PLANES]
 
 
 def dft(x, sign):
@@ -21,30 +30,53 @@ def dft(x, sign):
     return np.exp(sign * 2j * np.pi * np.outer(k, k) / len(x)) @ x
 
 
-@pytest.mark.parametrize("n,a,b", PLANS)
-def test_two_steps_are_the_transform_and_its_reverse(n, a, b):
-    assert n == a * b and a <= b
+def indices(n, r1, r2, prime_factor):
+    """Input index of (item j, element r) and output index of (item q, element p)."""
+    if not prime_factor:
+        return (lambda j, r: j + r2 * r), (lambda q, p: q + r1 * p)
+    e1 = next(k for k in range(n) if k % r1 == 1 % r1 and k % r2 == 0)
+    e2 = next(k for k in range(n) if k % r1 == 0 and k % r2 == 1 % r2)
+    return (lambda j, r: (r1 * j + r2 * r) % n), (lambda q, p: (q * e1 + p * e2) % n)
+
+
+def check(n, r1, r2, prime_factor):
     rng = np.random.default_rng(n)
     x = rng.standard_normal(n) + 1j * rng.standard_normal(n)
     v = rng.standard_normal(n)
-    for r1, r2 in ((a, b), (b, a)):
-        j, q = np.arange(r2)[:, None], np.arange(r1)[None, :]
-        tw = np.exp(-2j * np.pi * j * q / n)
-        # inverse: item j takes j + r2 r, item q ends on q + r1 p
-        A = np.array([dft(x[i::r2], +1) for i in range(r2)]) * tw.conj()
-        y = np.array([dft(A[:, i], +1) for i in range(r1)])  # [q][p]
-        flat = np.empty(n, dtype=complex)
-        for i in range(r1):
-            flat[i::r1] = y[i]
-        want = np.fft.ifft(x) * n
-        assert np.abs(flat - want).max() < 1e-12 * np.abs(want).max()
-        # product on the same registers, then the forward transform backwards through the steps
-        B = np.array([dft(y[i] * v[i::r1], -1) for i in range(r1)]).T * tw  # [j][q]
-        out = np.empty(n, dtype=complex)
-        for i in range(r2):
-            out[i::r2] = dft(B[i], -1)
-        want = np.fft.fft(want * v)
-        assert np.abs(out - want).max() < 1e-12 * np.abs(want).max()
+    at, to = indices(n, r1, r2, prime_factor)
+    ins = np.array([[at(j, r) for r in range(r1)] for j in range(r2)])
+    outs = np.array([[to(q, p) for p in range(r2)] for q in range(r1)])
+    assert sorted(ins.ravel()) == sorted(outs.ravel()) == list(range(n))
+    j, q = np.arange(r2)[:, None], np.arange(r1)[None, :]
+    tw = np.ones((r2, r1)) if prime_factor else np.exp(-2j * np.pi * j * q / n)
+    A = np.array([dft(x[i], +1) for i in ins]) * tw.conj()          # [j][q]
+    y = np.array([dft(A[:, i], +1) for i in range(r1)])             # [q][p]
+    flat = np.empty(n, dtype=complex)
+    flat[outs] = y
+    want = np.fft.ifft(x) * n
+    assert np.abs(flat - want).max() < 1e-12 * np.abs(want).max()
+    # product on the same registers, then the forward transform backwards through the steps
+    B = np.array([dft(y[i] * v[outs[i]], -1) for i in range(r1)]).T * tw
+    out = np.empty(n, dtype=complex)
+    out[ins] = np.array([dft(B[i], -1) for i in range(r2)])
+    want = np.fft.fft(want * v)
+    assert np.abs(out - want).max() < 1e-12 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("n,a,b", LINES)
+def test_line_plans(n, a, b):
+    assert n == a * b and a <= b
+    check(n, a, b, False)
+
+
+@pytest.mark.parametrize("n,r1,r2", PLANES)
+def test_side_plans(n, r1, r2):
+    assert n == r1 * r2 and r1 >= r2
+    check(n, r1, r2, np.gcd(r1, r2) == 1)
+
+
+def test_every_side_is_a_line_too():
+    assert sorted(SIDES) == sorted(n for n, _, _ in plans("FDE_SPLIT_SIDES"))
 
 
 gpu = pytest.mark.gpu
