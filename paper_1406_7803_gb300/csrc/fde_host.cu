@@ -614,8 +614,8 @@ template <typename T> struct EngineT : Engine {
     launch_fft3d<double>(x, g, plans64.fp, sign, st);
   }
 
-  // Divergence-argument grid c of pair q in the working precision: the packed gradient grid
-  // itself (overwritten in place) in FP64 contexts, a separate FP32 grid in mixed ones.
+  // Gradient (then divergence-argument) grid c of pair q in the working precision: the packed grid
+  // itself in FP64 contexts, a separate FP32 grid in mixed ones.
   std::vector<DBuf<cplx<T>>> dpacks;
   DBuf<cplx<T>> fpot;
   cplx<T>* dgrid(int q, int c, double2* packed) {
@@ -629,6 +629,16 @@ template <typename T> struct EngineT : Engine {
       return b.p;
     }
   }
+  // A gradient's transform x (FP64, destroyed) into its grid in the working precision.
+  void fft_gradient(double2* x, cplx<T>* out) {
+    if constexpr (sizeof(T) == 4) {
+      if (launch_fft3d_dd(x, g, plansdd.fp, +1, st, out)) return;
+      launch_fft3d<double>(x, g, plans64.fp, +1, st);
+      grid_narrow(x, out, nr, st);
+    } else {
+      launch_fft3d<double>(x, g, plans64.fp, +1, st);
+    }
+  }
   // Reciprocal-space potentials of a pair (the packed transform grid in FP64 contexts).
   cplx<T>* fgrid() {
     if constexpr (sizeof(T) == 8) {
@@ -639,8 +649,10 @@ template <typename T> struct EngineT : Engine {
     }
   }
 
-  // Packed gradient grids of subsystem pair q (three complex grids).
+  // Packed gradient transforms of subsystem pair q (three complex grids; in mixed contexts work space of
+  // one pair's transforms, whose results are FP32 grids).
   double2* pack(int q, int c) {
+    if constexpr (sizeof(T) == 4) q = 0;
     const size_t need = (size_t)3 * (q + 1);
     if (packs.size() < need) packs.resize(need);
     DBuf<double2>& b = packs[(size_t)3 * q + c];
@@ -674,7 +686,7 @@ template <typename T> struct EngineT : Engine {
     double2* RT = cb[1].p;
     sum_densities();
     // 1. densities to reciprocal space, total density, Hartree sums and gradients
-    GradPacks gp{};
+    GradPacks<T> gp{};
     gp.npairs = grad ? npairs : 0;
     for (int q = 0; q < npairs; ++q) {
       const int ia = 2 * q, ib = 2 * q + 1;
@@ -690,19 +702,21 @@ template <typename T> struct EngineT : Engine {
         if (hb) grid_finalize(partial.p + nrb, 1, 0.5 * omega, scal.p + 4 + 3 * ib, st);
       }
       if (grad) {
-        fft_density(Pa, +1);
-        if (hb) fft_density(Pb, +1);
-        fft_density(Pz, +1);
-        gp.a[q] = Pa;
-        gp.b[q] = Pb;
-        gp.z[q] = Pz;
+        cplx<T>* Ga = dgrid(q, 0, Pa);
+        cplx<T>* Gb = hb ? dgrid(q, 1, Pb) : nullptr;
+        cplx<T>* Gz = dgrid(q, 2, Pz);
+        fft_gradient(Pa, Ga);
+        if (hb) fft_gradient(Pb, Gb);
+        fft_gradient(Pz, Gz);
+        gp.a[q] = Ga;
+        gp.b[q] = Gb;
+        gp.z[q] = Gz;
         gp.has_b[q] = hb ? 1 : 0;
       }
     }
     // 2. functionals of the total density
-    grid_pw_total(rho_tot.p, gp, func.xc, func.kedf, func.rho_cut, want_pot ? vpart.p : nullptr,
-                  (want_pot && grad) ? htot[0].p : nullptr, htot[1].p, htot[2].p, nr, partial.p, sizeof(T) == 4,
-                  st);
+    grid_pw_total<T>(rho_tot.p, gp, func.xc, func.kedf, func.rho_cut, want_pot ? vpart.p : nullptr,
+                     (want_pot && grad) ? htot[0].p : nullptr, htot[1].p, htot[2].p, nr, partial.p, st);
     if (want_e) {  // the pointwise kernels always leave their block sums; reduce them only when asked
       grid_finalize(partial.p, 2, dv, scal.p + 1, st);
       grid_dot_partial(vloc.p, rho_tot.p, nr, 0, partial.p, st);
@@ -725,13 +739,13 @@ template <typename T> struct EngineT : Engine {
       double2* Pb = (grad && hb) ? pack(q, 1) : nullptr;
       double2* Pz = grad ? pack(q, 2) : nullptr;
       const bool pot = pa || pb;
-      // divergence arguments, reciprocal-space potentials and their transforms in the working
-      // precision (FP32 in mixed contexts: they enter V_eff linearly, unlike the gradients)
+      // divergence arguments (over the gradients), reciprocal-space potentials and their transforms in
+      // the working precision
       cplx<T>* Da = grad ? dgrid(q, 0, Pa) : nullptr;
       cplx<T>* Db = (grad && hb) ? dgrid(q, 1, Pb) : nullptr;
       cplx<T>* Dz = grad ? dgrid(q, 2, Pz) : nullptr;
       cplx<T>* F = fgrid();
-      grid_pw_pair<T>(A.rho.p, B ? B->rho.p : nullptr, Pa, Pb, Pz, Da, Db, Dz, htot[0].p, htot[1].p, htot[2].p,
+      grid_pw_pair<T>(A.rho.p, B ? B->rho.p : nullptr, Da, Db, Dz, htot[0].p, htot[1].p, htot[2].p,
                       want_pot ? vpart.p : nullptr, want_e ? func.xc : -1, func.kedf, func.rho_cut,
                       pa ? A.veff.p : nullptr, pb ? B->veff.p : nullptr, (pot && grad) ? 1 : 0, nr, partial.p, st);
       if (want_e) {

@@ -21,10 +21,18 @@ template <typename C> __host__ __device__ constexpr int ax_lines() { return 16; 
 template <typename C, int R1, int R2> __host__ __device__ constexpr int ax_threads() {
   return round_up(ax_lines<C>() * (R1 > R2 ? R1 : R2), 32);
 }
+// Lines and threads of a CTA of the contiguous axis: one round of items.  (256 threads for the 120
+// items of eight double-float lines held 8 of 15 warps a CTA at its barrier: 70 us for 180-point lines
+// of 72 x 72 x 180.)
+template <typename C> __host__ __device__ constexpr int ctg_lines() { return sizeof(C) == 8 ? 16 : 8; }
+template <typename C, int R1, int R2> __host__ __device__ constexpr int ctg_threads() {
+  return round_up(ctg_lines<C>() * (R1 > R2 ? R1 : R2), 32);
+}
 
 // Global forms of the grid a pass reads and writes.
 struct AsIs {};  // values of the transform's own type
 struct AsF64 {}; // FP64 values of a double-float transform: split on reading, joined on writing
+struct AsHigh {};  // FP32: the high parts (a normalised double-float rounded to FP32)
 template <typename C> __device__ __forceinline__ C ax_get(const void* p, int i, AsIs) {
   return reinterpret_cast<const C*>(p)[i];
 }
@@ -44,6 +52,9 @@ template <typename C> __device__ __forceinline__ ddc ax_get(const void* p, int i
 template <typename C> __device__ __forceinline__ void ax_put(void* p, int i, C v, AsIs) {
   reinterpret_cast<C*>(p)[i] = v;
 }
+template <typename C> __device__ __forceinline__ void ax_put(void* p, int i, ddc v, AsHigh) {
+  reinterpret_cast<float2*>(p)[i] = make_float2(v.x.hi, v.y.hi);
+}
 template <typename C> __device__ __forceinline__ void ax_put(void* p, int i, ddc v, AsF64) {
   reinterpret_cast<double2*>(p)[i] = make_double2(dd_to_double(v.x), dd_to_double(v.y));
 }
@@ -52,7 +63,7 @@ template <typename C> __device__ __forceinline__ void ax_put(void* p, int i, ddc
 // (prime-factor indices where it has coprime factors: no twiddles).
 template <typename T, typename Plan, typename IN, typename OUT>
 __global__ void __launch_bounds__(ax_threads<cplx<T>, Plan::R1, Plan::R2>())
-k_fft_strided(void* __restrict__ data, int nlines, int stride, const cplx<T>* __restrict__ tw, bool conj) {
+k_fft_strided(const void* data, void* out, int nlines, int stride, const cplx<T>* __restrict__ tw, bool conj) {
   using C = cplx<T>;
   constexpr int R1 = Plan::R1, R2 = Plan::R2, N = Plan::N, L = ax_lines<C>(), NT = ax_threads<C, R1, R2>();
   __shared__ __align__(16) C X[N * L];
@@ -81,17 +92,17 @@ k_fft_strided(void* __restrict__ data, int nlines, int stride, const cplx<T>* __
     }
     dft_r<R2>(v, -1);
 #pragma unroll
-    for (int p = 0; p < R2; ++p) ax_put<C>(data, base + Plan::output(i, p) * stride, ax_conj(v[p], conj), OUT());
+    for (int p = 0; p < R2; ++p) ax_put<C>(out, base + Plan::output(i, p) * stride, ax_conj(v[p], conj), OUT());
   }
 }
 
 // Contiguous axis: line l at l N.  The exchange pads each run of R2 values to an odd length, so
 // that step 2's lanes (neighbouring q) lie on different banks.
 template <typename T, int R1, int R2, typename IN, typename OUT>
-__global__ void __launch_bounds__(ax_threads<cplx<T>, R1, R2>())
+__global__ void __launch_bounds__(ctg_threads<cplx<T>, R1, R2>())
 k_fft_contig(void* __restrict__ data, int nlines, const cplx<T>* __restrict__ tw, bool conj) {
   using C = cplx<T>;
-  constexpr int N = R1 * R2, L = sizeof(C) == 8 ? 16 : 8, NT = ax_threads<C, R1, R2>(), RP = R2 | 1, XP = R1 * RP | 1;
+  constexpr int N = R1 * R2, L = ctg_lines<C>(), NT = ctg_threads<C, R1, R2>(), RP = R2 | 1, XP = R1 * RP | 1;
   __shared__ __align__(16) C X[L * XP];
   const int l0 = blockIdx.x * L;
   for (int w = threadIdx.x; w < L * R2; w += NT) {
@@ -127,7 +138,7 @@ k_fft_contig(void* __restrict__ data, int nlines, const cplx<T>* __restrict__ tw
 // One pass over the lengths of LIST; false when n is none of them.
 #define FDE_AXIS_LAUNCHERS(SIDES, LINES)                                                                          \
   template <typename T, typename IN, typename OUT>                                                               \
-  bool strided_axis(int n, long long nlines, int stride, void* data, const cplx<T>* tw, int sign,                \
+  bool strided_axis(int n, long long nlines, int stride, void* data, void* out, const cplx<T>* tw, int sign,     \
                     cudaStream_t st) {                                                                            \
     const unsigned blocks = (unsigned)ceil_div(nlines, ax_lines<cplx<T>>());                                      \
     switch (n) { SIDES(FDE_STRIDED_CASE) }                                                                        \
@@ -135,7 +146,7 @@ k_fft_contig(void* __restrict__ data, int nlines, const cplx<T>* __restrict__ tw
   }                                                                                                               \
   template <typename T, typename IN, typename OUT>                                                               \
   bool contig_axis(int n, long long nlines, void* data, const cplx<T>* tw, int sign, cudaStream_t st) {          \
-    const unsigned blocks = (unsigned)ceil_div(nlines, sizeof(cplx<T>) == 8 ? 16 : 8);                            \
+    const unsigned blocks = (unsigned)ceil_div(nlines, ctg_lines<cplx<T>>());                                     \
     switch (n) { LINES(FDE_CONTIG_CASE) }                                                                         \
     return false;                                                                                                 \
   }
@@ -143,12 +154,12 @@ k_fft_contig(void* __restrict__ data, int nlines, const cplx<T>* __restrict__ tw
   case N:                                                                                                         \
     count_launches(1);                                                                                            \
     k_fft_strided<T, SidePlan<R1, R2>, IN, OUT><<<blocks, ax_threads<cplx<T>, R1, R2>(), 0, st>>>(               \
-        data, (int)nlines, stride, tw, sign > 0);                                                                 \
+        data, out, (int)nlines, stride, tw, sign > 0);                                                            \
     return true;
 #define FDE_CONTIG_CASE(N, R1, R2)                                                                                \
   case N:                                                                                                         \
     count_launches(1);                                                                                            \
-    k_fft_contig<T, R1, R2, IN, OUT><<<blocks, ax_threads<cplx<T>, R1, R2>(), 0, st>>>(data, (int)nlines, tw,    \
+    k_fft_contig<T, R1, R2, IN, OUT><<<blocks, ctg_threads<cplx<T>, R1, R2>(), 0, st>>>(data, (int)nlines, tw,   \
                                                                                         sign > 0);               \
     return true;
 

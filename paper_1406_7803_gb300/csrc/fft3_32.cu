@@ -13,8 +13,8 @@ bool launch_fft3d_two_step<float>(cplx<float>* data, const GridDims& g, const Ff
   ProfScope prof_("k_fft_axis_f32", st);
   const long long nr = (long long)g.n1 * g.n2 * g.n3;
   contig_axis<float, AsIs, AsIs>(g.n3, nr / g.n3, data, fp.p3.tw, sign, st);
-  strided_axis<float, AsIs, AsIs>(g.n2, nr / g.n2, g.n3, data, fp.p2.tw, sign, st);
-  strided_axis<float, AsIs, AsIs>(g.n1, nr / g.n1, g.n2 * g.n3, data, fp.p1.tw, sign, st);
+  strided_axis<float, AsIs, AsIs>(g.n2, nr / g.n2, g.n3, data, data, fp.p2.tw, sign, st);
+  strided_axis<float, AsIs, AsIs>(g.n1, nr / g.n1, g.n2 * g.n3, data, data, fp.p1.tw, sign, st);
   return true;
 }
 

@@ -493,22 +493,22 @@ k_unpack_density(const double2* __restrict__ C, int has_b, double2* __restrict__
 // h = (d f / d grad rho) in hx, hy, hz (real; when there are gradients); energy partial rows
 // 0 (xc) and 1 (kinetic).
 template <typename R>
-__global__ void k_pw_total(const double* __restrict__ rho, GradPacks gp, int xc_mode, int kedf, double rho_cut,
+__global__ void k_pw_total(const double* __restrict__ rho, GradPacks<R> gp, int xc_mode, int kedf, double rho_cut,
                            double* __restrict__ vpart, double* __restrict__ hx, double* __restrict__ hy,
                            double* __restrict__ hz, long long nr, double* partial) {
   double ax = 0, ak = 0;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < nr; idx += (long long)gridDim.x * blockDim.x) {
     R x = 0, y = 0, z = 0;
     for (int q = 0; q < gp.npairs; ++q) {
-      const double2 pa = gp.a[q][idx], pz = gp.z[q][idx];
-      x += narrow<R>(pa.x);
-      y += narrow<R>(pa.y);
-      z += narrow<R>(pz.x);
+      const cplx<R> pa = gp.a[q][idx], pz = gp.z[q][idx];
+      x += pa.x;
+      y += pa.y;
+      z += pz.x;
       if (gp.has_b[q]) {
-        const double2 pb = gp.b[q][idx];
-        x += narrow<R>(pb.x);
-        y += narrow<R>(pb.y);
-        z += narrow<R>(pz.y);
+        const cplx<R> pb = gp.b[q][idx];
+        x += pb.x;
+        y += pb.y;
+        z += pz.y;
       }
     }
     R v, h, ex, ek;
@@ -530,11 +530,10 @@ __global__ void k_pw_total(const double* __restrict__ rho, GradPacks gp, int xc_
 // pair: w_x = vpart_tot - d f_kin / d rho_x (the pointwise part of v~_kin[rho] - v~_kin[rho_x]
 // with the xc part of the total), and, in place of the packed gradients, the packed
 // divergence arguments d_x = h_tot - h_x.  Energy partial rows 0/1 (xc/kin of a), 2/3 (b).
-// The divergence arguments go to Da, Db, Dz in precision TD (FP64: in place over Pa, Pb, Pz;
-// FP32: separate grids for the single-precision transforms of the mixed path).
+// Gradients and divergence arguments are in the working precision; the latter take the former's place.
 template <typename TD>
-__global__ void k_pw_pair(const double* __restrict__ ra, const double* __restrict__ rb, const double2* Pa,
-                          const double2* Pb, const double2* Pz, cplx<TD>* Da, cplx<TD>* Db, cplx<TD>* Dz,
+__global__ void k_pw_pair(const double* __restrict__ ra, const double* __restrict__ rb, cplx<TD>* Pa, cplx<TD>* Pb,
+                          cplx<TD>* Pz,
                           const double* __restrict__ hx, const double* __restrict__ hy,
                           const double* __restrict__ hz, const double* __restrict__ vtot, int xc_mode, int kedf,
                           double rho_cut, double* __restrict__ wa, double* __restrict__ wb, int write_d, long long nr,
@@ -542,14 +541,13 @@ __global__ void k_pw_pair(const double* __restrict__ ra, const double* __restric
   double xa = 0, ka = 0, xb = 0, kb = 0;
   const bool has_b = rb != nullptr;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < nr; idx += (long long)gridDim.x * blockDim.x) {
-    double2 pa = make_double2(0, 0), pb = make_double2(0, 0), pz = make_double2(0, 0);
+    cplx<TD> pa = mk<TD>(0, 0), pb = mk<TD>(0, 0), pz = mk<TD>(0, 0);
     if (Pa) {
       pa = Pa[idx];
       pz = Pz[idx];
       if (has_b) pb = Pb[idx];
     }
-    const TD pax = narrow<TD>(pa.x), pay = narrow<TD>(pa.y), pzx = narrow<TD>(pz.x);
-    const TD pbx = narrow<TD>(pb.x), pby = narrow<TD>(pb.y), pzy = narrow<TD>(pz.y);
+    const TD pax = pa.x, pay = pa.y, pzx = pz.x, pbx = pb.x, pby = pb.y, pzy = pz.y;
     TD va, ha, ex, ek;
     point_functional<TD>(narrow<TD>(ra[idx]), pax, pay, pzx, xc_mode, 0, kedf, (TD)rho_cut, &va, &ha, &ex, &ek);
     xa += widen(ex);
@@ -565,9 +563,9 @@ __global__ void k_pw_pair(const double* __restrict__ ra, const double* __restric
     if (wb) wb[idx] = widen(vt - vb);
     if (write_d) {
       const TD tx = narrow<TD>(hx[idx]), ty = narrow<TD>(hy[idx]), tz = narrow<TD>(hz[idx]);
-      Da[idx] = mk<TD>(tx - ha * pax, ty - ha * pay);
-      if (has_b) Db[idx] = mk<TD>(tx - hb * pbx, ty - hb * pby);
-      Dz[idx] = mk<TD>(tz - ha * pzx, has_b ? tz - hb * pzy : TD(0));
+      Pa[idx] = mk<TD>(tx - ha * pax, ty - ha * pay);
+      if (has_b) Pb[idx] = mk<TD>(tx - hb * pbx, ty - hb * pby);
+      Pz[idx] = mk<TD>(tz - ha * pzx, has_b ? tz - hb * pzy : TD(0));
     }
   }
   block_sum_store(xa, partial + blockIdx.x);
@@ -580,15 +578,10 @@ __global__ void k_pw_pair(const double* __restrict__ ra, const double* __restric
 // Vx(G) = v_H(G) - i G . d_x(G), v_H = 4 pi RT / G^2 (RT = rho_tot(G), scaled), the d_x
 // unpacked from the forward transforms Da (x, y of a), Db (x, y of b), Dz (z of a and b),
 // unscaled; without gradients Va = Vb = v_H.  Hartree sum of rho_tot into partial row 0 (SUMS).
-// FP32 grids are widened and the result narrowed on the bit patterns (dd.cuh).
-__device__ __forceinline__ double2 wide2(double2 v) { return v; }
-__device__ __forceinline__ double2 wide2(float2 v) {
-  return make_double2(float_to_double_bits(v.x), float_to_double_bits(v.y));
-}
-template <typename TD, bool SUMS>
+template <bool SUMS>
 __global__ void __launch_bounds__(kRedThreads)
-k_assemble_pair(const double2* __restrict__ RT, const cplx<TD>* __restrict__ Da, const cplx<TD>* __restrict__ Db,
-                const cplx<TD>* __restrict__ Dz, int has_b, cplx<TD>* __restrict__ F, GridDims g, CellDev c,
+k_assemble_pair(const double2* __restrict__ RT, const double2* __restrict__ Da, const double2* __restrict__ Db,
+                const double2* __restrict__ Dz, int has_b, double2* __restrict__ F, GridDims g, CellDev c,
                 double inv_nr, double* partial) {
   __shared__ GTables tab;
   fill_tables(tab, g, c);
@@ -609,12 +602,12 @@ k_assemble_pair(const double2* __restrict__ RT, const cplx<TD>* __restrict__ Da,
       vb = va;
       if (Da) {
         // G . d of both fields at G (twice the unpacked values): x and y of a in Da, of b in Db, z in Dz
-        const double2 u = wide2(Da[p.idx]), un = wide2(Da[p.jn]), z = wide2(Dz[p.idx]), zn = wide2(Dz[p.jn]);
+        const double2 u = (Da[p.idx]), un = (Da[p.jn]), z = (Dz[p.idx]), zn = (Dz[p.jn]);
         const double dar = p.gx * (u.x + un.x) + p.gy * (u.y + un.y) + p.gz * (z.x + zn.x);
         const double dai = p.gx * (u.y - un.y) + p.gy * (un.x - u.x) + p.gz * (z.y - zn.y);
         va = make_double2(va.x + dai * s, va.y - dar * s);
         if (has_b) {
-          const double2 w = wide2(Db[p.idx]), wn = wide2(Db[p.jn]);
+          const double2 w = (Db[p.idx]), wn = (Db[p.jn]);
           const double dbr = p.gx * (w.x + wn.x) + p.gy * (w.y + wn.y) + p.gz * (z.y + zn.y);
           const double dbi = p.gx * (w.y - wn.y) + p.gy * (wn.x - w.x) + p.gz * (zn.x - z.x);
           vb = make_double2(vb.x + dbi * s, vb.y - dbr * s);
@@ -624,15 +617,84 @@ k_assemble_pair(const double2* __restrict__ RT, const cplx<TD>* __restrict__ Da,
     if (F) {
       // V(-G) = conj V(G)
       if (has_b) {
-        F[p.idx] = mk<TD>(narrow<TD>(va.x - vb.y), narrow<TD>(va.y + vb.x));
-        F[p.jn] = mk<TD>(narrow<TD>(va.x + vb.y), narrow<TD>(vb.x - va.y));
+        F[p.idx] = make_double2((va.x - vb.y), (va.y + vb.x));
+        F[p.jn] = make_double2((va.x + vb.y), (vb.x - va.y));
       } else {
-        F[p.idx] = mk<TD>(narrow<TD>(va.x), narrow<TD>(va.y));
-        F[p.jn] = mk<TD>(narrow<TD>(va.x), narrow<TD>(-va.y));
+        F[p.idx] = make_double2((va.x), (va.y));
+        F[p.jn] = make_double2((va.x), (-va.y));
       }
     }
   }
   if (SUMS) block_sum_store(eh, partial + blockIdx.x);
+}
+
+// The same for FP32 grids in double-float arithmetic (dd.cuh, ~46 bits, rounded once to FP32): some 600
+// FP32 operations a pair where 62 FP64 instructions take the time of 4000.
+struct GTablesDd {
+  dd x[kAxisMax], y[kAxisMax], z[kAxisMax];
+};
+__device__ __forceinline__ dd dd_dot3(dd a, dd p, dd b, dd q, dd c, dd r) { return dd_dot2(a, p, b, q) + c * r; }
+__device__ __forceinline__ float dd_sum_to_float(dd a, dd b) {
+  const dd s = dd_two_sum(a.hi, b.hi);
+  return __fadd_rn(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+}
+__global__ void __launch_bounds__(kRedThreads)
+k_assemble_pair_f32(const double2* __restrict__ RT, const float2* __restrict__ Da, const float2* __restrict__ Db,
+                    const float2* __restrict__ Dz, int has_b, float2* __restrict__ F, GridDims g, CellDev c,
+                    double inv_nr) {
+  __shared__ GTablesDd t;
+  for (int i = threadIdx.x; i < g.n1; i += blockDim.x) t.x[i] = dd_from_double(axis_g(i, g.n1, c.b[0][0]));
+  for (int i = threadIdx.x; i < g.n2; i += blockDim.x) t.y[i] = dd_from_double(axis_g(i, g.n2, c.b[1][1]));
+  for (int i = threadIdx.x; i < g.n3; i += blockDim.x) t.z[i] = dd_from_double(axis_g(i, g.n3, c.b[2][2]));
+  __syncthreads();
+  const int end = pair_end(g);
+  const dd s = dd_from_double(0.5 * inv_nr), zero = dd(0);
+  const dd four_pi = dd(4.0 * 3.14159265358979323846);
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < end; idx += gridDim.x * blockDim.x) {
+    const int i3 = idx % g.n3, r = idx / g.n3;
+    const int i2 = r % g.n2, i1 = r / g.n2;
+    const int j1 = i1 ? g.n1 - i1 : 0, j2 = i2 ? g.n2 - i2 : 0, j3 = i3 ? g.n3 - i3 : 0;
+    const int jn = (j1 * g.n2 + j2) * g.n3 + j3;
+    if (jn < idx) continue;
+    const bool nyq = (2 * i1 == g.n1) || (2 * i2 == g.n2) || (2 * i3 == g.n3);
+    dd ax = zero, ay = zero, bx = zero, by = zero;
+    if (!nyq) {
+      const dd gx = t.x[i1], gy = t.y[i2], gz = t.z[i3];
+      if (idx > 0) {
+        const dd g2 = dd_dot3(gx, gx, gy, gy, gz, gz);
+        // 1 / G^2 by one Newton step from the FP32 reciprocal
+        const float q = __frcp_rn(g2.hi);
+        const float e = __fmaf_rn(-g2.lo, q, __fmaf_rn(-g2.hi, q, 1.0f));
+        const dd f = four_pi * dd_fast_two_sum(q, __fmul_rn(q, e));
+        const double2 rt = RT[idx];
+        ax = f * dd_from_double(rt.x);
+        ay = f * dd_from_double(rt.y);
+      }
+      bx = ax;
+      by = ay;
+      if (Da) {
+        const float2 u = Da[idx], un = Da[jn], z = Dz[idx], zn = Dz[jn];
+        const dd dar = dd_dot3(gx, dd_two_sum(u.x, un.x), gy, dd_two_sum(u.y, un.y), gz, dd_two_sum(z.x, zn.x));
+        const dd dai = dd_dot3(gx, dd_two_sum(u.y, -un.y), gy, dd_two_sum(un.x, -u.x), gz, dd_two_sum(z.y, -zn.y));
+        ax += dai * s;
+        ay -= dar * s;
+        if (has_b) {
+          const float2 w = Db[idx], wn = Db[jn];
+          const dd dbr = dd_dot3(gx, dd_two_sum(w.x, wn.x), gy, dd_two_sum(w.y, wn.y), gz, dd_two_sum(z.y, zn.y));
+          const dd dbi = dd_dot3(gx, dd_two_sum(w.y, -wn.y), gy, dd_two_sum(wn.x, -w.x), gz, dd_two_sum(zn.x, -z.x));
+          bx += dbi * s;
+          by -= dbr * s;
+        }
+      }
+    }
+    if (has_b) {
+      F[idx] = make_float2(dd_sum_to_float(ax, -by), dd_sum_to_float(ay, bx));
+      F[jn] = make_float2(dd_sum_to_float(ax, by), dd_sum_to_float(bx, -ay));
+    } else {
+      F[idx] = make_float2(ax.hi, ay.hi);
+      F[jn] = make_float2(ax.hi, -ay.hi);
+    }
+  }
 }
 
 // veff_x = vloc + Re/Im F (inverse-transformed reciprocal part) + w_x for the pair's subsystems (either
@@ -849,37 +911,51 @@ void grid_unpack_density(const double2* C, int has_b, double2* RT, int accumulat
   else
     k_unpack_density<false><<<kRedBlocks, kRedThreads, 0, st>>>(C, has_b, RT, accumulate, Pa, Pb, Pz, g, c, inv, nullptr);
 }
-void grid_pw_total(const double* rho, const GradPacks& gp, int xc_mode, int kedf, double rho_cut, double* vpart,
-                   double* hx, double* hy, double* hz, long long nr, double* partial, bool fp32, cudaStream_t st) {
+template <typename R>
+void grid_pw_total(const double* rho, const GradPacks<R>& gp, int xc_mode, int kedf, double rho_cut, double* vpart,
+                   double* hx, double* hy, double* hz, long long nr, double* partial, cudaStream_t st) {
   count_launches(1);
   ProfScope prof_("k_pw_total", st);
-  if (fp32)
-    k_pw_total<float><<<kRedBlocks, kRedThreads, 0, st>>>(rho, gp, xc_mode, kedf, rho_cut, vpart, hx, hy, hz, nr,
-                                                          partial);
-  else
-    k_pw_total<double><<<kRedBlocks, kRedThreads, 0, st>>>(rho, gp, xc_mode, kedf, rho_cut, vpart, hx, hy, hz, nr,
-                                                           partial);
+  k_pw_total<R><<<kRedBlocks, kRedThreads, 0, st>>>(rho, gp, xc_mode, kedf, rho_cut, vpart, hx, hy, hz, nr, partial);
 }
 template <typename TD>
-void grid_pw_pair(const double* ra, const double* rb, const double2* Pa, const double2* Pb, const double2* Pz,
-                  cplx<TD>* Da, cplx<TD>* Db, cplx<TD>* Dz, const double* hx, const double* hy, const double* hz,
-                  const double* vtot, int xc_mode, int kedf, double rho_cut, double* wa, double* wb, int write_d,
-                  long long nr, double* partial, cudaStream_t st) {
+void grid_pw_pair(const double* ra, const double* rb, cplx<TD>* Pa, cplx<TD>* Pb, cplx<TD>* Pz, const double* hx,
+                  const double* hy, const double* hz, const double* vtot, int xc_mode, int kedf, double rho_cut,
+                  double* wa, double* wb, int write_d, long long nr, double* partial, cudaStream_t st) {
   count_launches(1);
   ProfScope prof_("k_pw_pair", st);
-  k_pw_pair<TD><<<kRedBlocks, kRedThreads, 0, st>>>(ra, rb, Pa, Pb, Pz, Da, Db, Dz, hx, hy, hz, vtot, xc_mode, kedf,
-                                                    rho_cut, wa, wb, write_d, nr, partial);
+  k_pw_pair<TD><<<kRedBlocks, kRedThreads, 0, st>>>(ra, rb, Pa, Pb, Pz, hx, hy, hz, vtot, xc_mode, kedf, rho_cut, wa, wb,
+                                                    write_d, nr, partial);
 }
-template <typename TD>
-void grid_assemble_pair(const double2* RT, const cplx<TD>* Da, const cplx<TD>* Db, const cplx<TD>* Dz, int has_b,
-                        cplx<TD>* F, const GridDims& g, const CellDev& c, double* partial, cudaStream_t st) {
+// FP64 grid rounded to FP32 (lengths without a double-float transform).
+__global__ void k_narrow_grid(const double2* __restrict__ a, float2* __restrict__ b, long long n) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const double2 v = a[i];
+    b[i] = make_float2(float_of_double_bits(v.x), float_of_double_bits(v.y));
+  }
+}
+void grid_narrow(const double2* a, float2* b, long long n, cudaStream_t st) {
+  count_launches(1);
+  k_narrow_grid<<<gs(n), 256, 0, st>>>(a, b, n);
+}
+template <>
+void grid_assemble_pair<double>(const double2* RT, const double2* Da, const double2* Db, const double2* Dz, int has_b,
+                                double2* F, const GridDims& g, const CellDev& c, double* partial, cudaStream_t st) {
   count_launches(1);
   ProfScope prof_("k_assemble_pair", st);
   const double inv = 1.0 / ((double)g.n1 * g.n2 * g.n3);
   if (partial)
-    k_assemble_pair<TD, true><<<kRedBlocks, kRedThreads, 0, st>>>(RT, Da, Db, Dz, has_b, F, g, c, inv, partial);
+    k_assemble_pair<true><<<kRedBlocks, kRedThreads, 0, st>>>(RT, Da, Db, Dz, has_b, F, g, c, inv, partial);
   else
-    k_assemble_pair<TD, false><<<kRedBlocks, kRedThreads, 0, st>>>(RT, Da, Db, Dz, has_b, F, g, c, inv, nullptr);
+    k_assemble_pair<false><<<kRedBlocks, kRedThreads, 0, st>>>(RT, Da, Db, Dz, has_b, F, g, c, inv, nullptr);
+}
+template <>
+void grid_assemble_pair<float>(const double2* RT, const float2* Da, const float2* Db, const float2* Dz, int has_b,
+                               float2* F, const GridDims& g, const CellDev& c, double*, cudaStream_t st) {
+  count_launches(1);
+  ProfScope prof_("k_assemble_pair", st);
+  k_assemble_pair_f32<<<kRedBlocks, kRedThreads, 0, st>>>(RT, Da, Db, Dz, has_b, F, g, c,
+                                                          1.0 / ((double)g.n1 * g.n2 * g.n3));
 }
 template <typename TD>
 void grid_finish_pair(const cplx<TD>* F, const double* vloc, double* va, double* vb, TD* pa, TD* pb, const GridDims& g,
@@ -902,12 +978,11 @@ int grid_red_blocks() { return kRedBlocks; }
   template void grid_c_to_real<T>(const cplx<T>*, double*, long long, cudaStream_t);                           \
   template void grid_combine<T>(const double*, const double*, const double*, const cplx<T>*, double, double*,   \
                                 long long, cudaStream_t);                                                      \
-  template void grid_pw_pair<T>(const double*, const double*, const double2*, const double2*, const double2*,   \
-                                cplx<T>*, cplx<T>*, cplx<T>*, const double*, const double*, const double*,       \
-                                const double*, int, int, double, double*, double*, int, long long, double*,      \
-                                cudaStream_t);                                                                 \
-  template void grid_assemble_pair<T>(const double2*, const cplx<T>*, const cplx<T>*, const cplx<T>*, int,      \
-                                      cplx<T>*, const GridDims&, const CellDev&, double*, cudaStream_t);        \
+  template void grid_pw_total<T>(const double*, const GradPacks<T>&, int, int, double, double*, double*, double*, \
+                                 double*, long long, double*, cudaStream_t);                                    \
+  template void grid_pw_pair<T>(const double*, const double*, cplx<T>*, cplx<T>*, cplx<T>*, const double*,       \
+                                const double*, const double*, const double*, int, int, double, double*, double*, \
+                                int, long long, double*, cudaStream_t);                                         \
   template void grid_finish_pair<T>(const cplx<T>*, const double*, double*, double*, T*, T*, const GridDims&,   \
                                     unsigned*, cudaStream_t);
 FDE_GRID_INST(float)

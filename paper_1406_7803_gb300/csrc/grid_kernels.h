@@ -39,29 +39,37 @@ void grid_aug_screening(const double2* VG, const GridDims& g, const CellDev& c, 
 
 // ---- packed pairs of real fields (two real grids in one complex transform) ----
 constexpr int kMaxPairs = 32;
-struct GradPacks {  // real-space gradients of the subsystem densities, pairwise packed
-  const double2* a[kMaxPairs];  // d/dx + i d/dy of the first density of pair q
-  const double2* b[kMaxPairs];  // the same for the second density (when has_b)
-  const double2* z[kMaxPairs];  // d/dz of the first + i d/dz of the second
+template <typename R> struct GradPacks {  // real-space gradients of the subsystem densities, pairwise packed
+  const cplx<R>* a[kMaxPairs];  // d/dx + i d/dy of the first density of pair q
+  const cplx<R>* b[kMaxPairs];  // the same for the second density (when has_b)
+  const cplx<R>* z[kMaxPairs];  // d/dz of the first + i d/dz of the second
   int has_b[kMaxPairs];
   int npairs;
 };
 void grid_pack2(const double* a, const double* b, double2* c, long long n, cudaStream_t st);
 void grid_unpack_density(const double2* C, int has_b, double2* RT, int accumulate, double2* Pa, double2* Pb,
                          double2* Pz, const GridDims& g, const CellDev& c, double* partial, cudaStream_t st);
-// fp32: the pointwise functionals in FP32 arithmetic (mixed path), else FP64.
-void grid_pw_total(const double* rho, const GradPacks& gp, int xc_mode, int kedf, double rho_cut, double* vpart,
-                   double* hx, double* hy, double* hz, long long nr, double* partial, bool fp32, cudaStream_t st);
-// The divergence arguments (Da, Db, Dz), the reciprocal-space potentials F and their transforms
-// are in precision TD: FP64 in FP64 contexts (Da.. may alias Pa..), FP32 in mixed ones.
+// The pointwise functionals in the working precision R / TD (FP64 in FP64 contexts, FP32 in mixed ones),
+// as are the gradients Pa, Pb, Pz, the divergence arguments that replace them, the reciprocal-space
+// potentials F and their transforms.
+template <typename R>
+void grid_pw_total(const double* rho, const GradPacks<R>& gp, int xc_mode, int kedf, double rho_cut, double* vpart,
+                   double* hx, double* hy, double* hz, long long nr, double* partial, cudaStream_t st);
 template <typename TD>
-void grid_pw_pair(const double* ra, const double* rb, const double2* Pa, const double2* Pb, const double2* Pz,
-                  cplx<TD>* Da, cplx<TD>* Db, cplx<TD>* Dz, const double* hx, const double* hy, const double* hz,
-                  const double* vtot, int xc_mode, int kedf, double rho_cut, double* wa, double* wb, int write_d,
-                  long long nr, double* partial, cudaStream_t st);
+void grid_pw_pair(const double* ra, const double* rb, cplx<TD>* Pa, cplx<TD>* Pb, cplx<TD>* Pz, const double* hx,
+                  const double* hy, const double* hz, const double* vtot, int xc_mode, int kedf, double rho_cut,
+                  double* wa, double* wb, int write_d, long long nr, double* partial, cudaStream_t st);
+void grid_narrow(const double2* a, float2* b, long long n, cudaStream_t st);
+// partial: Hartree sum of RT wanted (FP64 alone).
 template <typename TD>
 void grid_assemble_pair(const double2* RT, const cplx<TD>* Da, const cplx<TD>* Db, const cplx<TD>* Dz, int has_b,
                         cplx<TD>* F, const GridDims& g, const CellDev& c, double* partial, cudaStream_t st);
+template <>
+void grid_assemble_pair<double>(const double2* RT, const double2* Da, const double2* Db, const double2* Dz, int has_b,
+                                double2* F, const GridDims& g, const CellDev& c, double* partial, cudaStream_t st);
+template <>
+void grid_assemble_pair<float>(const double2* RT, const float2* Da, const float2* Db, const float2* Dz, int has_b,
+                               float2* F, const GridDims& g, const CellDev& c, double* partial, cudaStream_t st);
 // pa, pb: plane-major copies [n3][n1][n2] of the potentials va, vb (each given with its potential).
 template <typename TD>
 void grid_finish_pair(const cplx<TD>* F, const double* vloc, double* va, double* vb, TD* pa, TD* pb, const GridDims& g,

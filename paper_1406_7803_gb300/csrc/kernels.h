@@ -204,7 +204,9 @@ void launch_fft3d(cplx<T>* data, const GridDims& g, const FftPlans<T>& fp, int s
 // The same 3D transform of an FP64 grid computed in double-float arithmetic on the FP32 pipes
 // (fft_dd.cu): converted on the first axis pass, converted back on the last.  False (nothing
 // launched) when an axis length has no compiled kernel.
-bool launch_fft3d_dd(double2* data, const GridDims& g, const FftPlans<dd>& fp, int sign, cudaStream_t st);
+// high: the result goes there rounded to FP32 (the high parts), and data is left as work.
+bool launch_fft3d_dd(double2* data, const GridDims& g, const FftPlans<dd>& fp, int sign, cudaStream_t st,
+                     float2* high = nullptr);
 
 struct CellDev {
   double b[3][3];  // reciprocal rows
