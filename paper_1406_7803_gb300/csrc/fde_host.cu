@@ -346,6 +346,10 @@ template <typename T> struct EngineT : Engine {
   void fft3d_f64(double2* data, int sign, int arith) override {
     REQ(data && (sign == 1 || sign == -1) && (arith == 0 || arith == 1), FDE_EINVAL, "bad transform arguments");
     if (arith == 1) {
+      // the lengths this entry point states; the potential build takes more
+      for (int n : {g.n1, g.n2, g.n3})
+        REQ(n == 24 || n == 32 || n == 60 || n == 72 || n == 96 || n == 144 || n == 180 || n == 288, FDE_EUNSUPPORTED,
+            "no double-float kernel for a length");
       if constexpr (sizeof(T) == 4) {
         REQ(launch_fft3d_dd(data, g, plansdd.fp, sign, st), FDE_EUNSUPPORTED, "no double-float kernel for a length");
       } else {

@@ -108,9 +108,33 @@ def test_every_side_transforms(lib, n, prec, tol):
             ctx.fft3d(d, sign)
             assert np.abs(d.cpu().numpy() - want).max() < tol * np.abs(want).max(), (shape, sign)
         d = torch.from_numpy(f).to("cuda")
-        ctx.fft3d_f64(d, -1, 1)  # double-float: ~48 bits
-        want = np.fft.fftn(f) / f.size
-        assert np.abs(d.cpu().numpy() - want).max() < 2e-13 * np.abs(want).max(), shape
+        with pytest.raises(fde.FDEError) as e:  # 30 is not among the lengths it states
+            ctx.fft3d_f64(d, -1, 1)
+        assert e.value.status == fde.FDE_EUNSUPPORTED
+
+
+@gpu
+@pytest.mark.parametrize("n", [n for n in SIDES if n not in (24, 32, 60, 72, 96, 144)])
+def test_mixed_potentials_on_general_sides(lib, n):
+    """Potential build of two subsystems (one transform pair) and of three (a pair and a single) in
+    double-float and FP32 against the all-FP64 build: 1e-5 of the largest value, the mixed path's bound."""
+    torch, fde = lib
+    for grid, subs in (((n, 24, 32), 2), ((24, n, 32), 3)):
+        L = 0.25 * np.array(grid)
+        x, y, z = np.meshgrid(*[2 * np.pi * np.arange(k) / k for k in grid], indexing="ij")
+        out = {}
+        for prec in ("fp64", "mixed"):
+            ctx = fde.Context(np.diag(L), grid, 5.0, 1, 1, prec=prec)
+            for i in range(subs):
+                ctx.add_subsystem(np.array([[1.0 + i, 2.0, 3.0]]), np.ones(1), 0.5, 2, np.zeros((1, 3)), np.ones(1), 2.0,
+                                  0.01)
+                rho = 0.02 * (2.5 + np.cos(x + i) * np.cos(y) + 0.5 * np.sin(2 * z - i) + 0.3 * np.cos(x - y + z))
+                ctx.set_density(i, np.ascontiguousarray(rho))
+            v = torch.zeros((subs,) + grid, dtype=torch.float64, device="cuda")
+            ctx.build_vemb(v)
+            ctx.sync()
+            out[prec] = v.cpu().numpy()
+        assert np.abs(out["mixed"] - out["fp64"]).max() < 1e-5 * np.abs(out["fp64"]).max(), grid
 
 
 @gpu
