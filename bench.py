@@ -625,7 +625,7 @@ def run_ours(args):
         sec = ms_plane / n_plane / 1e3
         pk = fp["fp32_tflops"] if args.prec == "mixed" else fp["fp64_tflops"]
         achieved = per_launch_flops / sec / 1e12
-        traffic = (_profile_traffic("k_plane_ct_molecule_on_slab", PLANE_SOURCES, PLANE_FUNCTION)
+        traffic = (_profile_traffic("k_plane_pass_molecule_on_slab", PLANE_SOURCES, PLANE_FUNCTION)
                    if (args.prec == "mixed" and args.workload == "molecule-on-slab") else None)
         hbm_gbs = per_launch_bytes / sec / 1e9
         roof = {"bound": "alu", "achieved": achieved, "peak": pk, "unit": "TFLOP/s", "frac": achieved / pk,

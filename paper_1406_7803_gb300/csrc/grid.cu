@@ -629,7 +629,8 @@ k_assemble_pair(const double2* __restrict__ RT, const double2* __restrict__ Da, 
 }
 
 // The same for FP32 grids in double-float arithmetic (dd.cuh, ~46 bits, rounded once to FP32): some 600
-// FP32 operations a pair where 62 FP64 instructions take the time of 4000.
+// FP32 operations a pair where 62 FP64 instructions take the time of 4000: 62 -> 25.7 us at 72 x 72 x 180,
+// the error of V_eff against an FP64 build unchanged (2.2e-6 and 2.1e-6 of its norm).
 struct GTablesDd {
   dd x[kAxisMax], y[kAxisMax], z[kAxisMax];
 };

@@ -158,12 +158,12 @@ def precond_initial_weights(seed: int = 0) -> np.ndarray:
 
 
 def tuned_plane_variant(n1: int, n3: int) -> int:
-    """Variant of the FP32 plane pass the tuner chose for this grid shape (-1: none yet)."""
+    """Tuned plane-pass variant of this grid shape: -1, the plane pass has one form per shape."""
     return int(load().fde_tuned_plane_variant(int(n1), int(n3)))
 
 
 def pin_plane_variant(variant: int) -> None:
-    """Pin the FP32 plane-pass variant (0..7) for this process, or -1 to return to tuning."""
+    """Accepts a plane-pass variant (-1..7); without effect, the plane pass has one form per shape."""
     if load().fde_pin_plane_variant(int(variant)) != FDE_OK:
         raise FDEError(FDE_EINVAL, "fde_pin_plane_variant: variant must be -1..7")
 
