@@ -6,16 +6,17 @@
 
 namespace fde {
 
-// Run up to kBatchMax items per launch; items[i].zstart / pstart are filled here.
+// Run up to kBatchMax items per launch, as many as fit together; items[i].zstart / pstart are filled here.
 template <typename T>
 bool launch_hpsi_batch(const HpsiItemDesc<T>* items, int nitems, const GridDims& g, const FftPlans<T>& fp,
                        cudaStream_t st) {
   for (int i = 0; i < nitems; ++i)
     if (!two_step_grid<T>(g, items[i].sp)) return false;
   const T inv_nr = (T)(1.0 / ((double)g.n1 * g.n2 * g.n3));
-  for (int i0 = 0; i0 < nitems; i0 += kBatchMax) {
+  for (int i0 = 0, n = 0; i0 < nitems; i0 += n) {
+    n = plane_group<T>(g, items + i0, nitems - i0, kBatchMax);  // at least one: each fits alone
     HpsiBatch<T> B;
-    B.n = std::min(kBatchMax, nitems - i0);
+    B.n = n;
     int zb = 0, pb = 0;
     for (int j = 0; j < B.n; ++j) {
       const HpsiItemDesc<T>& d = items[i0 + j];

@@ -131,9 +131,25 @@ template <typename T> static int plane_lb(int n1, int n2) {
   return plane_batch(n2, side_rmax(n1), n1 == n2 ? plane_shape<T>(n1).nt : kPlaneThreads2);
 }
 
+// Bytes of a launch whose widest spans are span1 and span2.
+template <typename T> static size_t plane_launch_smem(const GridDims& g, int span1, int span2) {
+  return plane_smem2<T>(g.n1, g.n2, span1, span2, plane_lb<T>(g.n1, g.n2));
+}
+template <typename T> static bool plane_fits(const GridDims& g, int span1, int span2) {
+  return plane_launch_smem<T>(g, span1, span2) <= kPlaneSmemMax;
+}
 template <typename T> bool two_step_grid(const GridDims& g, const SphereDev& sp) {
   if (!split_side_ok(g.n1) || !split_side_ok(g.n2) || split_of(g.n3).a == 0) return false;
-  return plane_smem2<T>(g.n1, g.n2, sp.span1, sp.span2, plane_lb<T>(g.n1, g.n2)) <= kPlaneSmemMax;
+  return plane_fits<T>(g, sp.span1, sp.span2);
+}
+template <typename T> int plane_group(const GridDims& g, const HpsiItemDesc<T>* items, int nitems, int most) {
+  int s1 = 0, s2 = 0, n = 0;
+  for (; n < std::min(nitems, most); ++n) {
+    s1 = std::max(s1, items[n].sp.span1);
+    s2 = std::max(s2, items[n].sp.span2);
+    if (!plane_fits<T>(g, s1, s2)) break;
+  }
+  return n;
 }
 
 template <typename K> static inline void allow_smem2(K kernel, size_t bytes) {
@@ -160,7 +176,7 @@ void launch_plane_pass(const GridDims& g, unsigned blocks, const HpsiBatch<T>& B
     s2 = std::max(s2, B.it[i].sp.span2);
   }
   const int lb = plane_lb<T>(g.n1, g.n2);
-  const size_t sm = plane_smem2<T>(g.n1, g.n2, s1, s2, lb);
+  const size_t sm = plane_launch_smem<T>(g, s1, s2);
   const int psize = s1 * (g.n2 | 1);
   if (g.n1 == g.n2) {
     switch (g.n1) {
@@ -214,7 +230,7 @@ void launch_plane_density(const GridDims& g, const cplx<T>* scr, const SphereDev
   A* part = reinterpret_cast<A*>(part_);
   const int groups = plane_density_groups(nb, g.n3);
   const int lb = plane_lb<T>(g.n1, g.n2);
-  const size_t sm = plane_smem2<T>(g.n1, g.n2, sp.span1, sp.span2, lb);
+  const size_t sm = plane_launch_smem<T>(g, sp.span1, sp.span2);
   const int psize = sp.span1 * (g.n2 | 1);
   const dim3 grid(g.n3, groups);
   if (g.n1 == g.n2) {

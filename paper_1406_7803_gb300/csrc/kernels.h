@@ -56,7 +56,7 @@ template <typename T> struct HpsiItemDesc {
   cplx<T>* scratch;  // [nb][n3][ldc] of this item
   int ld, nb;
 };
-// Local H psi of many items in three launches (batches of up to 24 items each); false (nothing
+// Local H psi of many items in three launches (batches of up to 24 items that fit together); false (nothing
 // launched) when a length of the grid has no two-step plan (fft2.cuh): the runtime-length kernels
 // of hpsi.cu serve those grids.
 template <typename T>
@@ -79,6 +79,9 @@ void launch_plane_density(const GridDims& g, const cplx<T>* scratch, const Spher
                           double* part, double* rho_plane, int accumulate, const FftPlans<T>& fp, cudaStream_t st);
 // Whether a grid has two-step plans and its plane kernel fits shared memory for a sphere.
 template <typename T> bool two_step_grid(const GridDims& g, const SphereDev& sp);
+// How many of the first items one launch takes: one shared-memory size serves a launch, so its largest
+// spans, which may come from different items, have to fit together.  0 when the first does not fit alone.
+template <typename T> int plane_group(const GridDims& g, const HpsiItemDesc<T>* items, int nitems, int most);
 // Variant of the plane pass in use for a grid shape (-1: none was tuned), and the pinned one
 // (false for values outside -1 .. 7).
 int query_plane_variant(int n1, int n3);
