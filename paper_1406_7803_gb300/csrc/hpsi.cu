@@ -140,10 +140,6 @@ template <typename T> static size_t plane_smem(const GridDims& g) {
   return (size_t)g.n1 * (g.n2 + 1) * sizeof(cplx<T>);
 }
 
-template <typename K> static void allow_smem(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <typename T>
 void launch_hpsi_local(const cplx<T>* psi, int ldpsi, cplx<T>* hpsi, int ldh, int nb,
                        const T* kin, const T* vplane, cplx<T>* scratch, const SphereDev& sp,

@@ -12,6 +12,15 @@
 
 namespace fde {
 
+// The dynamic shared memory a kernel may be launched with is a property of the kernel, shared by every
+// thread that launches it, so it is always set to the most a CTA can have: set to the bytes of one
+// launch, it could be lowered between another thread's setting and launch, which is then refused.
+constexpr size_t kCtaSmemMax = 232448;  // 227 KB
+template <typename K> inline void allow_smem(K kernel, size_t bytes) {
+  if (bytes > 48 * 1024)
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCtaSmemMax);
+}
+
 // Every (subsystem, k) block of bands is an item; the kernels below run a batch of items in
 // one launch (the batch travels as a kernel parameter), so subsystems of uneven size share
 // the GPU instead of taking one small launch each.  The first z-block and the first plane

@@ -99,7 +99,6 @@ template <typename T> static size_t plane_smem2(int n1, int n2, int span1, int s
   const size_t x = std::max((size_t)n1 * lb, (size_t)span1 * (span2 | 1));
   return (p + x) * sizeof(cplx<T>);
 }
-constexpr size_t kPlaneSmemMax = 232448;  // 227 KB a CTA can have
 
 // Threads and least resident CTAs of a square plane's kernel.  A CTA has threads for one row of items of
 // the y steps (0.46 N rows hold columns at the cutoffs the grids are made for) and for whole batches
@@ -136,7 +135,7 @@ template <typename T> static size_t plane_launch_smem(const GridDims& g, int spa
   return plane_smem2<T>(g.n1, g.n2, span1, span2, plane_lb<T>(g.n1, g.n2));
 }
 template <typename T> static bool plane_fits(const GridDims& g, int span1, int span2) {
-  return plane_launch_smem<T>(g, span1, span2) <= kPlaneSmemMax;
+  return plane_launch_smem<T>(g, span1, span2) <= kCtaSmemMax;
 }
 template <typename T> bool two_step_grid(const GridDims& g, const SphereDev& sp) {
   if (!split_side_ok(g.n1) || !split_side_ok(g.n2) || split_of(g.n3).a == 0) return false;
@@ -152,17 +151,13 @@ template <typename T> int plane_group(const GridDims& g, const HpsiItemDesc<T>* 
   return n;
 }
 
-template <typename K> static inline void allow_smem2(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <typename T, int R1, int R2>
 static void plane_square(unsigned blocks, const HpsiBatch<T>& B, int n3, const FftPlans<T>& fp, size_t sm, int psize,
                          cudaStream_t st) {
   constexpr PlaneShape S = plane_shape<T>(R1 * R2);
   using Plan = SidePlan<R1, R2>;
   auto* k = k_plane_pass<T, Plan, Plan, S.nt, S.minb>;
-  allow_smem2(k, sm);
+  allow_smem(k, sm);
   count_launches(1);
   k<<<blocks, S.nt, sm, st>>>(B, n3, fp.p1.tw, fp.p2.tw, psize);
 }
@@ -189,7 +184,7 @@ void launch_plane_pass(const GridDims& g, unsigned blocks, const HpsiBatch<T>& B
     }
     return;
   }
-  allow_smem2(k_plane_pass_any<T>, sm);
+  allow_smem(k_plane_pass_any<T>, sm);
   count_launches(1);
   k_plane_pass_any<T><<<blocks, kPlaneThreads2, sm, st>>>(B, g.n1, g.n2, g.n3, fp.p1.tw, fp.p2.tw, psize, lb);
 }
@@ -214,7 +209,7 @@ static void rho_square(dim3 grid, const cplx<T>* scr, const SphereDev& sp, int n
   constexpr PlaneShape S = plane_shape<T>(R1 * R2);
   using Plan = SidePlan<R1, R2>;
   auto* k = k_plane_rho<T, Plan, Plan, S.nt, S.minb>;
-  allow_smem2(k, sm);
+  allow_smem(k, sm);
   count_launches(1);
   k<<<grid, S.nt, sm, st>>>(scr, sp, nb, weight, part, n3, fp.p1.tw, fp.p2.tw, psize);
 }
@@ -243,7 +238,7 @@ void launch_plane_density(const GridDims& g, const cplx<T>* scr, const SphereDev
 #undef FDE_CASE
     }
   } else {
-    allow_smem2(k_plane_rho_any<T>, sm);
+    allow_smem(k_plane_rho_any<T>, sm);
     count_launches(1);
     k_plane_rho_any<T><<<grid, kPlaneThreads2, sm, st>>>(scr, sp, nb, weight, part, g.n1, g.n2, g.n3, fp.p1.tw,
                                                          fp.p2.tw, psize, lb);

@@ -31,12 +31,12 @@ template <typename T> static int check(const GridDims& g, const std::vector<Hpsi
       s1 = std::max(s1, it[j].sp.span1);
       s2 = std::max(s2, it[j].sp.span2);
     }
-    if (plane_launch_smem<T>(g, s1, s2) > kPlaneSmemMax) return 2;
+    if (plane_launch_smem<T>(g, s1, s2) > kCtaSmemMax) return 2;
     if (i0 + k < n && k < kBatchMax) {
       ++cuts;
       s1 = std::max(s1, it[i0 + k].sp.span1);
       s2 = std::max(s2, it[i0 + k].sp.span2);
-      if (plane_launch_smem<T>(g, s1, s2) <= kPlaneSmemMax) return 3;
+      if (plane_launch_smem<T>(g, s1, s2) <= kCtaSmemMax) return 3;
     }
   }
   return 0;
@@ -88,16 +88,52 @@ int main() {
 """
 
 
-def test_launches_fit_shared_memory_for_every_side_and_pair_of_spans(tmp_path):
+def run(tmp_path, text):
     src, exe = tmp_path / "fit.cu", tmp_path / "fit"
-    src.write_text(PROGRAM)
+    src.write_text(text)
     cmd = [build.nvcc()] + build.ARCH + ["-std=c++17", "-O1", "-I", build.CSRC, "-I",
                                          os.path.join(build.ROOT, "include"), str(src), "-o", str(exe)]
     r = subprocess.run(cmd, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
-    assert int(r.stdout.split()[2]) > 0, "no list needed a cut: the test would not see a missing rule"
+    return r.stdout
+
+
+def test_launches_fit_shared_memory_for_every_side_and_pair_of_spans(tmp_path):
+    assert int(run(tmp_path, PROGRAM).split()[2]) > 0, "no list needed a cut: the test would not see a missing rule"
+
+
+# A launch of no blocks is refused before anything runs, with or without a GPU: the program sees what the
+# host side does around it.
+ATTRIBUTE = r"""
+#include <cstdio>
+#include <vector>
+#include <cuda_runtime.h>
+static std::vector<int> limits;
+template <typename K> static cudaError_t record(K, cudaFuncAttribute a, int v) {
+  if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) limits.push_back(v);
+  return cudaSuccess;
+}
+#define cudaFuncSetAttribute record
+#include "hpsi2_p.cuh"
+namespace fde { thread_local Profiler* tl_prof = nullptr; }
+using namespace fde;
+int main() {
+  HpsiBatch<float> B{};
+  FftPlans<float> fp{};
+  for (size_t bytes : {100000, 200000, 60000}) plane_square<float, 9, 8>(0, B, 24, fp, bytes, 0, 0);
+  for (int v : limits)
+    if (v != (int)kCtaSmemMax) return printf("limit set to %d\n", v), 1;
+  return limits.size() == 3 ? 0 : 1;
+}
+"""
+
+
+def test_no_launch_lowers_the_shared_memory_limit_of_its_kernel(tmp_path):
+    """Threads share the limit: one that a launch lowers to its own bytes makes another thread's launch of
+    the same kernel, with more, fail."""
+    run(tmp_path, ATTRIBUTE)
 
 
 gpu = pytest.mark.gpu
