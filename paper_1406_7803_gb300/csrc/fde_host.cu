@@ -847,7 +847,7 @@ template <typename T> struct EngineT : Engine {
   void apply_h_dev(Sub<T>& s, KP<T>& q, const C* psi, C* hpsi, int nb) {
     hpsi_bands += nb;
     scratch.ensure((size_t)nb * g.n3 * q.sp.ldc);
-    launch_hpsi_local<T>(psi, q.npw, hpsi, q.npw, nb, q.kin_d.p, s.vplane.p, scratch.p, q.sp, g, plans.fp, st);
+    CK(launch_hpsi_local<T>(psi, q.npw, hpsi, q.npw, nb, q.kin_d.p, s.vplane.p, scratch.p, q.sp, g, plans.fp, st));
     apply_nl(s, q, psi, hpsi, nb);
   }
   // hpsi += sum_{a in I} beta D <beta|psi> (projectors of the subsystem's own atoms)
@@ -936,11 +936,13 @@ template <typename T> struct EngineT : Engine {
         items.push_back(HpsiItemDesc<T>{q.sp, q.X.p, q.HX.p, q.kin_d.p, sp->vplane.p, scratch.p + off, q.npw, sp->nb});
         off += (size_t)sp->nb * g.n3 * q.sp.ldc;
       }
-    if (!launch_hpsi_batch<T>(items.data(), (int)items.size(), g, plans.fp, st)) {
+    cudaError_t e = cudaSuccess;
+    if (!launch_hpsi_batch<T>(items.data(), (int)items.size(), g, plans.fp, st, &e)) {
       for (auto& sp : subs)
         for (auto& q : sp->kp) apply_h_dev(*sp, q, q.X.p, q.HX.p, sp->nb);
       return;
     }
+    CK(e);
     for (auto& sp : subs)
       for (auto& q : sp->kp) {
         hpsi_bands += sp->nb;
@@ -1436,7 +1438,7 @@ template <typename T> struct EngineT : Engine {
       CK(cudaMemcpyAsync(occw.p, w.data(), s.nb * sizeof(double), cudaMemcpyHostToDevice, st));
       scratch.ensure((size_t)s.nb * g.n3 * q.sp.ldc);
       rho_part.ensure((size_t)plane_density_groups(s.nb, g.n3) * nr);
-      launch_density<T>(q.X.p, q.npw, s.nb, occw.p, scratch.p, rho_part.p, rho_plane.p, k > 0, q.sp, g, plans.fp, st);
+      CK(launch_density<T>(q.X.p, q.npw, s.nb, occw.p, scratch.p, rho_part.p, rho_plane.p, k > 0, q.sp, g, plans.fp, st));
       CK(cudaStreamSynchronize(st));  // occw is reused by the next k
     }
     launch_transpose<double, double>(rho_plane.p, out, g.n3, (int)((long long)g.n1 * g.n2), 0, st);

@@ -141,35 +141,31 @@ template <typename T> static size_t plane_smem(const GridDims& g) {
 }
 
 template <typename T>
-void launch_hpsi_local(const cplx<T>* psi, int ldpsi, cplx<T>* hpsi, int ldh, int nb,
-                       const T* kin, const T* vplane, cplx<T>* scratch, const SphereDev& sp,
-                       const GridDims& g, const FftPlans<T>& fp, cudaStream_t st) {
-  if (nb <= 0) return;
+cudaError_t launch_hpsi_local(const cplx<T>* psi, int ldpsi, cplx<T>* hpsi, int ldh, int nb, const T* kin,
+                              const T* vplane, cplx<T>* scratch, const SphereDev& sp, const GridDims& g,
+                              const FftPlans<T>& fp, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  if (nb <= 0) return e;
   if (ldpsi == ldh) {
     const HpsiItemDesc<T> d{sp, psi, hpsi, kin, vplane, scratch, ldpsi, nb};
-    if (launch_hpsi_batch<T>(&d, 1, g, fp, st)) return;
+    if (launch_hpsi_batch<T>(&d, 1, g, fp, st, &e)) return e;
   }
   const dim3 gz(ceil_div(sp.ncol, kColsPerCta), nb);
   const size_t zs = zpass_smem<T>(g.n3), ps = plane_smem<T>(g);
-  allow_smem(k_zinv<T>, zs);
-  allow_smem(k_zfwd<T>, zs);
-  allow_smem(k_plane<T>, ps);
   {
     ProfScope p("k_zinv", st, 1);
-    count_launches(1);
-    k_zinv<T><<<gz, kColsPerCta * 32, zs, st>>>(psi, ldpsi, scratch, sp, g.n3, fp.p3);
+    e = launch_sized(k_zinv<T>, gz, kColsPerCta * 32, zs, st, psi, ldpsi, scratch, sp, g.n3, fp.p3);
+    if (e != cudaSuccess) return e;
   }
   {
     ProfScope p("k_plane", st, 1);
-    count_launches(1);
-    k_plane<T><<<dim3(g.n3, nb), kPlaneThreads, ps, st>>>(scratch, sp, vplane, g, fp.p1, fp.p2);
+    e = launch_sized(k_plane<T>, dim3(g.n3, nb), kPlaneThreads, ps, st, scratch, sp, vplane, g, fp.p1, fp.p2);
+    if (e != cudaSuccess) return e;
   }
   const T inv_nr = (T)(1.0 / ((double)g.n1 * g.n2 * g.n3));
-  {
-    ProfScope p("k_zfwd", st, 1);
-    count_launches(1);
-    k_zfwd<T><<<gz, kColsPerCta * 32, zs, st>>>(scratch, psi, ldpsi, hpsi, ldh, kin, sp, g.n3, inv_nr, fp.p3);
-  }
+  ProfScope p("k_zfwd", st, 1);
+  return launch_sized(k_zfwd<T>, gz, kColsPerCta * 32, zs, st, scratch, psi, ldpsi, hpsi, ldh, kin, sp, g.n3, inv_nr,
+                      fp.p3);
 }
 
 // ---- densities ---------------------------------------------------------------------------
@@ -209,10 +205,10 @@ k_plane_density(const cplx<T>* __restrict__ scratch, SphereDev sp, int nb, const
 }
 
 template <typename T>
-void launch_density(const cplx<T>* psi, int ldpsi, int nb, const double* weight, cplx<T>* scratch, double* part,
-                    double* rho_plane, int accumulate, const SphereDev& sp, const GridDims& g, const FftPlans<T>& fp,
-                    cudaStream_t st) {
-  if (nb <= 0) return;
+cudaError_t launch_density(const cplx<T>* psi, int ldpsi, int nb, const double* weight, cplx<T>* scratch, double* part,
+                           double* rho_plane, int accumulate, const SphereDev& sp, const GridDims& g,
+                           const FftPlans<T>& fp, cudaStream_t st) {
+  if (nb <= 0) return cudaSuccess;
   if (two_step_grid<T>(g, sp)) {
     HpsiBatch<T> B;
     B.n = 1;
@@ -222,17 +218,14 @@ void launch_density(const cplx<T>* psi, int ldpsi, int nb, const double* weight,
       launch_zinv_cols<T>(g.n3, (unsigned)(ceil_div(sp.ncol, z_cols<T>()) * nb), B, fp.p3.tw, st);
     }
     ProfScope prof_("k_plane_density", st);
-    launch_plane_density<T>(g, scratch, sp, nb, weight, part, rho_plane, accumulate, fp, st);
-    return;
+    return launch_plane_density<T>(g, scratch, sp, nb, weight, part, rho_plane, accumulate, fp, st);
   }
   const dim3 gz(ceil_div(sp.ncol, kColsPerCta), nb);
   const size_t zs = zpass_smem<T>(g.n3), ps = plane_smem<T>(g);
-  allow_smem(k_zinv<T>, zs);
-  allow_smem(k_plane_density<T>, ps);
-  count_launches(1);
-  k_zinv<T><<<gz, kColsPerCta * 32, zs, st>>>(psi, ldpsi, scratch, sp, g.n3, fp.p3);
-  count_launches(1);
-  k_plane_density<T><<<g.n3, kPlaneThreads, ps, st>>>(scratch, sp, nb, weight, rho_plane, accumulate, g, fp.p1, fp.p2);
+  const cudaError_t e = launch_sized(k_zinv<T>, gz, kColsPerCta * 32, zs, st, psi, ldpsi, scratch, sp, g.n3, fp.p3);
+  if (e != cudaSuccess) return e;
+  return launch_sized(k_plane_density<T>, g.n3, kPlaneThreads, ps, st, scratch, sp, nb, weight, rho_plane, accumulate, g,
+                      fp.p1, fp.p2);
 }
 
 // ---- transposes ----------------------------------------------------------------------------
@@ -262,15 +255,16 @@ void launch_transpose(const Tin* in, Tout* out, int rows, int cols, int accumula
   k_transpose<Tin, Tout><<<grid, dim3(32, 8), 0, st>>>(in, out, rows, cols, accumulate);
 }
 
-template void launch_hpsi_local<float>(const float2*, int, float2*, int, int, const float*, const float*, float2*,
-                                       const SphereDev&, const GridDims&, const FftPlans<float>&, cudaStream_t);
-template void launch_hpsi_local<double>(const double2*, int, double2*, int, int, const double*, const double*,
-                                        double2*, const SphereDev&, const GridDims&, const FftPlans<double>&,
-                                        cudaStream_t);
-template void launch_density<float>(const float2*, int, int, const double*, float2*, double*, double*, int,
-                                    const SphereDev&, const GridDims&, const FftPlans<float>&, cudaStream_t);
-template void launch_density<double>(const double2*, int, int, const double*, double2*, double*, double*, int,
-                                     const SphereDev&, const GridDims&, const FftPlans<double>&, cudaStream_t);
+template cudaError_t launch_hpsi_local<float>(const float2*, int, float2*, int, int, const float*, const float*,
+                                              float2*, const SphereDev&, const GridDims&, const FftPlans<float>&,
+                                              cudaStream_t);
+template cudaError_t launch_hpsi_local<double>(const double2*, int, double2*, int, int, const double*, const double*,
+                                               double2*, const SphereDev&, const GridDims&, const FftPlans<double>&,
+                                               cudaStream_t);
+template cudaError_t launch_density<float>(const float2*, int, int, const double*, float2*, double*, double*, int,
+                                           const SphereDev&, const GridDims&, const FftPlans<float>&, cudaStream_t);
+template cudaError_t launch_density<double>(const double2*, int, int, const double*, double2*, double*, double*, int,
+                                            const SphereDev&, const GridDims&, const FftPlans<double>&, cudaStream_t);
 template void launch_transpose<double, double>(const double*, double*, int, int, int, cudaStream_t);
 template void launch_transpose<double, float>(const double*, float*, int, int, int, cudaStream_t);
 

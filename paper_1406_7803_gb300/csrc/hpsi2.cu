@@ -9,7 +9,8 @@ namespace fde {
 // Run up to kBatchMax items per launch, as many as fit together; items[i].zstart / pstart are filled here.
 template <typename T>
 bool launch_hpsi_batch(const HpsiItemDesc<T>* items, int nitems, const GridDims& g, const FftPlans<T>& fp,
-                       cudaStream_t st) {
+                       cudaStream_t st, cudaError_t* status) {
+  *status = cudaSuccess;
   for (int i = 0; i < nitems; ++i)
     if (!two_step_grid<T>(g, items[i].sp)) return false;
   const T inv_nr = (T)(1.0 / ((double)g.n1 * g.n2 * g.n3));
@@ -31,7 +32,8 @@ bool launch_hpsi_batch(const HpsiItemDesc<T>* items, int nitems, const GridDims&
     }
     {
       ProfScope p("k_plane", st, 1);
-      launch_plane_pass<T>(g, (unsigned)pb, B, fp, st);
+      *status = launch_plane_pass<T>(g, (unsigned)pb, B, fp, st);
+      if (*status != cudaSuccess) return true;
     }
     {
       ProfScope p("k_zfwd", st, 1);
@@ -41,9 +43,9 @@ bool launch_hpsi_batch(const HpsiItemDesc<T>* items, int nitems, const GridDims&
   return true;
 }
 template bool launch_hpsi_batch<float>(const HpsiItemDesc<float>*, int, const GridDims&, const FftPlans<float>&,
-                                       cudaStream_t);
+                                       cudaStream_t, cudaError_t*);
 template bool launch_hpsi_batch<double>(const HpsiItemDesc<double>*, int, const GridDims&, const FftPlans<double>&,
-                                        cudaStream_t);
+                                        cudaStream_t, cudaError_t*);
 
 int plane_density_groups(int nb, int n3) {
   const int g = ceil_div(4 * 152, n3);

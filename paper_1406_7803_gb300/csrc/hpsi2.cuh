@@ -12,13 +12,26 @@
 
 namespace fde {
 
+// Launches a kernel whose shared memory is computed when it runs, and returns the launch's own status: a
+// refused launch leaves no other trace, and the passes after it would run on the data of the one before.
 // The dynamic shared memory a kernel may be launched with is a property of the kernel, shared by every
 // thread that launches it, so it is always set to the most a CTA can have: set to the bytes of one
 // launch, it could be lowered between another thread's setting and launch, which is then refused.
 constexpr size_t kCtaSmemMax = 232448;  // 227 KB
-template <typename K> inline void allow_smem(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024)
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCtaSmemMax);
+template <typename... A, typename... B>
+inline cudaError_t launch_sized(void (*kernel)(A...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                const B&... args) {
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCtaSmemMax);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  count_launches(1);
+  return cudaLaunchKernelEx(&cfg, kernel, A(args)...);
 }
 
 // Every (subsystem, k) block of bands is an item; the kernels below run a batch of items in

@@ -152,19 +152,17 @@ template <typename T> int plane_group(const GridDims& g, const HpsiItemDesc<T>* 
 }
 
 template <typename T, int R1, int R2>
-static void plane_square(unsigned blocks, const HpsiBatch<T>& B, int n3, const FftPlans<T>& fp, size_t sm, int psize,
-                         cudaStream_t st) {
+static cudaError_t plane_square(unsigned blocks, const HpsiBatch<T>& B, int n3, const FftPlans<T>& fp, size_t sm,
+                                int psize, cudaStream_t st) {
   constexpr PlaneShape S = plane_shape<T>(R1 * R2);
   using Plan = SidePlan<R1, R2>;
-  auto* k = k_plane_pass<T, Plan, Plan, S.nt, S.minb>;
-  allow_smem(k, sm);
-  count_launches(1);
-  k<<<blocks, S.nt, sm, st>>>(B, n3, fp.p1.tw, fp.p2.tw, psize);
+  return launch_sized(k_plane_pass<T, Plan, Plan, S.nt, S.minb>, blocks, S.nt, sm, st, B, n3, fp.p1.tw, fp.p2.tw,
+                      psize);
 }
 
 template <typename T>
-void launch_plane_pass(const GridDims& g, unsigned blocks, const HpsiBatch<T>& B, const FftPlans<T>& fp,
-                       cudaStream_t st) {
+cudaError_t launch_plane_pass(const GridDims& g, unsigned blocks, const HpsiBatch<T>& B, const FftPlans<T>& fp,
+                              cudaStream_t st) {
   int s1 = 0, s2 = 0;
   for (int i = 0; i < B.n; ++i) {
     s1 = std::max(s1, B.it[i].sp.span1);
@@ -175,18 +173,16 @@ void launch_plane_pass(const GridDims& g, unsigned blocks, const HpsiBatch<T>& B
   const int psize = s1 * (g.n2 | 1);
   if (g.n1 == g.n2) {
     switch (g.n1) {
-#define FDE_CASE(N, R1, R2)                                          \
-  case N:                                                            \
-    plane_square<T, R1, R2>(blocks, B, g.n3, fp, sm, psize, st);     \
-    return;
+#define FDE_CASE(N, R1, R2) \
+  case N:                   \
+    return plane_square<T, R1, R2>(blocks, B, g.n3, fp, sm, psize, st);
       FDE_PLANE_SIDES(FDE_CASE)
 #undef FDE_CASE
     }
-    return;
+    return cudaErrorInvalidValue;
   }
-  allow_smem(k_plane_pass_any<T>, sm);
-  count_launches(1);
-  k_plane_pass_any<T><<<blocks, kPlaneThreads2, sm, st>>>(B, g.n1, g.n2, g.n3, fp.p1.tw, fp.p2.tw, psize, lb);
+  return launch_sized(k_plane_pass_any<T>, blocks, kPlaneThreads2, sm, st, B, g.n1, g.n2, g.n3, fp.p1.tw, fp.p2.tw,
+                      psize, lb);
 }
 
 // rho_plane (+)= the groups' partial sums, in group order.
@@ -203,23 +199,22 @@ __global__ void k_rho_groups(const A* __restrict__ part, int groups, double* __r
 }
 
 template <typename T, int R1, int R2>
-static void rho_square(dim3 grid, const cplx<T>* scr, const SphereDev& sp, int nb, const double* weight,
-                       typename RhoAcc<T>::t* part, int n3, const FftPlans<T>& fp, size_t sm, int psize,
-                       cudaStream_t st) {
+static cudaError_t rho_square(dim3 grid, const cplx<T>* scr, const SphereDev& sp, int nb, const double* weight,
+                              typename RhoAcc<T>::t* part, int n3, const FftPlans<T>& fp, size_t sm, int psize,
+                              cudaStream_t st) {
   constexpr PlaneShape S = plane_shape<T>(R1 * R2);
   using Plan = SidePlan<R1, R2>;
-  auto* k = k_plane_rho<T, Plan, Plan, S.nt, S.minb>;
-  allow_smem(k, sm);
-  count_launches(1);
-  k<<<grid, S.nt, sm, st>>>(scr, sp, nb, weight, part, n3, fp.p1.tw, fp.p2.tw, psize);
+  return launch_sized(k_plane_rho<T, Plan, Plan, S.nt, S.minb>, grid, S.nt, sm, st, scr, sp, nb, weight, part, n3,
+                      fp.p1.tw, fp.p2.tw, psize);
 }
 
 // Groups of bands of a plane density: enough CTAs for four on each of 152 SMs.
 int plane_density_groups(int nb, int n3);
 
 template <typename T>
-void launch_plane_density(const GridDims& g, const cplx<T>* scr, const SphereDev& sp, int nb, const double* weight,
-                          double* part_, double* rho_plane, int accumulate, const FftPlans<T>& fp, cudaStream_t st) {
+cudaError_t launch_plane_density(const GridDims& g, const cplx<T>* scr, const SphereDev& sp, int nb,
+                                 const double* weight, double* part_, double* rho_plane, int accumulate,
+                                 const FftPlans<T>& fp, cudaStream_t st) {
   using A = typename RhoAcc<T>::t;
   static_assert(sizeof(A) == sizeof(double), "partial sums take the space of a double");
   A* part = reinterpret_cast<A*>(part_);
@@ -228,25 +223,26 @@ void launch_plane_density(const GridDims& g, const cplx<T>* scr, const SphereDev
   const size_t sm = plane_launch_smem<T>(g, sp.span1, sp.span2);
   const int psize = sp.span1 * (g.n2 | 1);
   const dim3 grid(g.n3, groups);
+  cudaError_t e = cudaErrorInvalidValue;
   if (g.n1 == g.n2) {
     switch (g.n1) {
-#define FDE_CASE(N, R1, R2)                                                                        \
-  case N:                                                                                          \
-    rho_square<T, R1, R2>(grid, scr, sp, nb, weight, part, g.n3, fp, sm, psize, st);               \
+#define FDE_CASE(N, R1, R2)                                                              \
+  case N:                                                                                \
+    e = rho_square<T, R1, R2>(grid, scr, sp, nb, weight, part, g.n3, fp, sm, psize, st); \
     break;
       FDE_PLANE_SIDES(FDE_CASE)
 #undef FDE_CASE
     }
   } else {
-    allow_smem(k_plane_rho_any<T>, sm);
-    count_launches(1);
-    k_plane_rho_any<T><<<grid, kPlaneThreads2, sm, st>>>(scr, sp, nb, weight, part, g.n1, g.n2, g.n3, fp.p1.tw,
-                                                         fp.p2.tw, psize, lb);
+    e = launch_sized(k_plane_rho_any<T>, grid, kPlaneThreads2, sm, st, scr, sp, nb, weight, part, g.n1, g.n2, g.n3,
+                     fp.p1.tw, fp.p2.tw, psize, lb);
   }
+  if (e != cudaSuccess) return e;
   const long long n = (long long)g.n1 * g.n2 * g.n3;
   count_launches(1);
   k_rho_groups<A><<<(unsigned)std::min<long long>((n + 255) / 256, 4096), 256, 0, st>>>(part, groups, rho_plane,
                                                                                       accumulate, n);
+  return cudaSuccess;
 }
 
 }  // namespace fde

@@ -283,8 +283,10 @@ extern "C" fde_status fde_apply_h_local_static(const fde_cell_desc* cell, const 
   const int chunk = (int)std::min<long long>(nb, kStScratch / per_band);
   for (int b0 = 0; b0 < nb; b0 += chunk) {
     const int nbc = std::min(chunk, nb - b0);
-    launch_hpsi_local<double>((const double2*)d_psi + (size_t)b0 * npw, npw, (double2*)d_hpsi + (size_t)b0 * npw,
-                              npw, nbc, P.kin, P.vplane, P.scratch, sp, g, fp, st);
+    const cudaError_t e =
+        launch_hpsi_local<double>((const double2*)d_psi + (size_t)b0 * npw, npw, (double2*)d_hpsi + (size_t)b0 * npw,
+                                  npw, nbc, P.kin, P.vplane, P.scratch, sp, g, fp, st);
+    if (e != cudaSuccess) return FDE_ECUDA;
   }
   if (cudaGetLastError() != cudaSuccess) return FDE_ECUDA;
   return FDE_OK;

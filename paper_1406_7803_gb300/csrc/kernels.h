@@ -33,18 +33,19 @@ template <typename T> struct FftPlans {
 };
 
 // ---- H psi local part and densities (hpsi.cu) -----------------------------------------
-// scratch: [nb][n3][ldc] complex T.  vplane: [n3][n1][n2] real T.
+// scratch: [nb][n3][ldc] complex T.  vplane: [n3][n1][n2] real T.  These return the status of the launches
+// with computed shared memory; after a refused one nothing more is launched.
 template <typename T>
-void launch_hpsi_local(const cplx<T>* psi, int ldpsi, cplx<T>* hpsi, int ldh, int nb,
-                       const T* kin, const T* vplane, cplx<T>* scratch, const SphereDev& sp,
-                       const GridDims& g, const FftPlans<T>& fp, cudaStream_t st);
+cudaError_t launch_hpsi_local(const cplx<T>* psi, int ldpsi, cplx<T>* hpsi, int ldh, int nb, const T* kin,
+                              const T* vplane, cplx<T>* scratch, const SphereDev& sp, const GridDims& g,
+                              const FftPlans<T>& fp, cudaStream_t st);
 
 // rho_plane[n3][n1][n2] (+)= sum_b weight[b] |u_b(r)|^2 for the block of nb orbitals; part: work of
 // plane_density_groups(nb, n3) N_r doubles.
 template <typename T>
-void launch_density(const cplx<T>* psi, int ldpsi, int nb, const double* weight,
-                    cplx<T>* scratch, double* part, double* rho_plane, int accumulate, const SphereDev& sp,
-                    const GridDims& g, const FftPlans<T>& fp, cudaStream_t st);
+cudaError_t launch_density(const cplx<T>* psi, int ldpsi, int nb, const double* weight, cplx<T>* scratch, double* part,
+                           double* rho_plane, int accumulate, const SphereDev& sp, const GridDims& g,
+                           const FftPlans<T>& fp, cudaStream_t st);
 
 // One (subsystem, k) block of bands of a batched H psi launch.
 template <typename T> struct HpsiItemDesc {
@@ -58,10 +59,10 @@ template <typename T> struct HpsiItemDesc {
 };
 // Local H psi of many items in three launches (batches of up to 24 items that fit together); false (nothing
 // launched) when a length of the grid has no two-step plan (fft2.cuh): the runtime-length kernels
-// of hpsi.cu serve those grids.
+// of hpsi.cu serve those grids.  *status: that of the launches.
 template <typename T>
 bool launch_hpsi_batch(const HpsiItemDesc<T>* items, int nitems, const GridDims& g, const FftPlans<T>& fp,
-                       cudaStream_t st);
+                       cudaStream_t st, cudaError_t* status);
 // The same three phases' launches on a prepared batch (hpsi2_z32.cu, hpsi2_z64.cu, hpsi2_p32.cu,
 // hpsi2_p64.cu).
 template <typename T> struct HpsiBatch;
@@ -70,13 +71,15 @@ void launch_zinv_cols(int n3, unsigned blocks, const HpsiBatch<T>& B, const cplx
 template <typename T>
 void launch_zfwd_cols(int n3, unsigned blocks, const HpsiBatch<T>& B, T inv_nr, const cplx<T>* tw, cudaStream_t st);
 template <typename T>
-void launch_plane_pass(const GridDims& g, unsigned blocks, const HpsiBatch<T>& B, const FftPlans<T>& fp, cudaStream_t st);
+cudaError_t launch_plane_pass(const GridDims& g, unsigned blocks, const HpsiBatch<T>& B, const FftPlans<T>& fp,
+                              cudaStream_t st);
 // rho_plane (+)= sum_b weight[b] |u_b|^2 from the z pass's scratch; part: plane_density_groups
 // partial densities (N_r doubles each).
 int plane_density_groups(int nb, int n3);
 template <typename T>
-void launch_plane_density(const GridDims& g, const cplx<T>* scratch, const SphereDev& sp, int nb, const double* weight,
-                          double* part, double* rho_plane, int accumulate, const FftPlans<T>& fp, cudaStream_t st);
+cudaError_t launch_plane_density(const GridDims& g, const cplx<T>* scratch, const SphereDev& sp, int nb,
+                                 const double* weight, double* part, double* rho_plane, int accumulate,
+                                 const FftPlans<T>& fp, cudaStream_t st);
 // Whether a grid has two-step plans and its plane kernel fits shared memory for a sphere.
 template <typename T> bool two_step_grid(const GridDims& g, const SphereDev& sp);
 // How many of the first items one launch takes: one shared-memory size serves a launch, so its largest

@@ -130,10 +130,30 @@ int main() {
 """
 
 
+# The same launches' own status, and the limit's when that is what fails.
+STATUS = ATTRIBUTE[:ATTRIBUTE.index("int main")].replace("return cudaSuccess;", "return answer;").replace(
+    "template <typename K>", "static cudaError_t answer = cudaSuccess;\ntemplate <typename K>", 1) + r"""
+int main() {
+  HpsiBatch<float> B{};
+  FftPlans<float> fp{};
+  SphereDev sp{};
+  if (plane_square<float, 9, 8>(0, B, 24, fp, 60000, 0, 0) == cudaSuccess) return printf("plane pass\n"), 1;
+  if (rho_square<float, 9, 8>(dim3(0), nullptr, sp, 1, nullptr, nullptr, 24, fp, 60000, 0, 0) == cudaSuccess)
+    return printf("density\n"), 1;
+  answer = cudaErrorInvalidValue;
+  return plane_square<float, 9, 8>(0, B, 24, fp, 60000, 0, 0) == answer ? 0 : 1;
+}
+"""
+
+
 def test_no_launch_lowers_the_shared_memory_limit_of_its_kernel(tmp_path):
     """Threads share the limit: one that a launch lowers to its own bytes makes another thread's launch of
     the same kernel, with more, fail."""
     run(tmp_path, ATTRIBUTE)
+
+
+def test_a_refused_launch_is_reported(tmp_path):
+    run(tmp_path, STATUS)
 
 
 gpu = pytest.mark.gpu
