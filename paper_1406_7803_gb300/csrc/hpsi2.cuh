@@ -211,9 +211,9 @@ template <typename Plan> __device__ __forceinline__ int span_base(int j, int lo)
   return b < 0 ? b + Plan::N : b;
 }
 
+// Inverse y transforms: step 1 takes the columns from X to the rows of P, step 2 runs within P.
 template <typename T, typename Plan>
-__device__ __forceinline__ void plane_y_inv(cplx<T>* P, const cplx<T>* X, const PlaneDims& D, int pitch, int nt,
-                                            const cplx<T>* __restrict__ tw) {
+__device__ __forceinline__ void plane_y_inv_1(cplx<T>* P, const cplx<T>* X, const PlaneDims& D, int pitch, int nt) {
   using C = cplx<T>;
   constexpr int R1 = Plan::R1, R2 = Plan::R2;
   const unsigned inv = (1u << 20) / (unsigned)D.n1s + 1u;  // w / n1s = w inv >> 20 for w < 2^20 / n1s
@@ -233,7 +233,13 @@ __device__ __forceinline__ void plane_y_inv(cplx<T>* P, const cplx<T>* X, const 
 #pragma unroll
     for (int q = 0; q < R1; ++q) o[Plan::wrap(Plan::out0(q) + oj)] = v[q];
   }
-  __syncthreads();
+}
+template <typename T, typename Plan>
+__device__ __forceinline__ void plane_y_inv_2(cplx<T>* P, const PlaneDims& D, int pitch, int nt,
+                                              const cplx<T>* __restrict__ tw) {
+  using C = cplx<T>;
+  constexpr int R1 = Plan::R1, R2 = Plan::R2;
+  const unsigned inv = (1u << 20) / (unsigned)D.n1s + 1u;
   for (int w = threadIdx.x; w < D.n1s * R1; w += nt) {
     const int q = (int)(((unsigned)w * inv) >> 20), r = w - q * D.n1s;
     C* o = P + r * pitch;
@@ -249,9 +255,10 @@ __device__ __forceinline__ void plane_y_inv(cplx<T>* P, const cplx<T>* X, const 
   }
 }
 
+// Forward y transforms: the same steps backwards.
 template <typename T, typename Plan>
-__device__ __forceinline__ void plane_y_fwd(cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, int nt,
-                                            const cplx<T>* __restrict__ tw) {
+__device__ __forceinline__ void plane_y_fwd_2(cplx<T>* P, const PlaneDims& D, int pitch, int nt,
+                                              const cplx<T>* __restrict__ tw) {
   using C = cplx<T>;
   constexpr int R1 = Plan::R1, R2 = Plan::R2;
   const unsigned inv = (1u << 20) / (unsigned)D.n1s + 1u;
@@ -265,7 +272,12 @@ __device__ __forceinline__ void plane_y_fwd(cplx<T>* P, cplx<T>* X, const PlaneD
 #pragma unroll
     for (int j = 0; j < R2; ++j) o[Plan::output(q, j)] = (!Plan::kCoprime && j) ? twist(v[j], tw[j * q], -1) : v[j];
   }
-  __syncthreads();
+}
+template <typename T, typename Plan>
+__device__ __forceinline__ void plane_y_fwd_1(const cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, int nt) {
+  using C = cplx<T>;
+  constexpr int R1 = Plan::R1, R2 = Plan::R2;
+  const unsigned inv = (1u << 20) / (unsigned)D.n1s + 1u;
   for (int w = threadIdx.x; w < D.n1s * R2; w += nt) {
     const int j = (int)(((unsigned)w * inv) >> 20), r = w - j * D.n1s;
     const C* o = P + r * pitch;
@@ -380,17 +392,77 @@ template <typename T>
 __device__ __forceinline__ PlaneDims plane_dims(const SphereDev& sp) {
   return PlaneDims{sp.span1, sp.span2, sp.lo1, sp.lo2, sp.span2 | 1};
 }
-// Sphere columns of one plane into X[row][m2 - lo2] (slots without a column are zero), and back.
-template <typename T>
+// Sphere columns of one plane into X[row][m2 - lo2] (slots without a column are zero), and back; RUNS: the
+// columns of D.n1s rows alone, whose first slot is p0.
+template <typename T, bool RUNS>
 __device__ __forceinline__ void plane_columns_in(cplx<T>* X, const cplx<T>* __restrict__ S, const SphereDev& sp,
-                                                 const PlaneDims& D, int nt) {
-  for (int i = threadIdx.x; i < D.n1s * D.W; i += nt) X[i] = mk<T>(0, 0);
+                                                 const PlaneDims& D, int p0, int nt) {
+  const int n = D.n1s * D.W;
+  for (int i = threadIdx.x; i < n; i += nt) X[i] = mk<T>(0, 0);
   __syncthreads();
-  for (int c = threadIdx.x; c < sp.ncol; c += nt) X[sp.col_pos[c]] = S[c];
+  for (int c = threadIdx.x; c < sp.ncol; c += nt) {
+    const int i = RUNS ? sp.col_pos[c] - p0 : sp.col_pos[c];
+    if (!RUNS || (i >= 0 && i < n)) X[i] = S[c];
+  }
 }
-template <typename T>
-__device__ __forceinline__ void plane_columns_out(const cplx<T>* X, cplx<T>* __restrict__ S, const SphereDev& sp, int nt) {
-  for (int c = threadIdx.x; c < sp.ncol; c += nt) S[c] = X[sp.col_pos[c]];
+template <typename T, bool RUNS>
+__device__ __forceinline__ void plane_columns_out(const cplx<T>* X, cplx<T>* __restrict__ S, const SphereDev& sp,
+                                                  const PlaneDims& D, int p0, int nt) {
+  const int n = D.n1s * D.W;
+  for (int c = threadIdx.x; c < sp.ncol; c += nt) {
+    const int i = RUNS ? sp.col_pos[c] - p0 : sp.col_pos[c];
+    if (!RUNS || (i >= 0 && i < n)) S[c] = X[i];
+  }
+}
+
+// Columns -> X -> y inverse transforms in P, and back.  RUNS: X holds the columns of `rows` rows at a
+// time, for spheres so wide that those of all rows do not fit beside P.  The alternative is the
+// runtime-length kernels.  H psi on n x n x 96, FP32, n = 144, 32 bands, spans of 114 / 128 / 142: 6.08 /
+// 6.76 / 7.58 ms there, 0.89 / 1.06 / 1.48 ms in runs; FP64, n = 96, 16 bands, spans of 88 / 94: 5.42 / 5.82
+// and 3.07 / 3.26 ms.
+template <typename T, typename Plan, bool RUNS>
+__device__ __forceinline__ void plane_in(cplx<T>* P, cplx<T>* X, const cplx<T>* __restrict__ S, const SphereDev& sp,
+                                         const PlaneDims& D, int rows, int pitch, int nt,
+                                         const cplx<T>* __restrict__ tw) {
+  if constexpr (!RUNS) {
+    plane_columns_in<T, false>(X, S, sp, D, 0, nt);
+    __syncthreads();
+    plane_y_inv_1<T, Plan>(P, X, D, pitch, nt);
+  } else {
+#pragma unroll 1
+    for (int r0 = 0; r0 < D.n1s; r0 += rows) {
+      PlaneDims R = D;
+      R.n1s = min(rows, D.n1s - r0);
+      if (r0) __syncthreads();  // the rows before have left X
+      plane_columns_in<T, true>(X, S, sp, R, r0 * D.W, nt);
+      __syncthreads();
+      plane_y_inv_1<T, Plan>(P + r0 * pitch, X, R, pitch, nt);
+    }
+  }
+  __syncthreads();
+  plane_y_inv_2<T, Plan>(P, D, pitch, nt, tw);
+}
+template <typename T, typename Plan, bool RUNS>
+__device__ __forceinline__ void plane_out(cplx<T>* P, cplx<T>* X, cplx<T>* __restrict__ S, const SphereDev& sp,
+                                          const PlaneDims& D, int rows, int pitch, int nt,
+                                          const cplx<T>* __restrict__ tw) {
+  plane_y_fwd_2<T, Plan>(P, D, pitch, nt, tw);
+  __syncthreads();
+  if constexpr (!RUNS) {
+    plane_y_fwd_1<T, Plan>(P, X, D, pitch, nt);
+    __syncthreads();
+    plane_columns_out<T, false>(X, S, sp, D, 0, nt);
+  } else {
+#pragma unroll 1
+    for (int r0 = 0; r0 < D.n1s; r0 += rows) {
+      PlaneDims R = D;
+      R.n1s = min(rows, D.n1s - r0);
+      if (r0) __syncthreads();
+      plane_y_fwd_1<T, Plan>(P + r0 * pitch, X, R, pitch, nt);
+      __syncthreads();
+      plane_columns_out<T, true>(X, S, sp, R, r0 * D.W, nt);
+    }
+  }
 }
 
 // Columns a batch of the x transforms takes: as many as let about NT threads hold one butterfly
@@ -403,10 +475,10 @@ __host__ __device__ constexpr int plane_batch(int n2, int rmax, int nt) {
   return (n2 + nb - 1) / nb;
 }
 
-template <typename T, typename PX, typename PY, int NT, int MINB>
+template <typename T, typename PX, typename PY, int NT, int MINB, bool RUNS>
 __global__ void __launch_bounds__(NT, MINB)
 k_plane_pass(const __grid_constant__ HpsiBatch<T> B, int n3, const cplx<T>* __restrict__ tw1,
-             const cplx<T>* __restrict__ tw2, int psize) {
+             const cplx<T>* __restrict__ tw2, int psize, int rows) {
   using C = cplx<T>;
   constexpr int PITCH = PY::N | 1, LB = plane_batch(PY::N, PX::R1, NT);
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -418,15 +490,11 @@ k_plane_pass(const __grid_constant__ HpsiBatch<T> B, int n3, const cplx<T>* __re
   const int b = local / n3, i3 = local - b * n3;
   C* S = I.scratch + ((size_t)b * n3 + i3) * sp.ldc;
   const PlaneDims D = plane_dims<T>(sp);
-  plane_columns_in<T>(X, S, sp, D, NT);
-  __syncthreads();
-  plane_y_inv<T, PY>(P, X, D, PITCH, NT, tw2);
+  plane_in<T, PY, RUNS>(P, X, S, sp, D, rows, PITCH, NT, tw2);
   __syncthreads();
   plane_x_all<T, PX>(P, X, D, PITCH, PY::N, LB, tw1, I.vplane + (size_t)i3 * PX::N * PY::N);
   __syncthreads();
-  plane_y_fwd<T, PY>(P, X, D, PITCH, NT, tw2);
-  __syncthreads();
-  plane_columns_out<T>(X, S, sp, NT);
+  plane_out<T, PY, RUNS>(P, X, S, sp, D, rows, PITCH, NT, tw2);
 }
 
 // ---- band densities --------------------------------------------------------------------------------
@@ -491,11 +559,11 @@ __device__ __forceinline__ void plane_x_rho(const cplx<T>* P, cplx<T>* X, const 
 }
 
 // Bands [nb g / groups, nb (g + 1) / groups) of group g.
-template <typename T, typename PX, typename PY, int NT, int MINB>
+template <typename T, typename PX, typename PY, int NT, int MINB, bool RUNS>
 __global__ void __launch_bounds__(NT, MINB)
 k_plane_rho(const cplx<T>* __restrict__ scratch, SphereDev sp, int nb, const double* __restrict__ weight,
             typename RhoAcc<T>::t* __restrict__ part, int n3, const cplx<T>* __restrict__ tw1,
-            const cplx<T>* __restrict__ tw2, int psize) {
+            const cplx<T>* __restrict__ tw2, int psize, int rows) {
   using C = cplx<T>;
   constexpr int PITCH = PY::N | 1, LB = plane_batch(PY::N, PX::R1, NT);
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -507,9 +575,7 @@ k_plane_rho(const cplx<T>* __restrict__ scratch, SphereDev sp, int nb, const dou
   auto* rho = part + ((size_t)g * n3 + i3) * PX::N * PY::N;
 #pragma unroll 1
   for (int b = b0; b < b1; ++b) {
-    plane_columns_in<T>(X, scratch + ((size_t)b * n3 + i3) * sp.ldc, sp, D, NT);
-    __syncthreads();
-    plane_y_inv<T, PY>(P, X, D, PITCH, NT, tw2);
+    plane_in<T, PY, RUNS>(P, X, scratch + ((size_t)b * n3 + i3) * sp.ldc, sp, D, rows, PITCH, NT, tw2);
     __syncthreads();
     plane_x_rho<T, PX>(P, X, D, PITCH, PY::N, LB, tw1, weight[b], b == b0, rho);
   }

@@ -76,12 +76,26 @@ template <typename T> static int sides(const std::vector<int>& ns) {
     }
   return 0;
 }
+// Spheres as wide as the plane, which the compiled-side kernels have always served.
+template <typename T> static int widest(const std::vector<int>& ns, size_t most) {
+  for (int n : ns)
+    for (int a = 1; a <= n; ++a)
+      for (int b = 1; b <= n; ++b) {
+        SphereDev sp{};
+        sp.span1 = a;
+        sp.span2 = b;
+        if ((size_t)n * n * sizeof(cplx<T>) <= most && !two_step_grid<T>(GridDims{n, n, 24}, sp))
+          return printf("%d x %d, %d bytes: spans %d, %d refused\n", n, n, (int)sizeof(T), a, b), 1;
+      }
+  return 0;
+}
 int main() {
   const std::vector<int> ns = {
 #define ONE(N, A, B) N,
       FDE_PLANE_SIDES(ONE)
   };
   if (sides<float>(ns) || sides<double>(ns)) return 1;
+  if (widest<float>(ns, 227 * 1024) || widest<double>(ns, 190 * 1024)) return 1;
   printf("%ld lists, %ld cuts\n", lists, cuts);
   return 0;
 }
@@ -122,7 +136,7 @@ using namespace fde;
 int main() {
   HpsiBatch<float> B{};
   FftPlans<float> fp{};
-  for (size_t bytes : {100000, 200000, 60000}) plane_square<float, 9, 8>(0, B, 24, fp, bytes, 0, 0);
+  for (size_t bytes : {100000, 200000, 60000}) plane_square<float, 9, 8>(0, B, 24, fp, bytes, 0, 1, false, 0);
   for (int v : limits)
     if (v != (int)kCtaSmemMax) return printf("limit set to %d\n", v), 1;
   return limits.size() == 3 ? 0 : 1;
@@ -137,11 +151,11 @@ int main() {
   HpsiBatch<float> B{};
   FftPlans<float> fp{};
   SphereDev sp{};
-  if (plane_square<float, 9, 8>(0, B, 24, fp, 60000, 0, 0) == cudaSuccess) return printf("plane pass\n"), 1;
-  if (rho_square<float, 9, 8>(dim3(0), nullptr, sp, 1, nullptr, nullptr, 24, fp, 60000, 0, 0) == cudaSuccess)
+  if (plane_square<float, 9, 8>(0, B, 24, fp, 60000, 0, 1, false, 0) == cudaSuccess) return printf("plane pass\n"), 1;
+  if (rho_square<float, 9, 8>(dim3(0), nullptr, sp, 1, nullptr, nullptr, 24, fp, 60000, 0, 1, 0) == cudaSuccess)
     return printf("density\n"), 1;
   answer = cudaErrorInvalidValue;
-  return plane_square<float, 9, 8>(0, B, 24, fp, 60000, 0, 0) == answer ? 0 : 1;
+  return plane_square<float, 9, 8>(0, B, 24, fp, 60000, 0, 1, false, 0) == answer ? 0 : 1;
 }
 """
 
