@@ -1111,10 +1111,16 @@ template <typename T> struct EngineT : Engine {
   // squared norm of a direction's part outside the earlier ones, and it carries the Gram
   // matrix's absolute rounding error, ~1e-6 of the diagonal for FP32 vectors (split-TF32
   // products): a pivot within ten times that error counts as a dependent direction (the
-  // previous directions are dropped first, then the iteration ends with the current orbitals).
-  // A stricter bound (1e-3) ends the FP32 solves of the 72 x 72 x 180 slab after a dozen
-  // iterations, short of a 1e-4 residual.  FP64 vectors: a rounding-level bound.
+  // previous directions are dropped first, then single ones, then the solve ends with the
+  // current orbitals).  A stricter bound (1e-3) ends the FP32 solves of the 72 x 72 x 180 slab
+  // after a dozen iterations, short of a 1e-4 residual.  A caller's own FP64 block is refused only
+  // when it is exactly dependent.
   static constexpr double rel_pivot() { return sizeof(T) == 4 ? 1e-5 : 1e-29; }
+  // The same for the search directions of a step, which the solver can do without.  FP64 Gram matrices
+  // of unit vectors err by some 1e-15: a pivot of that size is rounding noise, of either sign, and a
+  // direction kept on it comes out of the inverse factor as a vector of norm 1e-8 that stands for one of
+  // the lowest pairs.
+  static constexpr double direction_pivot() { return sizeof(T) == 4 ? rel_pivot() : 1e-13; }
   int bad_pivot = -1;  // column of the last failure
   void check_cholesky() {
     unsigned hs[2] = {0, 0};
@@ -1166,12 +1172,13 @@ template <typename T> struct EngineT : Engine {
   DBuf<C> SV, SV2, SPb;
   void rayleigh_ritz(KP<T>& q, int n, int nb, std::vector<double>& eps) {
     const int K = q.npw;
+    const double least = n > nb ? direction_pivot() : rel_pivot();
     gwork.ensure(gemm_hn_work(n, n, K));
     launch_gemm_hn<T>(V.p, K, use_s ? SV.p : V.p, K, n, n, K, S.p, n, gwork.p, st);
     launch_gemm_hn<T>(V.p, K, HV.p, K, n, n, K, Hs.p, n, gwork.p, st);
     launch_hermitize(S.p, n, st);
     launch_hermitize(Hs.p, n, st);
-    launch_cholesky_inv(S.p, n, L.p, Li.p, status.p, rel_pivot(), st);
+    launch_cholesky_inv(S.p, n, L.p, Li.p, status.p, least, st);
     check_cholesky();
     launch_small_gemm(Li.p, n, 0, Hs.p, n, 0, n, n, n, tmp.p, n, st);
     launch_small_gemm(tmp.p, n, 0, Li.p, n, 1, n, n, n, Ht.p, n, st);
