@@ -114,25 +114,17 @@ class Clocks:
         return out
 
 
-def kernel_source_digest(files, function=None):
-    """SHA-256 (16 hex digits) of the sources a kernel is built from: whole files, plus, for
-    (file, name), the text of the __global__ function `name` in that file."""
+def kernel_source_digest(files):
+    """SHA-256 (16 hex digits) of the sources a kernel is built from, whole files."""
     import hashlib
     h = hashlib.sha256()
     for f in files:
         with open(os.path.join(ROOT, f), "rb") as fh:
             h.update(f.encode() + b"\0" + fh.read())
-    if function:
-        f, name = function
-        text = open(os.path.join(ROOT, f)).read()
-        a = text.index(name + "(")
-        a = text.rindex("template", 0, a)
-        b = text.index("\n}\n", a) + 3
-        h.update(name.encode() + b"\0" + text[a:b].encode())
     return h.hexdigest()[:16]
 
 
-def _profile_traffic(name, files, function=None):
+def _profile_traffic(name, files):
     """DRAM bytes per launch of a kernel from its committed ncu summary (profiles/<name>.md),
     or None when the kernel's sources have changed since the counters were taken."""
     try:
@@ -141,15 +133,14 @@ def _profile_traffic(name, files, function=None):
         return None
     fields = dict(l.split(":", 1) for l in text.splitlines()
                   if l.startswith(("traffic_bytes_per_launch:", "source_sha256:")))
-    if fields.get("source_sha256", "").split()[0:1] != [kernel_source_digest(files, function)]:
+    if fields.get("source_sha256", "").split()[0:1] != [kernel_source_digest(files)]:
         return None
     return float(fields["traffic_bytes_per_launch"])
 
 
-# the plane pass: its own function text and steps in hpsi2.cuh plus the two-step transform core
-PLANE_SOURCES = ["paper_1406_7803_gb300/csrc/fft2.cuh", "paper_1406_7803_gb300/csrc/fft.cuh",
-                 "paper_1406_7803_gb300/csrc/common.cuh"]
-PLANE_FUNCTION = ("paper_1406_7803_gb300/csrc/hpsi2.cuh", "k_plane_pass")
+# the plane pass: its launch and thread rule, the kernel and its steps, the transform core
+PLANE_SOURCES = ["paper_1406_7803_gb300/csrc/" + f for f in
+                 ("hpsi2_p.cuh", "hpsi2.cuh", "fft2.cuh", "fft.cuh", "dd.cuh", "common.cuh")]
 
 
 def max_over_ranks(x, ws, device):
@@ -625,7 +616,7 @@ def run_ours(args):
         sec = ms_plane / n_plane / 1e3
         pk = fp["fp32_tflops"] if args.prec == "mixed" else fp["fp64_tflops"]
         achieved = per_launch_flops / sec / 1e12
-        traffic = (_profile_traffic("k_plane_pass_molecule_on_slab", PLANE_SOURCES, PLANE_FUNCTION)
+        traffic = (_profile_traffic("k_plane_pass_molecule_on_slab", PLANE_SOURCES)
                    if (args.prec == "mixed" and args.workload == "molecule-on-slab") else None)
         hbm_gbs = per_launch_bytes / sec / 1e9
         roof = {"bound": "alu", "achieved": achieved, "peak": pk, "unit": "TFLOP/s", "frac": achieved / pk,
