@@ -21,7 +21,7 @@ PROGRAM = r"""
 using namespace fde;
 static long lists = 0, cuts = 0;
 template <typename T> static int check(const GridDims& g, const std::vector<HpsiItemDesc<T>>& it) {
-  const int lb = plane_lb<T>(g.n1, g.n2), n = (int)it.size();
+  const int n = (int)it.size();
   ++lists;
   for (int i0 = 0, k = 0; i0 < n; i0 += k) {
     k = plane_group<T>(g, it.data() + i0, n - i0, kBatchMax);
@@ -31,12 +31,12 @@ template <typename T> static int check(const GridDims& g, const std::vector<Hpsi
       s1 = std::max(s1, it[j].sp.span1);
       s2 = std::max(s2, it[j].sp.span2);
     }
-    if (plane_launch_smem<T>(g, s1, s2) > kCtaSmemMax) return 2;
+    if (plane_fit<T>(g, s1, s2).smem > kCtaSmemMax) return 2;
     if (i0 + k < n && k < kBatchMax) {
       ++cuts;
       s1 = std::max(s1, it[i0 + k].sp.span1);
       s2 = std::max(s2, it[i0 + k].sp.span2);
-      if (plane_launch_smem<T>(g, s1, s2) <= kCtaSmemMax) return 3;
+      if (plane_fit<T>(g, s1, s2).smem <= kCtaSmemMax) return 3;
     }
   }
   return 0;
@@ -89,7 +89,18 @@ template <typename T> static int widest(const std::vector<int>& ns, size_t most)
       }
   return 0;
 }
+// The thread rule of a side: whole batches of items, one a thread, in a CTA that can run.
+template <typename T> static bool shape_ok(int n, int r1, int r2) {
+  const PlaneShape s = plane_shape<T>(n);
+  const int lb = plane_lb<T>(n, n);
+  const int runs = plane_has_runs<T>(n) ? plane_runs_lb<T>(n) * r1 : 0;
+  return s.nt >= 128 && s.nt <= 512 && s.nt % 32 == 0 && s.minb >= 1 && s.minb * s.nt <= 1024 && r1 >= r2 && lb >= 1 &&
+         lb * r1 <= s.nt && runs <= 512;
+}
 int main() {
+#define SHAPE(N, A, B) \
+  if (!shape_ok<float>(N, A, B) || !shape_ok<double>(N, A, B)) return printf("shape of %d\n", N), 1;
+  FDE_PLANE_SIDES(SHAPE)
   const std::vector<int> ns = {
 #define ONE(N, A, B) N,
       FDE_PLANE_SIDES(ONE)
@@ -136,7 +147,7 @@ using namespace fde;
 int main() {
   HpsiBatch<float> B{};
   FftPlans<float> fp{};
-  for (size_t bytes : {100000, 200000, 60000}) plane_square<float, 9, 8>(0, B, 24, fp, bytes, 0, 1, false, 0);
+  for (size_t bytes : {100000u, 200000u, 60000u}) plane_square<float, 9, 8>(0, B, 24, fp, 0, PlaneFit{1, false, bytes}, 0);
   for (int v : limits)
     if (v != (int)kCtaSmemMax) return printf("limit set to %d\n", v), 1;
   return limits.size() == 3 ? 0 : 1;
@@ -151,11 +162,12 @@ int main() {
   HpsiBatch<float> B{};
   FftPlans<float> fp{};
   SphereDev sp{};
-  if (plane_square<float, 9, 8>(0, B, 24, fp, 60000, 0, 1, false, 0) == cudaSuccess) return printf("plane pass\n"), 1;
-  if (rho_square<float, 9, 8>(dim3(0), nullptr, sp, 1, nullptr, nullptr, 24, fp, 60000, 0, 1, 0) == cudaSuccess)
+  const PlaneFit f{1, false, 60000};
+  if (plane_square<float, 9, 8>(0, B, 24, fp, 0, f, 0) == cudaSuccess) return printf("plane pass\n"), 1;
+  if (rho_square<float, 9, 8>(dim3(0), nullptr, sp, 1, nullptr, nullptr, 24, fp, 0, f, 0) == cudaSuccess)
     return printf("density\n"), 1;
   answer = cudaErrorInvalidValue;
-  return plane_square<float, 9, 8>(0, B, 24, fp, 60000, 0, 1, false, 0) == answer ? 0 : 1;
+  return plane_square<float, 9, 8>(0, B, 24, fp, 0, f, 0) == answer ? 0 : 1;
 }
 """
 
