@@ -36,17 +36,6 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// Block-wide sum (all threads receive it); red holds kClWarps doubles.
-__device__ __forceinline__ double block_sum_cl(double v, double* red) {
-  v = warp_sum_d(v);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0;
-  for (int k = 0; k < kClWarps; ++k) t += red[k];
-  return t;
-}
-
 struct ClusterLayout {
   int P, rank, nloc, sh;  // CTAs (a power of two, 2^sh), own rank, rows held
   __device__ __forceinline__ int owner(int i) const { return i & (P - 1); }

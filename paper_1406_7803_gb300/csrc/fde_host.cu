@@ -234,9 +234,10 @@ template <typename T> struct EngineT : Engine {
   DBuf<double> vloc;
   double enn = 0;
   // grid work
-  // Work grids of the embedding-potential build.  Its transforms run in FP64 in both
-  // precisions: FP32 gradients of the density are noise where the density is small (the
-  // vacuum above the slab), and the GGA potentials amplify that noise by rho^{-4/3}.
+  // Work grids of the embedding-potential build.  The transforms of the densities and their
+  // gradients run in FP64, in mixed contexts in double-float (~48 bits): FP32 gradients of the
+  // density are noise where the density is small (the vacuum above the slab), and the GGA
+  // potentials amplify that noise by rho^{-4/3}.
   DBuf<double2> cb[2];                // packed transform / potential; rho_tot(G)
   std::vector<DBuf<double2>> packs;   // per subsystem pair: packed gradient grids
   DBuf<double2> cvl;
@@ -246,7 +247,7 @@ template <typename T> struct EngineT : Engine {
   DBuf<C> scratch;
   DBuf<double2> gwork, Pm, Qm;
   DBuf<C> V, HV, V2, HV2, R, Pb, HPb;
-  DBuf<double2> S, Hs, L, Li, Ht, Y, Cc, tmp, jwork;
+  DBuf<double2> S, Hs, L, Li, Ht, Y, Cc, tmp;
   DBuf<double> wv, dnorm, deps, dtb, hwork;
   DBuf<int> didx;
   DBuf<double> rho_plane, rho_part, occw;
@@ -1136,7 +1137,7 @@ template <typename T> struct EngineT : Engine {
   void ensure_small(int n) {
     const size_t n2 = (size_t)n * n;
     S.ensure(n2); Hs.ensure(n2); L.ensure(n2); Li.ensure(n2); Ht.ensure(n2); Y.ensure(n2); Cc.ensure(n2);
-    tmp.ensure(n2); jwork.ensure(n2);
+    tmp.ensure(n2);
     wv.ensure(n); dnorm.ensure(n); deps.ensure(n); dtb.ensure(n); didx.ensure(n);
   }
 

@@ -10,7 +10,7 @@
 // the values item q of the forward starts with (a pointwise product fits between them in
 // registers), and item j of the forward ends on the indices item j of the inverse began with.
 //
-// Each thread owns whole butterflies (up to 20 values in registers), so a line crosses shared
+// Each thread owns whole butterflies (up to 25 values in registers), so a line crosses shared
 // memory once per direction instead of once per radix-8-or-9 stage (180 and 288 points took
 // three stages, 96 and 144 too), a butterfly reads its inputs straight from global memory and
 // writes its outputs straight back, and inputs outside the plane-wave sphere are never stored or

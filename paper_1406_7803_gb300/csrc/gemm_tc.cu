@@ -25,7 +25,7 @@
 //   M = 128, N = 128, K = 8 and commits them to the stage's mbarrier ; one stage per CTA,
 //   two CTAs per SM.
 //   Epilogue: tcgen05.ld of the 128 x 128 FP32 accumulators, FP32 partial tile to global;
-//   k_gemm_hn_reduce or k_gemm_hn_couple (linalg.cu) sums the K-splits in FP64 in a fixed order.
+//   k_gemm_hn_reduce or k_gemm_hn_couple (linalg.cu) sums the K-splits in double-float (48 bits) in a fixed order.
 // Every wait is bounded; on timeout the kernel sets ST_TIMEOUT, waits (bounded) for its
 // issued MMAs, frees its tensor memory and returns.
 #include <stdint.h>

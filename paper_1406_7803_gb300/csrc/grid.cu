@@ -376,8 +376,6 @@ __global__ void k_nonfinite(const double* __restrict__ a, long long n, unsigned*
 // a(G) = (C(G) + conj C(-G)) / 2 and b(G) = (C(G) - conj C(-G)) / (2 i).  The potential build
 // packs the subsystem densities, gradient components and divergence arguments in pairs, so
 // that it needs half the FP64 transforms while computing the same quantities.
-__device__ __forceinline__ double2 to_d2(double2 v) { return v; }
-__device__ __forceinline__ double2 to_d2(float2 v) { return make_double2((double)v.x, (double)v.y); }
 __global__ void k_pack2(const double* __restrict__ a, const double* __restrict__ b, double2* __restrict__ c,
                         long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -602,12 +600,12 @@ k_assemble_pair(const double2* __restrict__ RT, const double2* __restrict__ Da, 
       vb = va;
       if (Da) {
         // G . d of both fields at G (twice the unpacked values): x and y of a in Da, of b in Db, z in Dz
-        const double2 u = (Da[p.idx]), un = (Da[p.jn]), z = (Dz[p.idx]), zn = (Dz[p.jn]);
+        const double2 u = Da[p.idx], un = Da[p.jn], z = Dz[p.idx], zn = Dz[p.jn];
         const double dar = p.gx * (u.x + un.x) + p.gy * (u.y + un.y) + p.gz * (z.x + zn.x);
         const double dai = p.gx * (u.y - un.y) + p.gy * (un.x - u.x) + p.gz * (z.y - zn.y);
         va = make_double2(va.x + dai * s, va.y - dar * s);
         if (has_b) {
-          const double2 w = (Db[p.idx]), wn = (Db[p.jn]);
+          const double2 w = Db[p.idx], wn = Db[p.jn];
           const double dbr = p.gx * (w.x + wn.x) + p.gy * (w.y + wn.y) + p.gz * (z.y + zn.y);
           const double dbi = p.gx * (w.y - wn.y) + p.gy * (wn.x - w.x) + p.gz * (zn.x - z.x);
           vb = make_double2(vb.x + dbi * s, vb.y - dbr * s);
@@ -617,11 +615,11 @@ k_assemble_pair(const double2* __restrict__ RT, const double2* __restrict__ Da, 
     if (F) {
       // V(-G) = conj V(G)
       if (has_b) {
-        F[p.idx] = make_double2((va.x - vb.y), (va.y + vb.x));
-        F[p.jn] = make_double2((va.x + vb.y), (vb.x - va.y));
+        F[p.idx] = make_double2(va.x - vb.y, va.y + vb.x);
+        F[p.jn] = make_double2(va.x + vb.y, vb.x - va.y);
       } else {
-        F[p.idx] = make_double2((va.x), (va.y));
-        F[p.jn] = make_double2((va.x), (-va.y));
+        F[p.idx] = make_double2(va.x, va.y);
+        F[p.jn] = make_double2(va.x, -va.y);
       }
     }
   }

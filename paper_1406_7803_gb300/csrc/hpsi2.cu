@@ -2,8 +2,6 @@
 // three phases (z inverse, plane pass, z forward).
 #include "hpsi2.cuh"
 
-#include <atomic>
-
 namespace fde {
 
 // Run up to kBatchMax items per launch, as many as fit together; items[i].zstart / pstart are filled here.

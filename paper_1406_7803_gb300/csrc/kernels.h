@@ -90,7 +90,7 @@ template <typename T> int plane_group(const GridDims& g, const HpsiItemDesc<T>* 
 int query_plane_variant(int n1, int n3);
 bool pin_plane_variant(int v);
 
-// Full 3D transforms on two-step plans (fft3.cu); false when a length has none.
+// Full 3D transforms on two-step plans (fft3_32.cu, fft3_64.cu); false when a length has none.
 template <typename T>
 bool launch_fft3d_two_step(cplx<T>* data, const GridDims& g, const FftPlans<T>& fp, int sign, cudaStream_t st);
 template <>
@@ -126,7 +126,6 @@ unsigned gemm_tc_take_status(cudaStream_t st);
 bool set_tc_stage_spin(long long polls);
 void disable_tensor_cores();
 bool tensor_cores_disabled();
-void launch_gemm_hn_reduce(const float2* part, int nsplit, int m, int n, double2* C, int ldc, cudaStream_t st);
 template <typename T>
 void launch_gemm_hn(const cplx<T>* A, int lda, const cplx<T>* B, int ldb, int m, int n, int K,
                     double2* C, int ldc, double2* work, cudaStream_t st);

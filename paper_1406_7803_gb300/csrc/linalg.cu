@@ -269,9 +269,6 @@ static void hn_reduce(const P* part, int nsplit, int m, int n, double2* C, int l
   ProfScope prof_r("k_gemm_hn_reduce", st);
   k_gemm_hn_reduce<P><<<ceil_div((long long)m * n, 32), 32 * kRW, 0, st>>>(part, nsplit, m, n, C, ldc);
 }
-void launch_gemm_hn_reduce(const float2* part, int nsplit, int m, int n, double2* C, int ldc, cudaStream_t st) {
-  hn_reduce(part, nsplit, m, n, C, ldc, st);
-}
 
 // The product's partial tiles into work; returns their number (0: m or n is empty).
 static int hn_partial(const double2* A, int lda, const double2* B, int ldb, int m, int n, int K, double2* work,
