@@ -418,8 +418,8 @@ __device__ __forceinline__ void plane_columns_out(const cplx<T>* X, cplx<T>* __r
 // Columns -> X -> y inverse transforms in P, and back.  RUNS: X holds the columns of `rows` rows at a
 // time, for spheres so wide that those of all rows do not fit beside P.  The alternative is the
 // runtime-length kernels.  H psi on n x n x 96, FP32, n = 144, 32 bands, spans of 114 / 128 / 142: 6.08 /
-// 6.76 / 7.58 ms there, 0.89 / 1.06 / 1.48 ms in runs; FP64, n = 96, 16 bands, spans of 88 / 94: 5.42 / 5.82
-// and 3.07 / 3.26 ms.
+// 6.76 / 7.58 ms there, 0.84 / 1.00 / 1.34 ms in runs; FP64, n = 96, 16 bands, spans of 88 / 94: 5.42 / 5.82
+// and 2.83 / 3.06 ms.
 template <typename T, typename Plan, bool RUNS>
 __device__ __forceinline__ void plane_in(cplx<T>* P, cplx<T>* X, const cplx<T>* __restrict__ S, const SphereDev& sp,
                                          const PlaneDims& D, int rows, int pitch, int nt,
