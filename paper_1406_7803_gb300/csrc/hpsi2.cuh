@@ -202,7 +202,9 @@ struct PlaneDims {
   int n1s, n2s;   // span of m1 (rows of P) and of m2
   int lo1, lo2;   // grid index of the first row and column
   int W;          // X pitch of the column stage (odd)
+  unsigned inv;   // row_inv(n1s): w / n1s = w inv >> 20 for w < 2^20 / n1s
 };
+__device__ __forceinline__ unsigned row_inv(int n1s) { return (1u << 20) / (unsigned)n1s + 1u; }
 
 // Offset of the span's first index from element 0 of item j: element r sits at d = wrap(base + R2 r) of
 // the span, inside it when d < span.
@@ -216,9 +218,8 @@ template <typename T, typename Plan>
 __device__ __forceinline__ void plane_y_inv_1(cplx<T>* P, const cplx<T>* X, const PlaneDims& D, int pitch, int nt) {
   using C = cplx<T>;
   constexpr int R1 = Plan::R1, R2 = Plan::R2;
-  const unsigned inv = (1u << 20) / (unsigned)D.n1s + 1u;  // w / n1s = w inv >> 20 for w < 2^20 / n1s
   for (int w = threadIdx.x; w < D.n1s * R2; w += nt) {
-    const int j = (int)(((unsigned)w * inv) >> 20), r = w - j * D.n1s;
+    const int j = (int)(((unsigned)w * D.inv) >> 20), r = w - j * D.n1s;
     const int base = span_base<Plan>(j, D.lo2);
     const C* x = X + r * D.W;
     C v[R1];
@@ -239,9 +240,8 @@ __device__ __forceinline__ void plane_y_inv_2(cplx<T>* P, const PlaneDims& D, in
                                               const cplx<T>* __restrict__ tw) {
   using C = cplx<T>;
   constexpr int R1 = Plan::R1, R2 = Plan::R2;
-  const unsigned inv = (1u << 20) / (unsigned)D.n1s + 1u;
   for (int w = threadIdx.x; w < D.n1s * R1; w += nt) {
-    const int q = (int)(((unsigned)w * inv) >> 20), r = w - q * D.n1s;
+    const int q = (int)(((unsigned)w * D.inv) >> 20), r = w - q * D.n1s;
     C* o = P + r * pitch;
     C v[R2];
 #pragma unroll
@@ -261,9 +261,8 @@ __device__ __forceinline__ void plane_y_fwd_2(cplx<T>* P, const PlaneDims& D, in
                                               const cplx<T>* __restrict__ tw) {
   using C = cplx<T>;
   constexpr int R1 = Plan::R1, R2 = Plan::R2;
-  const unsigned inv = (1u << 20) / (unsigned)D.n1s + 1u;
   for (int w = threadIdx.x; w < D.n1s * R1; w += nt) {
-    const int q = (int)(((unsigned)w * inv) >> 20), r = w - q * D.n1s;
+    const int q = (int)(((unsigned)w * D.inv) >> 20), r = w - q * D.n1s;
     C* o = P + r * pitch;
     C v[R2];
 #pragma unroll
@@ -277,9 +276,8 @@ template <typename T, typename Plan>
 __device__ __forceinline__ void plane_y_fwd_1(const cplx<T>* P, cplx<T>* X, const PlaneDims& D, int pitch, int nt) {
   using C = cplx<T>;
   constexpr int R1 = Plan::R1, R2 = Plan::R2;
-  const unsigned inv = (1u << 20) / (unsigned)D.n1s + 1u;
   for (int w = threadIdx.x; w < D.n1s * R2; w += nt) {
-    const int j = (int)(((unsigned)w * inv) >> 20), r = w - j * D.n1s;
+    const int j = (int)(((unsigned)w * D.inv) >> 20), r = w - j * D.n1s;
     const C* o = P + r * pitch;
     const int oj = Plan::out(j);
     C v[R1];
@@ -390,7 +388,7 @@ __device__ __forceinline__ void plane_x_all(cplx<T>* P, cplx<T>* X, const PlaneD
 
 template <typename T>
 __device__ __forceinline__ PlaneDims plane_dims(const SphereDev& sp) {
-  return PlaneDims{sp.span1, sp.span2, sp.lo1, sp.lo2, sp.span2 | 1};
+  return PlaneDims{sp.span1, sp.span2, sp.lo1, sp.lo2, sp.span2 | 1, row_inv(sp.span1)};
 }
 // Sphere columns of one plane into X[row][m2 - lo2] (slots without a column are zero), and back; RUNS: the
 // columns of D.n1s rows alone, whose first slot is p0.
@@ -433,6 +431,7 @@ __device__ __forceinline__ void plane_in(cplx<T>* P, cplx<T>* X, const cplx<T>* 
     for (int r0 = 0; r0 < D.n1s; r0 += rows) {
       PlaneDims R = D;
       R.n1s = min(rows, D.n1s - r0);
+      R.inv = row_inv(R.n1s);
       if (r0) __syncthreads();  // the rows before have left X
       plane_columns_in<T, true>(X, S, sp, R, r0 * D.W, nt);
       __syncthreads();
@@ -457,6 +456,7 @@ __device__ __forceinline__ void plane_out(cplx<T>* P, cplx<T>* X, cplx<T>* __res
     for (int r0 = 0; r0 < D.n1s; r0 += rows) {
       PlaneDims R = D;
       R.n1s = min(rows, D.n1s - r0);
+      R.inv = row_inv(R.n1s);
       if (r0) __syncthreads();
       plane_y_fwd_1<T, Plan>(P + r0 * pitch, X, R, pitch, nt);
       __syncthreads();
