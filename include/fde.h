@@ -387,8 +387,10 @@ fde_status fde_fft3d(fde_ctx* ctx, void* d_data, int sign);
 /* The potential build's 3D transform of an FP64 grid (complex double [n1][n2][n3], in place,
  * scaled as fde_fft3d) in either arithmetic the library uses for it: arith 0 native FP64 (FP64
  * contexts), 1 double-float (two floats per value, about 48 significant bits, on the FP32
- * pipes; mixed contexts transform the densities and their gradients this way).  Exposed so
- * the transforms can be checked on their own. */
+ * pipes; mixed contexts transform the densities and their gradients this way).  arith 1 takes
+ * grids whose lengths are all among 24, 32, 60, 72, 96, 144, 180 and 288 (FDE_EUNSUPPORTED for
+ * others, though the potential build uses it for more).  Exposed so the transforms can be checked
+ * on their own. */
 fde_status fde_fft3d_f64(fde_ctx* ctx, double* d_data, int sign, int arith);
 
 /* The FP64 Hermitian eigensolver of the Rayleigh-Ritz step applied to a caller matrix:
